@@ -536,14 +536,14 @@ int pcal_rotfold_get_acc(pcal_rotfold* r, float* host_out);
  *
  * For a comb offset whose combined period L (Eq. 4) is beyond PCAL_MAX_L (a
  * prime offset) or that is not a whole number of hertz, pcal_rotplan_* rotates
- * every sample (Eq. 3) into N bins (Eq. 2) in double-float: per thread a
- * rotator advanced by one complex multiplication per sample and re-seeded
- * every 256 samples from the exact phase frac(n*f_offset/fs) (double-double,
- * FP64 sincospi); then the DFT, the products and the post-processing of the
+ * every sample (Eq. 3) into N bins (Eq. 2): stripes of samples share a table
+ * of rotators (FP64 sincospi of exactly reduced phases, to 2^-46 or better),
+ * their sums are exact (int8) or compensated, and everything after them is
+ * double-float; then the DFT, the products and the post-processing of the
  * folded path.  fs and f_comb integral Hz, N = fs/f_comb <= PCAL_BATCH_MAX_N,
  * 0 <= f_offset < f_comb any value; f32, int8 or 2-bit samples; at most 2^52
- * samples per plan.  The throughput is arithmetic-bound (several times below
- * the folded path).
+ * samples per plan.  The throughput is arithmetic-bound (below the folded
+ * path).
  */
 typedef struct pcal_rotplan pcal_rotplan;
 
@@ -556,12 +556,13 @@ int pcal_rotplan_create(double fs, double f_comb, double f_offset, int N, int sa
 int pcal_rotplan_destroy(pcal_rotplan* plan);
 /* 2-bit decode levels of codes 0..3 (host array, copied), as pcal_plan_set_levels. */
 int pcal_rotplan_set_levels(pcal_rotplan* plan, const double levels[4]);
-/* samples: DEVICE, n samples continuing the absolute index; asynchronous on stream. */
+/* samples: DEVICE, n samples continuing the absolute index (any alignment; float32 PCAL_EINVAL off
+ * 4 bytes); asynchronous on stream. */
 int pcal_rotplan_accumulate(pcal_rotplan* plan, const void* samples, int64_t n, void* stream);
 /* Finalize on `stream` (results stay on the device) and start the next period. */
 int pcal_rotplan_finalize_device(pcal_rotplan* plan, void* stream);
 /* Results of the last finalize (synchronises; layout as pcal_read_results and pcal_read_post;
- * any pointer may be NULL). */
+ * any pointer may be NULL).  PCAL_ETIMEOUT if a bounded device wait gave up. */
 int pcal_rotplan_read_results(pcal_rotplan* plan, double* phasors, double* amp, double* phase, double* unwrapped,
                               double* td, double* sigma, double* td_peak, double* bandpass_phase);
 

@@ -42,6 +42,7 @@ using pcal_df::df;
 
 constexpr int kDftInFoldMaxN = 256;
 constexpr int kDftTonesPerCta = 32;
+constexpr int kFmtRotated = 16;  // cluster finalize of bins that are rotated already
 
 struct FinArgs {
     int fmt;
@@ -73,6 +74,7 @@ struct FinArgs {
     double* res;
     double* extra;  // post-processing, N+2 doubles (or null): peak delay, peak position, corrected bandpass phase
     float2* Pout;   // cluster finalize: if set, store P here and stop before the DFT
+    float4* rows;   // kFmtRotated: [L / N][N] rotated sums in df
     double fs_hz;
     unsigned int* ticket;
 };
@@ -747,14 +749,38 @@ __device__ __forceinline__ double2 fold_residue(const FinArgs& a, int b, int m, 
     return make_double2(re, im);
 }
 
-// Tones [i0, i1) of the N-point DFT of sP in FP32 (g threads per tone,
-// combined by a fixed butterfly), written to dst[i] (shared memory of this
-// CTA or, through the cluster, of another).
-__device__ void dft_range(const float2* sP, const float2* sTw, int N, int i0, int i1, float2* dst) {
+// Residue b over m = m, m + step, ... below m_end as double-float (re hi, re
+// lo, im hi, im lo).  kFmtRotated: the bins are rotated complex sums already
+// (the rows of a long-period plan), added in row order.
+template <int FMT>
+__device__ __forceinline__ float4 residue_df(const FinArgs& a, int b, int m, int step, int m_end) {
+    if constexpr (FMT == kFmtRotated) {
+        df re{0.f, 0.f}, im{0.f, 0.f};
+        const int N = (int)a.N;
+#pragma unroll 4
+        for (; m < m_end; m += step) {
+            const float4 v = a.rows[(int64_t)m * N + b];
+            a.rows[(int64_t)m * N + b] = make_float4(0.f, 0.f, 0.f, 0.f);
+            re = pcal_df::add(re, df{v.x, v.y});
+            im = pcal_df::add(im, df{v.z, v.w});
+        }
+        return make_float4(re.hi, re.lo, im.hi, im.lo);
+    } else {
+        const double2 z = fold_residue<FMT>(a, b, m, step, m_end);
+        const df dre = df_of(z.x), dim = df_of(z.y);
+        return make_float4(dre.hi, dre.lo, dim.hi, dim.lo);
+    }
+}
+
+// Tones [i0, i1) of the N-point DFT of sP in FP32, written to dst[i] (shared
+// memory of this CTA or, through the cluster, of another).  The threads per
+// tone g, combined by a fixed butterfly, are as many as `share` tones leave
+// for each in the block: they set the order of a tone's FP32 sum.
+__device__ void dft_range(const float2* sP, const float2* sTw, int N, int i0, int i1, float2* dst, int share) {
     const int t = threadIdx.x;
     const int ntone = i1 - i0;
     int g = 1;
-    while (g < 32 && g * 2 * ntone <= (int)blockDim.x) g *= 2;
+    while (g < 32 && g * 2 * share <= (int)blockDim.x) g *= 2;
     const int groups = blockDim.x / g;
     const int gs = t % g;
 #pragma unroll 1
@@ -818,9 +844,7 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
         // thread t: residue t % N, every lanes-th m of this CTA's slice
         const int b = t % N, ml = t / N;
         if (ml < lanes) {
-            const double2 z = fold_residue<FMT>(a, b, per * r / C + ml, lanes, m1);
-            const df dre = df_of(z.x), dim = df_of(z.y);
-            part[t] = make_float4(dre.hi, dre.lo, dim.hi, dim.lo);
+            part[t] = residue_df<FMT>(a, b, per * r / C + ml, lanes, m1);
         }
         __syncthreads();
         if (t < N) {
@@ -836,11 +860,7 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     } else {
         // one thread per residue, the residues in turns
 #pragma unroll 1
-        for (int b = t; b < N; b += blockDim.x) {
-            const double2 z = fold_residue<FMT>(a, b, per * r / C, 1, m1);
-            const df dre = df_of(z.x), dim = df_of(z.y);
-            Pr[b] = make_float4(dre.hi, dre.lo, dim.hi, dim.lo);
-        }
+        for (int b = t; b < N; b += blockDim.x) Pr[b] = residue_df<FMT>(a, b, per * r / C, 1, m1);
     }
     cluster.sync();  // every CTA's partial P is complete
     if (r == 0) {
@@ -896,7 +916,7 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     }
     if (!big) {
         if (r != 0) return false;
-        dft_range(sP, sTw, N, 0, N, sT);
+        dft_range(sP, sTw, N, 0, N, sT, N);
     } else {
         // every CTA: its share of the tones from a copy of P, into CTA 0's sT
         if (r != 0) {
@@ -904,7 +924,9 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
             for (int i = t; i < N; i += blockDim.x) sP[i] = p0[i];
         }
         __syncthreads();
-        dft_range(sP, sTw, N, N * r / C, N * (r + 1) / C, cluster.map_shared_rank(sT, 0));
+        // (long-period plans: in the order of one CTA with all N tones)
+        const int i0 = N * r / C, i1 = N * (r + 1) / C;
+        dft_range(sP, sTw, N, i0, i1, cluster.map_shared_rank(sT, 0), FMT == kFmtRotated ? N : i1 - i0);
         cluster.sync();  // CTA 0 holds every tone; its sP is no longer read
         if (r != 0) return false;
     }
@@ -1187,56 +1209,21 @@ cudaError_t launch_cluster_finalize(const FinArgs& a, int C, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_F32>, a);
 }
 
-// Finalize of a long-period plan (one CTA): the lanes of each bin added in
-// df (lane order), then the DFT, the products and the post-processing of the
-// folded path.
-__global__ void __launch_bounds__(kClusterThreads) rot_finalize_kernel(FinArgs a, const float4* acc, int lanes) {
-    __shared__ float4 part[kClusterThreads];
-    extern __shared__ __align__(16) uint8_t dsm[];
-    const int N = (int)a.N;
-    const ClusterSmem sm = cluster_layout(dsm, N);
-    const int t = threadIdx.x;
-    for (int i = t; i < N; i += blockDim.x) sm.sTw[i] = a.twN[i];
-    // bin b: its lanes split over G threads, then the G partials in order
-    const int G = (int)blockDim.x / N > 0 ? (int)blockDim.x / N : 1;
-    const int per_round = (int)blockDim.x / G;
-    for (int b0 = 0; b0 < N; b0 += per_round) {
-        const int b = b0 + t / G, g = t % G;
-        df sr{0.f, 0.f}, si{0.f, 0.f};
-        if (t / G < per_round && b < N)
-            for (int l = g; l < lanes; l += G) {
-                const float4 v = acc[(int64_t)l * N + b];
-                sr = pcal_df::add(sr, df{v.x, v.y});
-                si = pcal_df::add(si, df{v.z, v.w});
-            }
-        part[t] = make_float4(sr.hi, sr.lo, si.hi, si.lo);
-        __syncthreads();
-        if (g == 0 && t / G < per_round && b < N) {
-            df tr{0.f, 0.f}, ti{0.f, 0.f};
-            for (int q = 0; q < G; ++q) {
-                const float4 v = part[t + q];
-                tr = pcal_df::add(tr, df{v.x, v.y});
-                ti = pcal_df::add(ti, df{v.z, v.w});
-            }
-            sm.sP[b] = make_float2(tr.hi + tr.lo, ti.hi + ti.lo);
-        }
-        __syncthreads();
-    }
-    dft_range(sm.sP, sm.sTw, N, 0, N, sm.sT);
-    __syncthreads();
-    if (t < 32) tone_products_warp(a, sm.sT, sm.pm.psi, sm.pm.w, sm.pm.un, sm.pm.out);
-    else if (t < 64) peak_delay_warp(a, sm.sP);
-    __syncthreads();
-    write_results_block(a, sm.sT, sm.pm);
+// Finalize of a long-period plan: its rows of partial sums are added (and
+// cleared) by one cluster, then the DFT, the products and the post-processing
+// of the folded path.  (One CTA that added 9,728 rows of 16 bins took 115 us.)
+__global__ void __launch_bounds__(kClusterThreads, 1) rot_finalize_kernel(FinArgs a) {
+    cluster_finalize<kFmtRotated>(a);
 }
 
 }  // namespace
 
-cudaError_t launch_rot_finalize(const float4* acc, int lanes, int N, double fs, double fc, int64_t M,
+cudaError_t launch_rot_finalize(float4* rows, int n_rows, int N, double fs, double fc, int64_t M,
                                 const float2* twN, double* res, cudaStream_t s) {
     FinArgs a{};
     a.N = N;
-    a.L = N;
+    a.L = (int64_t)N * n_rows;
+    a.rows = rows;
     a.fs_hz = fs;
     a.M = (double)M;
     a.two_over_m = M > 0 ? (float)(2.0 / (double)M) : 0.0f;
@@ -1246,15 +1233,29 @@ cudaError_t launch_rot_finalize(const float4* acc, int lanes, int N, double fs, 
     a.twN = twN;
     a.res = res;
     a.extra = res + 5 * (int64_t)N + 3;
-    static bool attr_set = false;
-    if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(rot_finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)cluster_smem_bytes(kClusterBigN));
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    rot_finalize_kernel<<<1, kClusterThreads, cluster_smem_bytes(N), s>>>(a, acc, lanes);
-    return cudaGetLastError();
+    const int C = cluster_size_for_device();
+    if (C == 0) return cudaErrorNotSupported;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = cluster_smem_bytes(N);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, rot_finalize_kernel, a);
+}
+
+cudaError_t prepare_rot_finalize() {
+    if (cluster_size_for_device() == 0) return cudaErrorNotSupported;
+    cudaError_t e = cudaFuncSetAttribute(rot_finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)cluster_smem_bytes(kClusterBigN));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(rot_finalize_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
 }
 
 cudaError_t prepare_batch_finalize() {

@@ -212,9 +212,12 @@ struct BatchPiece {
 };
 
 cudaError_t prepare_batch_finalize();
-// Finalize of a long-period plan: acc = [lanes][N] double-float bin sums.
-cudaError_t launch_rot_finalize(const float4* acc, int lanes, int N, double fs, double fc, int64_t M,
+// Finalize of a long-period plan: rows = [n_rows][N] double-float bin sums
+// (re hi, re lo, im hi, im lo), added and cleared.
+cudaError_t launch_rot_finalize(float4* rows, int n_rows, int N, double fs, double fc, int64_t M,
                                 const float2* twN, double* res, cudaStream_t s);
+// The CUDA calls launch_rot_finalize needs once per device.
+cudaError_t prepare_rot_finalize();
 // Finalize channels list[i] (or i when list is null), i < n, with one cluster each.
 // split: stop every channel after P (its P slot) for the batched DFT, which
 // launch_batch_products then finishes.
