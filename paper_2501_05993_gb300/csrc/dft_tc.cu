@@ -1,4 +1,7 @@
-// Batched tone DFT on the tensor cores (tcgen05): T_i = sum_b P[b] e^{-j2 pi ib/N}
+// Batched tone DFT: the entry points of every mode, and the tensor-core
+// (tcgen05) contraction for the tone counts that dft_fft.cu does not take (a
+// prime factor above 7; at C 4096, N 1024 the contraction takes 176 us in split
+// TF32, the FFT 53).  The contraction: T_i = sum_b P[b] e^{-j2 pi ib/N}
 // for C channels at once (the "DFT(P)" step of Sec. 2 after the L-to-N fold of
 // Eq. 2), as one real contraction
 //
@@ -43,6 +46,7 @@
 
 #include <new>
 
+#include "dft_fft.cuh"
 #include "internal.cuh"
 #include "ptx.cuh"
 
@@ -564,6 +568,7 @@ __global__ void dft_fp32_kernel(const float2* __restrict__ P, float2* __restrict
 
 struct pcal_dft {
     int N, mode, n_cols, k_chunks, col_tiles, parts;
+    FftPlan fft;      // every mode, where N has small prime factors; the contraction's state is then not made
     uint8_t* d_w;     // weight tiles (tensor-core modes)
     uint8_t* d_a;     // operand tiles of P (workspace)
     size_t a_cap;     // bytes of d_a
@@ -653,6 +658,18 @@ extern "C" int pcal_dft_create(int N, int mode, pcal_dft** out) {
     memset(static_cast<void*>(d), 0, sizeof(*d));
     d->N = N;
     d->mode = mode;
+    if (fft_factors(N, &d->fft)) {
+        cudaError_t e = cudaMalloc(&d->d_err, sizeof(unsigned int));
+        if (e == cudaSuccess) e = cudaMemset(d->d_err, 0, sizeof(unsigned int));
+        if (e == cudaSuccess) e = fft_create(N, mode != PCAL_DFT_FP32, &d->fft);
+        if (e != cudaSuccess) {
+            pcal_dft_destroy(d);
+            (void)cudaGetLastError();
+            return e == cudaErrorMemoryAllocation ? PCAL_ENOMEM : PCAL_ECUDA;
+        }
+        *out = d;
+        return PCAL_OK;
+    }
     d->n_cols = (2 * N + 15) / 16 * 16;
     const int tc = mode == PCAL_DFT_FP32 ? 0 : tile_cols(mode);
     d->col_tiles = mode == PCAL_DFT_FP32 ? 0 : (d->n_cols + tc - 1) / tc;
@@ -712,6 +729,7 @@ extern "C" int pcal_dft_create(int N, int mode, pcal_dft** out) {
 extern "C" int pcal_dft_destroy(pcal_dft* d) {
     if (!d) return PCAL_OK;
     cudaDeviceSynchronize();
+    fft_destroy(&d->fft);
     cudaFree(d->d_w);
     cudaFree(d->d_a);
     cudaFree(d->d_tw);
@@ -722,7 +740,7 @@ extern "C" int pcal_dft_destroy(pcal_dft* d) {
 
 // Operand workspace for C channels (allocates: not under stream capture).
 cudaError_t dft_reserve(pcal_dft* d, int64_t C) {
-    if (d->mode == PCAL_DFT_FP32 || C <= 0) return cudaSuccess;
+    if (d->fft.passes || d->mode == PCAL_DFT_FP32 || C <= 0) return cudaSuccess;
     const size_t need = (size_t)((C + kTcM - 1) / kTcM) * d->k_chunks * d->parts * kTcM * chunk_bytes(d->mode);
     if (need <= d->a_cap) return cudaSuccess;
     cudaFree(d->d_a);
@@ -735,6 +753,7 @@ cudaError_t dft_reserve(pcal_dft* d, int64_t C) {
 
 cudaError_t launch_dft(pcal_dft* d, const float2* P, int64_t C, float2* T, cudaStream_t s, unsigned int* err) {
     if (C <= 0) return cudaSuccess;
+    if (d->fft.passes) return launch_fft(d->fft, P, C, T, s);
     if (d->mode == PCAL_DFT_FP32) {
         dft_fp32_kernel<<<(unsigned)C, 256, 2 * d->N * sizeof(float2), s>>>(P, T, d->N, d->d_tw);
         return cudaGetLastError();
