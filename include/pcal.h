@@ -297,8 +297,8 @@ int pcal_tones_from_counts_noalloc(double fs, double f_comb, double f_offset, in
  * A batch holds up to PCAL_MAX_BATCH channels (2-bit or int8 samples), each
  * with its own fs, f_comb, f_offset and N, hence its own period L (Eq. 4).
  * One pcal_batch_accumulate call folds a run of samples of every channel with
- * ONE persistent kernel launch over a work list of all channels' tiles; the
- * same launch folds the ragged heads and tails (pieces of at most 8 KB) and
+ * ONE kernel launch over a work list of all channels' tiles; the
+ * same launch folds the ragged heads and tails and
  * its last CTA advances the channels' sample indices.  A call that repeats
  * the buffers and lengths of an earlier call on the same stream reuses that
  * call's device descriptors without a copy.  pcal_batch_finalize_device
@@ -317,7 +317,9 @@ typedef struct {
     int sample_format;           /* PCAL_2BIT or PCAL_I8                      */
 } pcal_channel_desc;
 
-/* Launch schedule of the persistent fold (pcal_batch_autotune picks one).
+/* Launch schedule of the persistent fold, which takes the calls of a batch once
+ * a schedule was set (or pcal_batch_autotune found one faster than the fold
+ * without a schedule that takes them otherwise; it picks one all the same).
  * A channel's tile is a column group of its rows (one row = a whole number of
  * periods L); its width is capped by the channel's bucket -- sample format x
  * row width -- or, where the bucket's cap is 0, by col_cap.  Bucket index =
@@ -405,7 +407,8 @@ int pcal_batch_get_stats(const pcal_batch* batch, pcal_stats* out);
 
 /*
  * Time candidate schedules on these inputs, accumulate only, and keep the
- * fastest; writes it to *chosen when not NULL.  Three passes: the batch-wide
+ * fastest; writes it to *chosen when not NULL.  Where the fold without a
+ * schedule is at least as fast, calls go on to take that.  Three passes: the batch-wide
  * choices (column-width cap, box rows, static share, chunk size; the four
  * fastest timed again), then the CTA count (one per SM, or 8 or 16 fewer),
  * then, one bucket at a time for the buckets the batch's channels occupy, the

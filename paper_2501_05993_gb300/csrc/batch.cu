@@ -2,7 +2,10 @@
 // sample rate, comb offset, period L and length, folded by ONE persistent
 // launch and finalized by one launch with a thread-block cluster per channel.
 //
-// Work list.  Every channel's call is split like a single-plan call: a
+// Two folds.  The direct fold (below) takes every call of a batch whose
+// schedule was neither set nor tuned; the persistent fold the others.
+//
+// Work list of the persistent fold.  Every channel's call is split like a single-plan call: a
 // ragged head up to its first 16-byte boundary, whole rows of row_samples
 // samples (a multiple of L, so word c of every row feeds fixed bins), and a
 // ragged tail.  The rows of each (channel, column group) form a segment; the
@@ -481,6 +484,286 @@ __global__ void __launch_bounds__(kMaxBlock, 1) batch_fold_kernel(const BatchFol
     }
 }
 
+// ---- the direct fold -----------------------------------------------------------------
+//
+// The persistent fold above pays for every run (a CTA's stay in one segment):
+// its pipeline drains, the replicas merge and the counts are flushed, about
+// 6 us before the next segment's first data.  A call of short rows -- 10 ms of
+// a live channel is 100 rows -- is mostly such changes (64 live channels,
+// 128 MB: 99 us).  Here a small CTA takes a column block of a row block: its
+// four warps take batches of rows in turn, every lane copies its own words of
+// a batch (int8 16 bytes, 2-bit 4 bytes a row; a warp reads a contiguous run
+// of each row) into its own part of a three-batch ring with cp.async and
+// counts them in registers, so no thread waits for another until the four
+// warps' counts are added and go to the channel's bins, consecutive lanes on
+// consecutive bins.  Four CTAs per SM keep 128 KB in flight and hide each
+// other's starts and flushes.
+
+constexpr int kDirectWarps = 4;
+constexpr int kDirectThreads = 32 * kDirectWarps;
+constexpr int kDirectCtas = 4;                     // per SM (48 KB of shared memory each)
+constexpr int kDirectU = 7;                        // upper bit planes: at most 4095 rows per warp
+constexpr int kDirectRows = 4064 * kDirectWarps;   // rows of a task, at most
+constexpr int kDirectBatch = 4096;                 // bytes of a batch: 8 int8 rows or 32 2-bit rows of a warp
+constexpr int kDirectRing = 3;
+constexpr int kDirectSmem = kDirectWarps * kDirectRing * kDirectBatch;
+
+__host__ __device__ constexpr int direct_cols(int fmt) { return fmt == PCAL_2BIT ? 32 : 128; }
+
+struct BatchDirectArgs {
+    const BatchDirect* dirs;
+    int n_dirs;
+    int total_tasks;
+    BatchChan* ch;
+    unsigned long long* ctr;  // as the persistent fold's; [0] hands out tasks
+    const BatchPiece* pieces;
+    int n_pieces;
+    int n_ch;
+    const long long* n_call;
+};
+
+// 16 bytes of this lane from global to shared memory; zeros where !have.
+__device__ __forceinline__ void copy_async(uint32_t dst, const void* src, bool have, uint64_t policy) {
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;" ::"r"(dst), "l"(src),
+                 "r"(have ? 16 : 0), "l"(policy)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void copy_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+
+// Bin of sample `off` behind bin `base` (both below 2^21).
+__device__ __forceinline__ uint32_t wrap_bin(uint32_t base, uint32_t off, uint32_t L) {
+    uint32_t b = base + off;
+    if (b >= L) b -= L;
+    if (b >= L) b %= L;
+    return b;
+}
+
+// The batches of rows [r0, r1) that warp `warp` takes: 4 KB each, ROWS rows of
+// 4096 / ROWS bytes, every kDirectWarps-th.  count(p) folds a batch that lies
+// at p row after row.
+template <int ROWS, class Count>
+__device__ __forceinline__ void direct_batches(const BatchDirect& D, long long r0, long long r1, int col, int warp,
+                                               uint8_t* ring, uint64_t policy, Count count) {
+    constexpr int kLanes = kDirectBatch / ROWS / 16;  // lanes that copy one row
+    constexpr int kStep = 32 / kLanes;                // rows of one copy of the warp
+    const int lane = threadIdx.x & 31, row_in = lane / kLanes, piece = lane % kLanes;
+    const int n = (int)(r1 - r0), all = (n + ROWS - 1) / ROWS;
+    const int mine = all > warp ? (all - warp + kDirectWarps - 1) / kDirectWarps : 0;
+    const bool active = col + 4 * piece < D.cols;
+    // (a lane without columns copies nothing, from an address of the block all the same)
+    const uint32_t* src0 = D.base + r0 * D.row_words + (active ? col + 4 * piece : 0);
+    const uint32_t dst0 = smem_addr(ring) + lane * 16;
+    auto issue = [&](int k) {
+        if (k < mine) {
+            const int row = (warp + k * kDirectWarps) * ROWS + row_in;
+            const uint32_t dst = dst0 + (k % kDirectRing) * kDirectBatch;
+            if (row + ROWS - kStep < n) {  // a whole batch
+                const uint32_t* src = src0 + (long long)row * D.row_words;
+#pragma unroll
+                for (int i = 0; i < ROWS / kStep; ++i, src += kStep * (long long)D.row_words)
+                    copy_async(dst + i * 512, src, active, policy);
+            } else {
+                for (int i = 0; i < ROWS / kStep; ++i) {
+                    const int r = row + i * kStep;
+                    copy_async(dst + i * 512, src0 + (long long)(r < n ? r : 0) * D.row_words, active && r < n, policy);
+                }
+            }
+        }
+        copy_commit();
+    };
+    issue(0);
+    issue(1);
+    for (int k = 0; k < mine; ++k) {
+        issue(k + 2);
+        copy_wait<2>();
+        __syncwarp();  // the other lanes' copies too
+        count(ring + (k % kDirectRing) * kDirectBatch);
+        __syncwarp();  // before the slot is filled again
+    }
+    copy_wait<0>();
+}
+
+// 2-bit: counts of the CTA's rows as the packed words of transpose16x2 in
+// every warp's scratch, added over the warps, then 16 bins a column.
+__device__ __forceinline__ void direct_2bit(const BatchDirect& D, const BatchChan& C, long long r0, long long r1, int col,
+                                            uint32_t base, uint8_t* smem, uint64_t policy) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t w1 = 0, w2 = 0, w4 = 0, w8 = 0, w16 = 0, wu[kDirectU], d1 = 0, d2 = 0, d4 = 0, d8 = 0, du[kDirectU];
+#pragma unroll
+    for (int u = 0; u < kDirectU; ++u) wu[u] = du[u] = 0;
+    uint8_t* ring = smem + warp * kDirectRing * kDirectBatch;
+    direct_batches<32>(D, r0, r1, col, warp, ring, policy, [&](const uint8_t* p) {
+        uint32_t x[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) x[i] = *reinterpret_cast<const uint32_t*>(p + i * 128 + 4 * lane);
+        pcal_bits::add32<kDirectU>(x, w1, w2, w4, w8, w16, wu, d1, d2, d4, d8, du);
+    });
+    // positions 2j (l) and 2j + 1 (h) of sample j: word position % 16, half
+    // position / 16; words 0..15 the l and h sums, 16..31 the (h AND l) sums
+    uint32_t* sm = reinterpret_cast<uint32_t*>(ring);
+    uint32_t A[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) A[i] = 0;
+    A[0] = w1;
+    A[1] = w2;
+    A[2] = w4;
+    A[3] = w8;
+    A[4] = w16;
+#pragma unroll
+    for (int u = 0; u < kDirectU; ++u) A[5 + u] = wu[u];
+    pcal_bits::transpose16x2(A);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sm[i * 33 + lane] = A[i];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) A[i] = 0;
+    A[0] = d1;
+    A[1] = d2;
+    A[2] = d4;
+    A[3] = d8;
+#pragma unroll
+    for (int u = 0; u < kDirectU; ++u) A[4 + u] = du[u];
+    pcal_bits::transpose16x2(A);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sm[(16 + i) * 33 + lane] = A[i];
+    __syncthreads();
+    // (at most 16,256 rows: no half of a sum overflows)
+    uint32_t* s0 = reinterpret_cast<uint32_t*>(smem);
+    constexpr int kPitch = kDirectRing * kDirectBatch / 4;
+#pragma unroll
+    for (int i = threadIdx.x; i < 1024; i += kDirectThreads) {
+        uint32_t* q = s0 + (i >> 5) * 33 + (i & 31);
+        uint32_t v = 0;
+#pragma unroll
+        for (int w = 0; w < kDirectWarps; ++w) v += q[w * kPitch];
+        q[0] = v;
+    }
+    __syncthreads();
+    unsigned long long* wide = C.wide2;
+    const uint32_t L = (uint32_t)C.L;
+    const int tasks = (D.cols - col < 32 ? D.cols - col : 32) * 16;
+#pragma unroll 2
+    for (int t = threadIdx.x; t < tasks; t += kDirectThreads) {
+        const int cl = t >> 4, j = t & 15;
+        const int pl = 2 * j, ph = 2 * j + 1;
+        const uint32_t sl = (s0[(pl & 15) * 33 + cl] >> (16 * (pl >> 4))) & 0xFFFFu;
+        const uint32_t sh = (s0[(ph & 15) * 33 + cl] >> (16 * (ph >> 4))) & 0xFFFFu;
+        const uint32_t shl = ((s0[(16 + (pl & 15)) * 33 + cl] >> (16 * (pl >> 4))) & 0xFFFFu) +
+                             ((s0[(16 + (ph & 15)) * 33 + cl] >> (16 * (ph >> 4))) & 0xFFFFu);
+        const uint32_t bin = wrap_bin(base, (uint32_t)t, L);
+        if (sl) atomicAdd(&wide[bin], (unsigned long long)sl);
+        if (sh) atomicAdd(&wide[L + bin], (unsigned long long)sh);
+        if (shl) atomicAdd(&wide[2 * L + bin], (unsigned long long)shl);
+    }
+}
+
+__device__ __forceinline__ void direct_i8(const BatchDirect& D, const BatchChan& C, long long r0, long long r1, int col,
+                                          uint32_t base, uint8_t* smem, uint64_t policy) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int s[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) s[i] = 0;
+    uint8_t* ring = smem + warp * kDirectRing * kDirectBatch;
+    direct_batches<8>(D, r0, r1, col, warp, ring, policy, [&](const uint8_t* p) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint4 v = *reinterpret_cast<const uint4*>(p + i * 512 + 16 * lane);
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                s[4 * q] = __dp4a((int)w[q], 0x00000001, s[4 * q]);
+                s[4 * q + 1] = __dp4a((int)w[q], 0x00000100, s[4 * q + 1]);
+                s[4 * q + 2] = __dp4a((int)w[q], 0x00010000, s[4 * q + 2]);
+                s[4 * q + 3] = __dp4a((int)w[q], 0x01000000, s[4 * q + 3]);
+            }
+        }
+    });
+    int* sm = reinterpret_cast<int*>(ring);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sm[lane * 17 + i] = s[i];
+    __syncthreads();
+    const int left = (D.cols - col) * 4;
+    const int tasks = left < 512 ? left : 512;
+    const uint32_t L = (uint32_t)C.L;
+    const int* s0 = reinterpret_cast<const int*>(smem);
+    constexpr int kPitch = kDirectRing * kDirectBatch / 4;
+#pragma unroll 4
+    for (int t = threadIdx.x; t < tasks; t += kDirectThreads) {
+        const int* q = s0 + (t >> 4) * 17 + (t & 15);
+        int v = 0;
+#pragma unroll
+        for (int w = 0; w < kDirectWarps; ++w) v += q[w * kPitch];
+        if (v) atomicAdd(reinterpret_cast<unsigned long long*>(&C.acc8[wrap_bin(base, (uint32_t)t, L)]),
+                         (unsigned long long)(long long)v);
+    }
+}
+
+__global__ void __launch_bounds__(kDirectThreads, kDirectCtas)
+    batch_direct_kernel(const __grid_constant__ BatchDirectArgs a) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ int s_next, s_last;
+    // the preceding kernel (a finalize or a fold of the same channels) has
+    // completed and its bins, indices and counters are visible
+    grid_dependency_wait();
+    allow_dependents();
+    const uint64_t policy = l2_policy_evict_first();
+    // the first task by CTA number, the others from the counter, asked for
+    // one task ahead
+    int t = blockIdx.x;
+    while (t < a.total_tasks) {
+        int next = 0;
+        if (threadIdx.x == 0) next = (int)gridDim.x + (int)atomicAdd(&a.ctr[0], 1ull);
+        int lo = 0, hi = a.n_dirs - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.dirs[mid].task0 <= t)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        const BatchDirect D = a.dirs[lo];
+        const BatchChan& C = a.ch[D.ch];
+        const int rel = t - D.task0;
+        const int chunk = rel / D.blocks, block = rel - chunk * D.blocks;
+        const long long r0 = (long long)chunk * D.chunk_rows;
+        const long long r1 = r0 + D.chunk_rows < D.rows ? r0 + D.chunk_rows : D.rows;
+        const int col = block * direct_cols(C.fmt);
+        // bin of the block's first sample (rows are whole periods)
+        const uint32_t base = (uint32_t)((C.n_abs + D.head + (long long)col * C.spw) % C.L);
+        if (C.fmt == PCAL_2BIT)
+            direct_2bit(D, C, r0, r1, col, base, smem, policy);
+        else
+            direct_i8(D, C, r0, r1, col, base, smem, policy);
+        if (threadIdx.x == 0) s_next = next;
+        __syncthreads();  // (and the rings are free again)
+        t = s_next;
+        __syncthreads();
+    }
+    // what is left over at the regions' ends (under 16 bytes each)
+    for (int pi = blockIdx.x * kDirectWarps + threadIdx.x / 32; pi < a.n_pieces; pi += gridDim.x * kDirectWarps)
+        fold_piece(a.pieces[pi], a.ch, threadIdx.x & 31, 32);
+    // the last CTA advances the indices and zeroes the counters (every CTA
+    // has read the indices it needs before its ticket)
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&a.ctr[2], 1ull) == (unsigned long long)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        for (int c = threadIdx.x; c < a.n_ch; c += blockDim.x) a.ch[c].n_abs += a.n_call[c];
+        if (threadIdx.x == 0) {
+            a.ctr[0] = 0;
+            a.ctr[1] = 0;
+            a.ctr[2] = 0;
+        }
+    }
+}
+
 __global__ void batch_tables_kernel(double2* tw, int64_t L, float2* twN, int64_t N, int64_t sc) {
     for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < L; m += (int64_t)gridDim.x * blockDim.x) {
         double s, c;
@@ -556,6 +839,7 @@ struct pcal_batch {
     pcal_stats stats;
     int dft_mode;                 // PCAL_DFT_FP32: the DFT inside each channel's cluster
     std::vector<DftGroup> dft;    // tensor-core modes: one group per distinct N
+    bool sched_set;               // the schedule was set or tuned: every call takes the persistent fold
 };
 
 int batch_shape(const pcal_schedule& sc, int cw_max, int num_sms, BatchShape* s) {
@@ -588,9 +872,70 @@ int batch_shape(const pcal_schedule& sc, int cw_max, int num_sms, BatchShape* s)
     z.run_boxes = kRunRows / z.box_rows;
     z.static_pct = sc.static_pct;
     z.min_chunk = sc.min_chunk > 0 ? sc.min_chunk : 1;
+    z.num_sms = num_sms;
     *s = z;
     return 0;
 }
+
+namespace {
+
+// The tasks of a call for the direct fold: the rows of every region, the whole
+// 16-byte words behind its last row as a part of one row, and what is left
+// (under 16 bytes at either end) as pieces.  About eight tasks per resident
+// CTA, so that the last ones end close together, but of at least 64 int8 or
+// 128 2-bit rows: the atomic adds of a task's 512 bins cost as much as its
+// loads below that.
+int direct_tasks(const BatchChan* h_ch, const std::vector<BatchRegion>& regions, const BatchShape& sh,
+                 std::vector<BatchDirect>* dirs, std::vector<BatchPiece>* pieces, int* total) {
+    int64_t all = 0;
+    for (const BatchRegion& rg : regions) all += h_ch[rg.ch].fmt == PCAL_2BIT ? rg.n / 4 : rg.n;
+    const int64_t task_bytes = all / (8 * sh.num_sms * kDirectCtas) + 1;
+    int64_t tasks = 0;
+    for (const BatchRegion& rg : regions) {
+        if (rg.n == 0) continue;
+        const BatchChan& C = h_ch[rg.ch];
+        const int spb = C.fmt == PCAL_2BIT ? 4 : 1;
+        const int64_t nbytes = rg.n / spb, row_bytes = C.row_samples / spb;
+        int64_t head = (int64_t)((16 - (reinterpret_cast<uintptr_t>(rg.ptr) & 15)) & 15);
+        if (head > nbytes) head = nbytes;
+        const int64_t rows = (nbytes - head) / row_bytes;
+        const int64_t part = (nbytes - head - rows * row_bytes) / 16 * 16;
+        const int64_t tail = nbytes - head - rows * row_bytes - part;
+        auto add = [&](int64_t at, int64_t n_rows, int64_t words) {
+            const int block_cols = direct_cols(C.fmt);
+            BatchDirect D{};
+            D.base = reinterpret_cast<const uint32_t*>(rg.ptr + at);
+            D.rows = n_rows;
+            D.head = rg.off + at * spb;
+            D.ch = rg.ch;
+            D.cols = (int)words;
+            D.row_words = C.cols_total;
+            D.blocks = (int)((words + block_cols - 1) / block_cols);
+            int64_t chunk = task_bytes / (4 * block_cols);
+            const int64_t least = C.fmt == PCAL_2BIT ? 128 : 64;
+            if (chunk < least) chunk = least;
+            if (chunk > kDirectRows) chunk = kDirectRows;
+            const int64_t parts = (n_rows + chunk / 2) / chunk > 0 ? (n_rows + chunk / 2) / chunk : 1;
+            chunk = (n_rows + parts - 1) / parts;
+            if (chunk > kDirectRows) chunk = kDirectRows;
+            D.chunk_rows = (int)((chunk + 31) / 32 * 32 <= kDirectRows ? (chunk + 31) / 32 * 32 : chunk);
+            D.task0 = (int)tasks;
+            tasks += (int64_t)D.blocks * ((n_rows + D.chunk_rows - 1) / D.chunk_rows);
+            dirs->push_back(D);
+        };
+        if (head > 0) pieces->push_back(BatchPiece{rg.ptr, head * spb, rg.off, rg.ch, 0});
+        if (rows > 0) add(head, rows, C.cols_total);
+        if (part > 0) add(head + rows * row_bytes, 1, part / 4);
+        if (tail > 0)
+            pieces->push_back(
+                BatchPiece{rg.ptr + nbytes - tail, tail * spb, rg.off + (nbytes - tail) * spb, rg.ch, 0});
+        if (tasks >= (1ll << 30)) return PCAL_ETOOLARGE;
+    }
+    *total = (int)tasks;
+    return PCAL_OK;
+}
+
+}  // namespace
 
 int batch_build(const BatchChan* h_ch, int n_ch, const std::vector<BatchRegion>& regions, const BatchShape& sh,
                 const std::vector<int>& fin_list, BatchCallDesc* out) {
@@ -598,9 +943,18 @@ int batch_build(const BatchChan* h_ch, int n_ch, const std::vector<BatchRegion>&
     if (!enc) return PCAL_ECUDA;
     std::vector<CUtensorMap> maps;
     std::vector<BatchSeg> segs;
+    std::vector<BatchDirect> dirs;
     std::vector<BatchPiece> pieces;
     std::vector<long long> ncall(n_ch, 0);
     long long total = 0;
+    int total_tasks = 0;
+    for (const BatchRegion& rg : regions)
+        if (rg.ch < 0 || rg.ch >= n_ch || rg.n < 0) return PCAL_EINVAL;
+    const bool direct = sh.direct;
+    if (direct) {
+        const int rc = direct_tasks(h_ch, regions, sh, &dirs, &pieces, &total_tasks);
+        if (rc != PCAL_OK) return rc;
+    }
     // a ragged run as pieces of at most kPieceBytes (one CTA folds a piece)
     auto add_run = [&](const uint8_t* p, int64_t n, int64_t off, int ch, int spb) {
         const int64_t step = kPieceBytes * spb;
@@ -608,11 +962,10 @@ int batch_build(const BatchChan* h_ch, int n_ch, const std::vector<BatchRegion>&
             pieces.push_back(BatchPiece{p + o / spb, n - o < step ? n - o : step, off + o, ch, 0});
     };
     for (const BatchRegion& rg : regions) {
-        if (rg.ch < 0 || rg.ch >= n_ch || rg.n < 0) return PCAL_EINVAL;
         const BatchChan& C = h_ch[rg.ch];
         const int64_t nc = rg.n;
         ncall[rg.ch] += nc;
-        if (nc == 0) continue;
+        if (nc == 0 || direct) continue;
         const uint8_t* p = rg.ptr;
         const int spb = C.fmt == PCAL_2BIT ? 4 : 1;  // samples per byte
         const int64_t nbytes = nc / spb;
@@ -664,17 +1017,21 @@ int batch_build(const BatchChan* h_ch, int n_ch, const std::vector<BatchRegion>&
     BatchCallDesc d;
     d.off_maps = 0;
     d.off_segs = align_up(sizeof(CUtensorMap) * maps.size(), 128);
-    d.off_pieces = align_up(d.off_segs + sizeof(BatchSeg) * segs.size(), 128);
+    d.off_dirs = align_up(d.off_segs + sizeof(BatchSeg) * segs.size(), 128);
+    d.off_pieces = align_up(d.off_dirs + sizeof(BatchDirect) * dirs.size(), 128);
     d.off_n = align_up(d.off_pieces + sizeof(BatchPiece) * pieces.size(), 128);
     d.off_list = align_up(d.off_n + sizeof(long long) * ncall.size(), 128);
     const size_t bytes = align_up(d.off_list + sizeof(int) * fin_list.size(), 128);
     d.blob.assign(bytes, 0);
     if (!maps.empty()) memcpy(d.blob.data() + d.off_maps, maps.data(), sizeof(CUtensorMap) * maps.size());
     if (!segs.empty()) memcpy(d.blob.data() + d.off_segs, segs.data(), sizeof(BatchSeg) * segs.size());
+    if (!dirs.empty()) memcpy(d.blob.data() + d.off_dirs, dirs.data(), sizeof(BatchDirect) * dirs.size());
     if (!pieces.empty()) memcpy(d.blob.data() + d.off_pieces, pieces.data(), sizeof(BatchPiece) * pieces.size());
     memcpy(d.blob.data() + d.off_n, ncall.data(), sizeof(long long) * ncall.size());
     if (!fin_list.empty()) memcpy(d.blob.data() + d.off_list, fin_list.data(), sizeof(int) * fin_list.size());
     d.n_segs = (int)segs.size();
+    d.n_dirs = (int)dirs.size();
+    d.total_tasks = total_tasks;
     d.n_pieces = (int)pieces.size();
     d.n_list = (int)fin_list.size();
     d.total_boxes = total;
@@ -687,7 +1044,34 @@ cudaError_t batch_launch_fold(const BatchCallDesc& d, void* d_desc, BatchChan* d
                               int* launches) {
     uint8_t* base = static_cast<uint8_t*>(d_desc);
     *launches = 0;
-    if (d.total_boxes == 0 && d.n_pieces == 0) return cudaSuccess;  // no samples in the call
+    if (d.total_boxes == 0 && d.total_tasks == 0 && d.n_pieces == 0) return cudaSuccess;  // no samples in the call
+    if (d.total_tasks > 0) {
+        BatchDirectArgs a{};
+        a.dirs = reinterpret_cast<const BatchDirect*>(base + d.off_dirs);
+        a.n_dirs = d.n_dirs;
+        a.total_tasks = d.total_tasks;
+        a.ch = d_ch;
+        a.ctr = d_ctr;
+        a.pieces = reinterpret_cast<const BatchPiece*>(base + d.off_pieces);
+        a.n_pieces = d.n_pieces;
+        a.n_ch = n_ch;
+        a.n_call = reinterpret_cast<const long long*>(base + d.off_n);
+        const int most = sh.num_sms * kDirectCtas;
+        const int grid = d.total_tasks < most ? d.total_tasks : most;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3(kDirectThreads);
+        cfg.dynamicSmemBytes = kDirectSmem;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, batch_direct_kernel, a);
+        if (e == cudaSuccess) *launches = 1;
+        return e;
+    }
     BatchFoldArgs a{};
     a.maps = reinterpret_cast<const CUtensorMap*>(base + d.off_maps);
     a.segs = reinterpret_cast<const BatchSeg*>(base + d.off_segs);
@@ -729,6 +1113,8 @@ cudaError_t batch_launch_fold(const BatchCallDesc& d, void* d_desc, BatchChan* d
 }
 
 cudaError_t batch_prepare_fold() {
+    const cudaError_t e = cudaFuncSetAttribute(batch_direct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDirectSmem);
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(batch_fold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
 }
 
@@ -814,7 +1200,11 @@ void batch_place_chan(BatchChan& C, const pcal_geometry& g, uint8_t* base) {
 
 namespace {
 
-int shape_for(const pcal_batch* b, BatchShape* s) { return batch_shape(b->sched, b->cw_max, b->num_sms, s); }
+int shape_for(const pcal_batch* b, BatchShape* s) {
+    const int rc = batch_shape(b->sched, b->cw_max, b->num_sms, s);
+    s->direct = !b->sched_set;
+    return rc;
+}
 
 // Column groups of every channel under a schedule's caps (the rule of
 // batch_fill_chan), and the widest group.
@@ -846,7 +1236,7 @@ cudaError_t launch_call(pcal_batch* b, const BatchCallDesc& d, void* d_desc, uns
     int launches = 0;
     const cudaError_t e = batch_launch_fold(d, d_desc, b->d_ch, b->n, d_ctr, sh, b->d_err, s, &launches);
     b->stats.kernel_launches += launches;
-    if (d.total_boxes > 0) b->stats.bulk_launches += 1;
+    if (d.total_boxes > 0 || d.total_tasks > 0) b->stats.bulk_launches += 1;
     return e;
 }
 
@@ -1077,6 +1467,7 @@ extern "C" int pcal_batch_set_schedule(pcal_batch* b, const pcal_schedule* s) {
         apply_col_caps(b, old);
         return PCAL_EINVAL;
     }
+    b->sched_set = true;
     return PCAL_OK;
 }
 
@@ -1377,6 +1768,11 @@ extern "C" int pcal_batch_autotune(pcal_batch* b, const void* const* samples, co
         }
         return rc == PCAL_OK ? ms / reps : -1.f;
     };
+    // the direct fold, which has no schedule: kept where no candidate is faster
+    const bool set_keep = b->sched_set;
+    b->sched_set = false;
+    const float direct_ms = time_cand(keep, 6);
+    b->sched_set = true;
     // pass 1, batch-wide: every candidate briefly, then the four fastest again with more runs
     std::vector<std::pair<float, int>> score;
     for (int i = 0; i < (int)cand.size() && rc == PCAL_OK; ++i) {
@@ -1444,9 +1840,11 @@ extern "C" int pcal_batch_autotune(pcal_batch* b, const void* const* samples, co
     }
     if (e == cudaSuccess)
         e = cudaMemcpy(b->d_ch, b->h_ch.data(), sizeof(BatchChan) * b->n, cudaMemcpyHostToDevice);
+    b->sched_set = set_keep;
     if (e != cudaSuccess) return PCAL_ECUDA;
     if (rc != PCAL_OK) return rc;
     rc = pcal_batch_set_schedule(b, &best_s);
+    if (rc == PCAL_OK && direct_ms >= 0.f && direct_ms <= best) b->sched_set = false;
     if (rc == PCAL_OK && chosen) *chosen = best_s;
     return rc;
 }

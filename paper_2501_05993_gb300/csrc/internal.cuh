@@ -202,6 +202,20 @@ struct BatchSeg {
     long long head;       // samples of the channel in this call before its first bulk row
 };
 
+// One block of rows (or a part of one row) of a call that the direct fold
+// takes: warp tasks task0 .. task0 + blocks * chunks - 1, column blocks fastest.
+struct BatchDirect {
+    const uint32_t* base;  // first word of row 0, 16-byte aligned
+    long long rows;
+    long long head;        // samples of the channel in this call before row 0
+    int ch;
+    int cols;              // words of a row that are folded, a multiple of 4
+    int row_words;         // words between rows
+    int blocks;            // column blocks (kDirectCols words of the channel's format)
+    int chunk_rows;        // rows of a task
+    int task0;
+};
+
 // A ragged run (head or tail) of one accumulate call.
 struct BatchPiece {
     const uint8_t* ptr;   // its first byte
@@ -249,15 +263,18 @@ struct BatchShape {
     int wpr, replicas, box_rows, stages, merge_stride, threads, grid, run_boxes, static_pct, min_chunk;
     uint32_t stage_stride;
     size_t smem;
+    bool direct;   // short calls may take the direct fold
+    int num_sms;
 };
 
 // Device descriptors of one call: tensor maps, segments, pieces, samples per
 // channel, and the channels to finalize.
 struct BatchCallDesc {
     std::vector<uint8_t> blob;  // host image of the device buffer
-    size_t off_maps, off_segs, off_pieces, off_n, off_list;
-    int n_segs, n_pieces, n_list;
+    size_t off_maps, off_segs, off_dirs, off_pieces, off_n, off_list;
+    int n_segs, n_dirs, n_pieces, n_list;
     long long total_boxes;
+    int total_tasks;  // > 0: the direct fold takes the call
 };
 
 int batch_shape(const pcal_schedule& sc, int cw_max, int num_sms, BatchShape* s);

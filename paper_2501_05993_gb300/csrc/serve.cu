@@ -288,6 +288,7 @@ void worker_loop(pcal_server* s) {
     cudaSetDevice(s->device);
     BatchShape sh;
     batch_shape(s->sched, s->cw_max, s->num_sms, &sh);
+    sh.direct = true;  // 10 ms chunks and the like
     for (;;) {
         std::vector<BatchRegion> regions;
         std::vector<int> fin_slots;
