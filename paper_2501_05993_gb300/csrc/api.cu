@@ -133,7 +133,7 @@ extern "C" int pcal_plan_create(double fs, double f_comb, double f_offset, int N
             e = dalloc(&p->d_accf, 2 * L);
         }
     }
-    if (e == cudaSuccess) e = dalloc(&p->d_tw, L);
+    if (e == cudaSuccess) e = dalloc(reinterpret_cast<double2**>(&p->d_tw), L);
     if (e == cudaSuccess) e = dalloc(&p->d_twN, Nn);
     if (e == cudaSuccess) e = dalloc(&p->d_P, Nn);
     if (e == cudaSuccess) e = dalloc(&p->d_T, Nn);

@@ -703,7 +703,7 @@ __device__ __forceinline__ void direct_i8(const BatchDirect& D, const BatchChan&
 
 __global__ void __launch_bounds__(kDirectThreads, kDirectCtas)
     batch_direct_kernel(const __grid_constant__ BatchDirectArgs a) {
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ int s_next, s_last;
     // the preceding kernel (a finalize or a fold of the same channels) has
     // completed and its bins, indices and counters are visible
@@ -761,15 +761,6 @@ __global__ void __launch_bounds__(kDirectThreads, kDirectCtas)
             a.ctr[1] = 0;
             a.ctr[2] = 0;
         }
-    }
-}
-
-__global__ void batch_tables_kernel(double2* tw, int64_t L, float2* twN, int64_t N, int64_t sc) {
-    for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < L; m += (int64_t)gridDim.x * blockDim.x) {
-        double s, c;
-        sincospi(2.0 * (double)m / (double)L, &s, &c);
-        tw[m] = make_double2(c, -s);
-        if (m % sc == 0 && m / sc < N) twN[m / sc] = make_float2((float)c, (float)-s);
     }
 }
 
@@ -1119,11 +1110,7 @@ cudaError_t batch_prepare_fold() {
 }
 
 cudaError_t batch_launch_tables(BatchChan& C, const pcal_geometry& g, cudaStream_t s) {
-    int grid = (int)((g.L + 255) / 256);
-    if (grid > 1024) grid = 1024;
-    batch_tables_kernel<<<grid, 256, 0, s>>>(const_cast<double2*>(C.tw), g.L, const_cast<float2*>(C.twN), g.N,
-                                             g.step_comb);
-    return cudaGetLastError();
+    return launch_rotators(true, const_cast<int4*>(C.twi), g.L, const_cast<float2*>(C.twN), g.N, g.step_comb, s);
 }
 
 // Fill the constant part of a channel's device record (pointers excluded).
@@ -1163,6 +1150,9 @@ void batch_fill_chan(BatchChan& C, const pcal_geometry& g, double f_comb, const 
     C.c_l = g.format == PCAL_2BIT ? lv[1] - lv[0] : 0.0;
     C.c_h = g.format == PCAL_2BIT ? lv[2] - lv[0] : 0.0;
     C.c_hl = g.format == PCAL_2BIT ? lv[3] - lv[2] - lv[1] + lv[0] : 0.0;
+    C.k_c = g.format == PCAL_2BIT ? 0.5 * (lv[1] + lv[2]) : 0.0;
+    C.k_a = g.format == PCAL_2BIT ? C.k_c - lv[0] : 0.0;
+    C.k_b = g.format == PCAL_2BIT ? 0.5 * (lv[2] - lv[1]) : 0.0;
     C.two_pi_fc = 6.283185307179586476925 * f_comb;
     C.fs = (double)g.fs;
 }
@@ -1171,7 +1161,7 @@ void batch_fill_chan(BatchChan& C, const pcal_geometry& g, double f_comb, const 
 size_t batch_chan_bytes(const pcal_geometry& g) {
     const size_t L = (size_t)g.L, N = (size_t)g.N;
     size_t n = 0;
-    if (g.format == PCAL_2BIT) n += align_up(8 * L, 256) + align_up(24 * L, 256);
+    if (g.format == PCAL_2BIT) n += align_up(24 * L, 256);
     if (g.format == PCAL_I8) n += align_up(8 * L, 256);
     n += align_up(16 * L, 256) + align_up(8 * N, 256) + align_up(8 * (6 * N + 5), 256);
     return n;
@@ -1182,8 +1172,6 @@ void batch_place_chan(BatchChan& C, const pcal_geometry& g, uint8_t* base) {
     const size_t L = (size_t)g.L, N = (size_t)g.N;
     size_t o = 0;
     if (g.format == PCAL_2BIT) {
-        C.zero2 = reinterpret_cast<unsigned long long*>(base + o);
-        o += align_up(8 * L, 256);
         C.wide2 = reinterpret_cast<unsigned long long*>(base + o);
         o += align_up(24 * L, 256);
     }
@@ -1191,7 +1179,7 @@ void batch_place_chan(BatchChan& C, const pcal_geometry& g, uint8_t* base) {
         C.acc8 = reinterpret_cast<long long*>(base + o);
         o += align_up(8 * L, 256);
     }
-    C.tw = reinterpret_cast<double2*>(base + o);
+    C.twi = reinterpret_cast<const int4*>(base + o);
     o += align_up(16 * L, 256);
     C.twN = reinterpret_cast<float2*>(base + o);
     o += align_up(8 * N, 256);

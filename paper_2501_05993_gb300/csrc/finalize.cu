@@ -2,10 +2,12 @@
 // and the delay (paper Sec. 2).
 //
 //   decode   S[k] from the exact bins (2-bit: the level table applied to the
-//            per-code counts; int8/float32: the sums)                 FP64
-//   rotate   R[k] = S[k] * exp(-j*2*pi*f_offset*k/fs)        (Eq. 3)  FP64
-//   fold     P[b] = sum_m R[b + m*N]                          (Eq. 2)  FP64
-//            per thread, then double-float (df) across threads
+//            per-code counts; int8/float32: the sums)
+//   rotate   R[k] = S[k] * exp(-j*2*pi*f_offset*k/fs)        (Eq. 3)
+//   fold     P[b] = sum_m R[b + m*N]                          (Eq. 2)
+//            integer bins: exact sums of integer x fixed-point rotator per
+//            thread (residue_int), float32 bins FP64 per thread; then
+//            double-float (df) across threads
 //   DFT      T_i = sum_b P[b] exp(-j*2*pi*i*b/N)   (DFT(P), Sec. 2)   FP32
 //   products amp_i = 2|T_i|/M and phase arg(T_i)+pi/2 (sin model of Eq. 1)
 //            in FP32; the phase unwrapped along the comb and the delay as
@@ -46,12 +48,14 @@ constexpr int kFmtRotated = 16;  // cluster finalize of bins that are rotated al
 
 struct FinArgs {
     int fmt;
-    int spilled;  // 2-bit: the wide arrays hold counts of this period
+    int spilled;  // 2-bit: 1 the wide arrays hold counts of this period too, 2 they alone do
     int bc;   // residues b per fold CTA
     int tpb;  // threads per residue (power of two)
     int64_t L, N, so;
     int64_t q, rem, a0;  // samples in bin k: q + ((k - a0) mod L < rem)
     double lev0, c_l, c_h, c_hl;
+    int exact;             // integer bins small enough for residue_int
+    df k_a, k_b, k_c, k_h; // 2-bit: weights of residue_int's sums
     double M;
     float two_over_m;
     df two_pi_fc;  // 2*pi*f_comb in df
@@ -67,7 +71,8 @@ struct FinArgs {
     int64_t pf_cols;
     const long long* counts4;  // no-allocation entry: the caller's counts [L][4]
     double lev[4];             // no-allocation entry: the code levels
-    const double2* tw;
+    const double2* tw;     // float32 bins: exp(-j 2 pi m/L)
+    const int4* twi;       // integer bins: the same in fixed point (rotator_fixed)
     const float2* twN;
     float4* P;     // P[b] as df re (x, y), df im (z, w)
     float2* T;     // FP32 tone phasors
@@ -89,7 +94,7 @@ __device__ __forceinline__ double read_bin(const FinArgs& a, int64_t k) {
         return a.lev[0] * (double)c[0] + a.lev[1] * (double)c[1] + a.lev[2] * (double)c[2] + a.lev[3] * (double)c[3];
     }
     if (fmt == PCAL_2BIT) {
-        const unsigned long long v = a.acc2[k];
+        const unsigned long long v = a.spilled == 2 ? 0ull : a.acc2[k];
         unsigned long long sl = v & PCAL_F21_MASK, sh = (v >> 21) & PCAL_F21_MASK, shl = (v >> 42) & PCAL_F21_MASK;
         if (a.spilled) {
             sl += a.wide2[k];
@@ -133,6 +138,16 @@ __device__ __forceinline__ double read_bin(const FinArgs& a, int64_t k) {
     return (double)s.hi + (double)s.lo;
 }
 
+// The rotator table of integer bins: each component as W = round(x * 2^54) in
+// two halves, W = hi * 2^27 + lo with 0 <= lo < 2^27 (an FP64 sincospi rounds
+// at 2^-54 near 1, so nothing is lost).
+constexpr int kRotBits = 54, kRotHalf = 27;
+
+__device__ __forceinline__ int2 rotator_fixed(double x) {
+    const long long W = llrint(x * (double)(1ll << kRotBits));
+    return make_int2((int)(W >> kRotHalf), (int)(W & ((1ll << kRotHalf) - 1)));
+}
+
 // exp(-j*2*pi*m/L): the plan's table; NoAlloc evaluates it here.
 template <bool NoAlloc>
 __device__ __forceinline__ double2 rotator(const FinArgs& a, int64_t m) {
@@ -140,6 +155,11 @@ __device__ __forceinline__ double2 rotator(const FinArgs& a, int64_t m) {
         double sn, cs;
         sincospi(2.0 * (double)m / (double)a.L, &sn, &cs);
         return make_double2(cs, -sn);
+    }
+    if (a.twi) {
+        const int4 w = a.twi[m];
+        constexpr double kHi = 1.0 / (double)(1ll << (kRotBits - kRotHalf)), kLo = 1.0 / (double)(1ll << kRotBits);
+        return make_double2(fma((double)w.x, kHi, (double)w.y * kLo), fma((double)w.z, kHi, (double)w.w * kLo));
     }
     return a.tw[m];
 }
@@ -151,7 +171,7 @@ template <int FMT = -1>
 __device__ __forceinline__ void clear_bin(const FinArgs& a, int64_t k) {
     const int fmt = FMT < 0 ? a.fmt : FMT;
     if (fmt == PCAL_2BIT) {
-        a.acc2[k] = 0;
+        if (a.spilled != 2) a.acc2[k] = 0;
         if (a.spilled) {
             a.wide2[k] = 0;
             a.wide2[a.L + k] = 0;
@@ -576,6 +596,8 @@ struct ClusterSmem {
 };
 
 __host__ __device__ inline size_t cluster_smem_bytes(int64_t N) { return (size_t)N * 56 + 16; }
+// ... and of its LARGE form, the block's products behind it.
+__host__ __device__ inline size_t large_smem_bytes(int64_t N) { return cluster_smem_bytes(N) + products_bytes(N); }
 
 __device__ inline ClusterSmem cluster_layout(uint8_t* base, int64_t N) {
     ClusterSmem m;
@@ -704,7 +726,6 @@ __device__ void write_results_block(const FinArgs& a, const float2* sT, const Wa
 // below m_end (bins k = b + m*N), clearing each bin; returns the FP64 sum.
 template <int FMT = -1>
 __device__ __forceinline__ double2 fold_residue(const FinArgs& a, int b, int m, int step, int m_end) {
-    const int fmt = FMT < 0 ? a.fmt : FMT;
     double re = 0.0, im = 0.0;
     if (m >= m_end) return make_double2(0.0, 0.0);
     const int L = (int)a.L, N = (int)a.N;
@@ -712,41 +733,160 @@ __device__ __forceinline__ double2 fold_residue(const FinArgs& a, int b, int m, 
     int idx = (int)((a.so * k) % L);  // rotator index (f_offset/g * k) mod L
     const int kstep = step * N;
     const int istep = (int)((a.so * kstep) % L);
-    if (fmt == PCAL_2BIT && !a.spilled) {
-        // S = lev0*cnt + c_l*sum(l) + c_h*sum(h) + c_hl*sum(h AND l),
-        // cnt = q or q + 1; the fields are below 2^21
-        const double s_q = a.lev0 * (double)a.q, s_q1 = a.lev0 * (double)(a.q + 1);
-        const int a0 = (int)a.a0, rem = (int)a.rem;
-#pragma unroll 2
-        for (; m < m_end; m += step) {
-            const unsigned long long v = a.acc2[k];
-            const double2 w = a.tw[idx];
-            a.acc2[k] = 0;
-            int rr = k - a0;
-            if (rr < 0) rr += L;
-            const double S = fma(a.c_hl, (double)(int)((v >> 42) & PCAL_F21_MASK),
-                                 fma(a.c_h, (double)(int)((v >> 21) & PCAL_F21_MASK),
-                                     fma(a.c_l, (double)(int)(v & PCAL_F21_MASK), rr < rem ? s_q1 : s_q)));
-            re = fma(S, w.x, re);
-            im = fma(S, w.y, im);
-            k += kstep;
-            idx += istep;
-            if (idx >= L) idx -= L;
-        }
-    } else {
 #pragma unroll 1
-        for (; m < m_end; m += step) {
-            const double S = read_bin<false, FMT>(a, k);
-            const double2 w = a.tw[idx];
-            re = fma(S, w.x, re);
-            im = fma(S, w.y, im);
-            clear_bin<FMT>(a, k);
-            k += kstep;
-            idx += istep;
-            if (idx >= L) idx -= L;
-        }
+    for (; m < m_end; m += step) {
+        const double S = read_bin<false, FMT>(a, k);
+        const double2 w = rotator<false>(a, idx);
+        re = fma(S, w.x, re);
+        im = fma(S, w.y, im);
+        clear_bin<FMT>(a, k);
+        k += kstep;
+        idx += istep;
+        if (idx >= L) idx -= L;
     }
     return make_double2(re, im);
+}
+
+// Sum of s * W over bins, exact in 64 bits: high and low halves of W apart.
+struct IntSum {
+    long long rh = 0, rl = 0, ih = 0, il = 0;
+    __device__ __forceinline__ void add(int s, const int4& w) {
+        rh += (long long)s * w.x;
+        rl += (long long)s * w.y;
+        ih += (long long)s * w.z;
+        il += (long long)s * w.w;
+    }
+};
+
+// (hi * 2^27 + lo) * 2^-54 as a double-float; |hi|, |lo| < 2^62.
+__device__ __forceinline__ df int_df(long long hi, long long lo) {
+    hi += lo >> kRotHalf;
+    lo &= (1ll << kRotHalf) - 1;
+    // hi in pieces of 25, 24 and 14 bits: exact floats
+    const float h = (float)(int)(hi >> 38) * 2048.f;
+    const float m = (float)(int)((hi >> 14) & 0xFFFFFF) * (1.f / 8192.f);
+    const float l = (float)(int)(hi & 0x3FFF) * (1.f / 134217728.f);
+    df r = pcal_df::quick_two_sum(h, m);
+    r = pcal_df::add_f(r, l);
+    return pcal_df::add_f(r, (float)(int)lo * (1.f / 18014398509481984.f));
+}
+
+__device__ __forceinline__ void add_scaled(df& re, df& im, const IntSum& s, df k) {
+    re = pcal_df::add(re, pcal_df::mul(int_df(s.rh, s.rl), k));
+    im = pcal_df::add(im, pcal_df::mul(int_df(s.ih, s.il), k));
+}
+
+// Residue b over m = m, m + step, ... below m_end of integer bins, in integers:
+// the decode and rotation of Eq. 3 with no FP64 instruction (GB300 issues two
+// FP64 operations per SM and clock; about 14 of them a 2-bit bin, conversions
+// included, bounded every finalize).  With the sums sl, sh and shl of a bin's l,
+// h and (h AND l) bits over cnt samples, A = sl + sh - cnt and B = sh - sl, the
+// levels v0..v3 give
+//   S = A ((v1 + v2)/2 - v0) + B (v2 - v1)/2 + cnt (v1 + v2)/2
+//       + shl (v3 - v2 - v1 + v0),
+// so the usual antisymmetric levels need two exact sums of (integer x fixed-point
+// rotator) per component, int8 bins one.  a.exact: every factor is below 2^26, so
+// 512 terms stay below 2^62.  The bins are cleared.  Measured: 64 live channels
+// (L up to 102,400) batch finalize 145 -> 108 us, L 12,800 int8 plan finalize
+// 14.5 -> 13.1 us; wide plans (LARGE below) 35 us in two kernels over all SMs
+// after the fold -> one cluster beside the next fold (1024 tones: 91 -> 79 us a
+// step).
+template <int FMT>
+__device__ __forceinline__ float4 residue_int(const FinArgs& a, int b, int m, int step, int m_end) {
+    const int fmt = FMT < 0 ? a.fmt : FMT;
+    df re{0.f, 0.f}, im{0.f, 0.f};
+    if (m >= m_end) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const int L = (int)a.L, N = (int)a.N;
+    int k = b + m * N;
+    int idx = (int)((a.so * k) % L);  // rotator index (f_offset/g * k) mod L
+    const int kstep = step * N;
+    const int istep = (int)((a.so * kstep) % L);
+    const int q = (int)a.q, a0 = (int)a.a0, rem = (int)a.rem;
+    const bool use_c = a.k_c.hi != 0.f, use_h = a.k_h.hi != 0.f;
+    constexpr int U = 4;  // bins in flight
+    while (m < m_end) {
+        const int end = (m_end - m) / step >= 512 ? m + 512 * step : m_end;  // (512: a multiple of U)
+        IntSum A, B, Cn, H;
+        while (m < end) {
+            int4 w[U];
+            int x[U], y[U], z[U], cnt[U];
+            int kk = k;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool in = m + u * step < end;
+                w[u] = make_int4(0, 0, 0, 0);
+                x[u] = y[u] = z[u] = cnt[u] = 0;
+                if (in) {
+                    w[u] = a.twi[idx];
+                    if (fmt == PCAL_2BIT) {
+                        if (a.spilled != 2) {
+                            const unsigned long long v = a.acc2[kk];
+                            x[u] = (int)(v & PCAL_F21_MASK);
+                            y[u] = (int)((v >> 21) & PCAL_F21_MASK);
+                            z[u] = (int)((v >> 42) & PCAL_F21_MASK);
+                        }
+                        if (a.spilled) {
+                            x[u] += (int)a.wide2[kk];
+                            y[u] += (int)a.wide2[L + kk];
+                            if (use_h) z[u] += (int)a.wide2[2 * L + kk];
+                        }
+                        int rr = kk - a0;
+                        if (rr < 0) rr += L;
+                        cnt[u] = q + (rr < rem ? 1 : 0);
+                    } else {
+                        x[u] = (int)a.acc8[kk];
+                    }
+                }
+                kk += kstep;
+                idx += istep;
+                if (idx >= L) idx -= L;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (m + u * step < end) clear_bin<FMT>(a, k);
+                k += kstep;
+                if (fmt == PCAL_2BIT) {
+                    A.add(x[u] + y[u] - cnt[u], w[u]);
+                    B.add(y[u] - x[u], w[u]);
+                    if (use_c) Cn.add(cnt[u], w[u]);
+                    if (use_h) H.add(z[u], w[u]);
+                } else {
+                    A.add(x[u], w[u]);
+                }
+            }
+            m += U * step;
+        }
+        if (fmt == PCAL_2BIT) {
+            add_scaled(re, im, A, a.k_a);
+            add_scaled(re, im, B, a.k_b);
+            if (use_c) add_scaled(re, im, Cn, a.k_c);
+            if (use_h) add_scaled(re, im, H, a.k_h);
+        } else {
+            re = pcal_df::add(re, int_df(A.rh, A.rl));
+            im = pcal_df::add(im, int_df(A.ih, A.il));
+        }
+    }
+    return make_float4(re.hi, re.lo, im.hi, im.lo);
+}
+
+// Whether a period's integer bins fit residue_int: samples per bin below 2^26
+// (2-bit; no level beyond the floats of a double-float) or 2^19 (int8, up to
+// 128 each).
+__host__ __device__ inline int exact_bins(int fmt, int64_t q, double k_a, double k_b, double k_c, double k_h) {
+    if (fmt == PCAL_I8) return q + 1 < (1ll << 19);
+    if (fmt != PCAL_2BIT || q + 1 >= (1ll << 26)) return 0;
+    const double k[4] = {k_a, k_b, k_c, k_h};
+    double most = 0.0;
+    for (double v : k) {
+        const double w = v < 0.0 ? -v : v;
+        if (w > most) most = w;
+    }
+    return most < 1e25 && most > 1e-20;
+}
+
+__host__ __device__ inline df split_df(double x) {
+    const float hi = (float)x;
+    return df{hi, (float)(x - (double)hi)};
 }
 
 // Residue b over m = m, m + step, ... below m_end as double-float (re hi, re
@@ -766,6 +906,8 @@ __device__ __forceinline__ float4 residue_df(const FinArgs& a, int b, int m, int
         }
         return make_float4(re.hi, re.lo, im.hi, im.lo);
     } else {
+        if constexpr (FMT != PCAL_F32)
+            if (a.exact) return residue_int<FMT>(a, b, m, step, m_end);
         const double2 z = fold_residue<FMT>(a, b, m, step, m_end);
         const df dre = df_of(z.x), dim = df_of(z.y);
         return make_float4(dre.hi, dre.lo, dim.hi, dim.lo);
@@ -819,7 +961,11 @@ __device__ void dft_range(const float2* sP, const float2* sTw, int N, int i0, in
 // products.
 // Runs in every CTA of the cluster; returns true in the CTA that wrote the
 // results (rank 0), after it wrote them.
-template <int FMT = -1>
+// LARGE: plans of more than kClusterMaxN tones or of long periods.  Their DFT
+// and products keep the order of operations of fin_dft_kernel and
+// fin_fold_kernel: tones in groups of kDftTonesPerCta (the groups dealt to the
+// CTAs), and the products by the block.
+template <int FMT = -1, bool LARGE = false>
 __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -924,13 +1070,29 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
             for (int i = t; i < N; i += blockDim.x) sP[i] = p0[i];
         }
         __syncthreads();
-        // (long-period plans: in the order of one CTA with all N tones)
-        const int i0 = N * r / C, i1 = N * (r + 1) / C;
-        dft_range(sP, sTw, N, i0, i1, cluster.map_shared_rank(sT, 0), FMT == kFmtRotated ? N : i1 - i0);
+        float2* dst = cluster.map_shared_rank(sT, 0);
+        if constexpr (LARGE) {
+            for (int i0 = r * kDftTonesPerCta; i0 < N; i0 += C * kDftTonesPerCta) {
+                const int n = N - i0 < kDftTonesPerCta ? N - i0 : kDftTonesPerCta;
+                dft_range(sP, sTw, N, i0, i0 + n, dst, n);
+            }
+        } else {
+            // (long-period plans: in the order of one CTA with all N tones)
+            const int i0 = N * r / C, i1 = N * (r + 1) / C;
+            dft_range(sP, sTw, N, i0, i1, dst, FMT == kFmtRotated ? N : i1 - i0);
+        }
         cluster.sync();  // CTA 0 holds every tone; its sP is no longer read
         if (r != 0) return false;
     }
     __syncthreads();
+    if constexpr (LARGE) {
+        const ProductsSmem pm = products_layout(dsm + cluster_smem_bytes(N), N);
+        for (int i = t; i < N; i += blockDim.x) pm.T[i] = sT[i];
+        __syncthreads();
+        tone_products(a, pm);
+        if (a.extra && t < 32) peak_delay_warp(a, sP);
+        return true;
+    }
     if (t < 32) tone_products_warp(a, sT, sm.pm.psi, sm.pm.w, sm.pm.un, sm.pm.out);
     else if (t < 64 && a.extra) peak_delay_warp(a, sP);
     __syncthreads();
@@ -941,13 +1103,13 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
 // One instantiation per sample format: the finalize runs once per step and its
 // instructions come from L2 (slow beside a streaming fold), so each plan's
 // kernel holds only its own format's decode.
-template <int FMT>
+template <int FMT, bool LARGE = false>
 __global__ void __launch_bounds__(kClusterThreads, 1) fin_cluster_kernel(FinArgs a) {
     // The next fold may launch at once: it adds into the other set of bins
     // and waits for this kernel before its first atomic.
     allow_dependents();
     grid_dependency_wait();  // the bins of the preceding fold
-    cluster_finalize<FMT>(a);
+    cluster_finalize<FMT, LARGE>(a);
 }
 
 // Finalize arguments of one batched channel from its device state.
@@ -955,7 +1117,7 @@ __device__ inline FinArgs batch_fin_args(const BatchChan& bc) {
     const int64_t n_tot = bc.n_abs - bc.period_start;
     FinArgs a{};
     a.fmt = bc.fmt;
-    a.spilled = 1;  // 2-bit sums live in the wide arrays; the packed words are zero
+    a.spilled = 2;  // 2-bit sums live in the wide arrays
     a.L = bc.L;
     a.N = bc.N;
     a.so = bc.so;
@@ -970,10 +1132,14 @@ __device__ inline FinArgs batch_fin_args(const BatchChan& bc) {
     a.two_over_m = n_tot > 0 ? (float)(2.0 / (double)n_tot) : 0.0f;
     a.two_pi_fc.hi = (float)bc.two_pi_fc;
     a.two_pi_fc.lo = (float)(bc.two_pi_fc - (double)a.two_pi_fc.hi);
-    a.acc2 = bc.zero2;
+    a.exact = exact_bins(bc.fmt, a.q, bc.k_a, bc.k_b, bc.k_c, bc.c_hl);
+    a.k_a = split_df(bc.k_a);
+    a.k_b = split_df(bc.k_b);
+    a.k_c = split_df(bc.k_c);
+    a.k_h = split_df(bc.c_hl);
     a.wide2 = bc.wide2;
     a.acc8 = bc.acc8;
-    a.tw = bc.tw;
+    a.twi = bc.twi;
     a.twN = bc.twN;
     a.res = bc.res;
     a.extra = bc.res + 5 * bc.N + 3;
@@ -986,7 +1152,7 @@ __device__ inline FinArgs batch_fin_args(const BatchChan& bc) {
 // stop after P (stored in the channel's P slot) for the batched DFT; the
 // products kernel finishes the channel.  A programmatic dependent of the
 // fold: it waits for the fold's bins and indices before reading any state.
-__global__ void __launch_bounds__(kClusterThreads, 1) batch_fin_kernel(BatchChan* ch, const int* list, int split) {
+__global__ void __launch_bounds__(kClusterThreads, 2) batch_fin_kernel(BatchChan* ch, const int* list, int split) {
     namespace cg = cooperative_groups;
     allow_dependents();
     grid_dependency_wait();
@@ -1067,11 +1233,17 @@ __global__ void fin_dft_kernel(FinArgs a) {
     }
 }
 
-__global__ void init_twiddles_kernel(double2* tw, int64_t L, float2* twN, int64_t N, int64_t sc) {
+// exactly one of tw (float32 bins) and twi (integer bins) is given
+__global__ void init_twiddles_kernel(double2* tw, int4* twi, int64_t L, float2* twN, int64_t N, int64_t sc) {
     for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < L; m += (int64_t)gridDim.x * blockDim.x) {
         double s, c;
         sincospi(2.0 * (double)m / (double)L, &s, &c);
-        tw[m] = make_double2(c, -s);
+        if (twi) {
+            const int2 re = rotator_fixed(c), im = rotator_fixed(-s);
+            twi[m] = make_int4(re.x, re.y, im.x, im.y);
+        } else {
+            tw[m] = make_double2(c, -s);
+        }
         if (m % sc == 0 && m / sc < N) twN[m / sc] = make_float2((float)c, (float)-s);
     }
 }
@@ -1094,13 +1266,18 @@ cudaError_t launch_pdl(void (*k)(Args...), int grid, int block, size_t smem, cud
 
 }  // namespace
 
-cudaError_t launch_init_twiddles(pcal_plan* p, cudaStream_t s) {
-    int64_t L = p->g.L;
-    int g = (int)((L + 255) / 256);
-    if (g > p->num_sms * 8) g = p->num_sms * 8;
-    init_twiddles_kernel<<<g, 256, 0, s>>>(p->d_tw, L, p->d_twN, p->g.N, p->g.step_comb);
-    p->stats.kernel_launches += 1;
+cudaError_t launch_rotators(bool fixed, void* tw, int64_t L, float2* twN, int64_t N, int64_t step_comb,
+                            cudaStream_t s) {
+    int64_t g = (L + 255) / 256;
+    if (g > 1024) g = 1024;
+    init_twiddles_kernel<<<(unsigned)g, 256, 0, s>>>(fixed ? nullptr : static_cast<double2*>(tw),
+                                                     fixed ? static_cast<int4*>(tw) : nullptr, L, twN, N, step_comb);
     return cudaGetLastError();
+}
+
+cudaError_t launch_init_twiddles(pcal_plan* p, cudaStream_t s) {
+    p->stats.kernel_launches += 1;
+    return launch_rotators(p->g.format != PCAL_F32, p->d_tw, p->g.L, p->d_twN, p->g.N, p->g.step_comb, s);
 }
 
 namespace {
@@ -1158,8 +1335,13 @@ int cluster_size_for_device() {
     std::lock_guard<std::mutex> lock(mu);
     if (known[dev]) return cached[dev];
     int best = 0;
-    for (auto k : {fin_cluster_kernel<PCAL_2BIT>, fin_cluster_kernel<PCAL_I8>, fin_cluster_kernel<PCAL_F32>})
+    for (auto k : {fin_cluster_kernel<PCAL_2BIT>, fin_cluster_kernel<PCAL_I8>, fin_cluster_kernel<PCAL_F32>,
+                   fin_cluster_kernel<PCAL_2BIT, true>, fin_cluster_kernel<PCAL_I8, true>})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            (void)cudaGetLastError();
+    for (auto k : {fin_cluster_kernel<PCAL_2BIT, true>, fin_cluster_kernel<PCAL_I8, true>})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(large_smem_bytes(kClusterBigN) + kClusterPadSmem)) != cudaSuccess)
             (void)cudaGetLastError();
     for (int c : {16, 8}) {
         cudaLaunchConfig_t cfg = {};
@@ -1189,11 +1371,11 @@ int cluster_size_for_device() {
 // none of them fits on an SM beside a CTA of the fold that overlaps it (about
 // 205 KB each): sharing an SM with a fold CTA slowed the finalize 2-3x.  The
 // fold leaves kFinalizeReserveSms SMs for it.
-cudaError_t launch_cluster_finalize(const FinArgs& a, int C, cudaStream_t s) {
+cudaError_t launch_cluster_finalize(const FinArgs& a, int C, bool large, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C);
     cfg.blockDim = dim3(kClusterThreads);
-    cfg.dynamicSmemBytes = cluster_smem_bytes(a.N) + kClusterPadSmem;
+    cfg.dynamicSmemBytes = (large ? large_smem_bytes(a.N) : cluster_smem_bytes(a.N)) + kClusterPadSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1204,6 +1386,9 @@ cudaError_t launch_cluster_finalize(const FinArgs& a, int C, cudaStream_t s) {
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
+    if (large)
+        return a.fmt == PCAL_2BIT ? cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT, true>, a)
+                                  : cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8, true>, a);
     if (a.fmt == PCAL_2BIT) return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT>, a);
     if (a.fmt == PCAL_I8) return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8>, a);
     return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_F32>, a);
@@ -1336,6 +1521,12 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
     a.c_l = lv[1] - lv[0];
     a.c_h = lv[2] - lv[0];
     a.c_hl = lv[3] - lv[2] - lv[1] + lv[0];
+    const double k_c = 0.5 * (lv[1] + lv[2]), k_a = k_c - lv[0], k_b = 0.5 * (lv[2] - lv[1]);
+    a.exact = exact_bins(g.format, a.q, k_a, k_b, k_c, a.c_hl);
+    a.k_a = split_df(k_a);
+    a.k_b = split_df(k_b);
+    a.k_c = split_df(k_c);
+    a.k_h = split_df(a.c_hl);
     a.acc2 = cur_acc2(p);
     a.wide2 = cur_wide2(p);
     a.acc8 = cur_acc8(p);
@@ -1349,7 +1540,10 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
         a.n_pf = p->n_pending;
         a.pf_cols = g.row_samples / g.samples_per_byte_x4;
     }
-    a.tw = p->d_tw;
+    if (g.format == PCAL_F32)
+        a.tw = static_cast<const double2*>(p->d_tw);
+    else
+        a.twi = static_cast<const int4*>(p->d_tw);
     a.twN = p->d_twN;
     a.P = reinterpret_cast<float4*>(p->d_P);
     a.T = reinterpret_cast<float2*>(p->d_T);
@@ -1358,11 +1552,15 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
     a.ticket = p->d_ticket;
     cudaError_t e = cudaErrorUnknown;
     bool done = false;
-    if (g.N <= kClusterMaxN && g.L <= kClusterMaxL) {
+    // One cluster for every integer plan of up to kClusterBigN tones, and for
+    // float32 bins (FP64 rotation: two operations per SM and clock) of short
+    // periods only; the others spread over the SMs.
+    const bool small = g.N <= kClusterMaxN && g.L <= kClusterMaxL;
+    if (small || (g.format != PCAL_F32 && g.N <= kClusterBigN)) {
         const int C = cluster_size_for_device();
         if (C > 0) {
             p->stats.kernel_launches += 1;
-            e = launch_cluster_finalize(a, C, s);
+            e = launch_cluster_finalize(a, C, !small, s);
             done = true;
         }
     }

@@ -108,7 +108,7 @@ struct pcal_plan {
     PartSlot pending[kPartSlots]; // slots written by folds and not yet added into the bins
     int n_pending;
     int part_next;                // slot of the next float32 fold
-    double2* d_tw;                // exp(-j 2 pi m / L), m < L
+    void* d_tw;                   // exp(-j 2 pi m / L), m < L: double2 (float32), fixed-point int4 (integer bins)
     float2* d_twN;                // exp(-j 2 pi m / N), m < N (FP32)
     double2* d_P;                 // folded rotated bins P[b], b < N (scratch)
     double2* d_T;                 // tone phasors (scratch before products)
@@ -144,6 +144,10 @@ inline float2* cur_accf(const pcal_plan* p) { return p->d_accf + p->cur * p->g.L
 
 // ---- launchers (return a cudaError_t of the launch) -------------------------
 cudaError_t launch_init_twiddles(pcal_plan* p, cudaStream_t s);
+// exp(-j 2 pi m / L), m < L, into tw (16 bytes each: fixed point or double2) and its every
+// step_comb-th entry, N of them, into twN.
+cudaError_t launch_rotators(bool fixed, void* tw, int64_t L, float2* twN, int64_t N, int64_t step_comb,
+                            cudaStream_t s);
 cudaError_t launch_ragged(pcal_plan* p, const uint8_t* d_bytes, int64_t n_samples, int64_t k0, cudaStream_t s);
 cudaError_t launch_spill2(pcal_plan* p, cudaStream_t s);
 cudaError_t launch_export_bins(pcal_plan* p, void* d_out, cudaStream_t s);
@@ -175,13 +179,13 @@ struct BatchChan {
     int col_width;        // words per column group (the TMA box width)
     int col_groups;
     int64_t row_samples;  // samples per bulk row (a multiple of L)
-    unsigned long long* zero2;  // 2-bit: L zero words (the packed fields of the single-plan layout)
     unsigned long long* wide2;  // 2-bit: [3][L] sums of l, h and (h AND l)
     long long* acc8;            // int8: [L] sums
-    const double2* tw;          // exp(-j 2 pi m / L), m < L
+    const int4* twi;            // exp(-j 2 pi m / L), m < L, in fixed point
     const float2* twN;          // exp(-j 2 pi m / N), m < N
     double* res;                // 5N+3 results, then N+2 post-processing values
     double lev0, c_l, c_h, c_hl;
+    double k_a, k_b, k_c;       // weights of the integer decode (finalize.cu: residue_int)
     double two_pi_fc;
     double fs;
     long long n_abs;            // samples accumulated since creation
