@@ -1141,6 +1141,7 @@ void batch_fill_chan(BatchChan& C, const pcal_geometry& g, double f_comb, const 
     C.spw = g.samples_per_byte_x4;
     C.N = (int)g.N;
     C.L = (int)g.L;
+    C.rcp_L = ~0ull / (unsigned long long)g.L;
     C.so = g.step_offset;
     C.row_samples = g.row_samples;
     C.cols_total = (int)(g.row_samples / C.spw);

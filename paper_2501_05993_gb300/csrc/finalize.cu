@@ -44,6 +44,8 @@ using pcal_df::df;
 
 constexpr int kDftInFoldMaxN = 256;
 constexpr int kDftTonesPerCta = 32;
+enum { kFew, kMany, kLarge, kAny };  // kinds of cluster finalize (cluster_finalize)
+constexpr int kFewN = 64;
 constexpr int kFmtRotated = 16;  // cluster finalize of bins that are rotated already
 
 struct FinArgs {
@@ -52,6 +54,7 @@ struct FinArgs {
     int bc;   // residues b per fold CTA
     int tpb;  // threads per residue (power of two)
     int64_t L, N, so;
+    unsigned long long rcp_L;  // floor((2^64 - 1) / L)
     int64_t q, rem, a0;  // samples in bin k: q + ((k - a0) mod L < rem)
     double lev0, c_l, c_h, c_hl;
     int exact;             // integer bins small enough for residue_int
@@ -71,8 +74,8 @@ struct FinArgs {
     int64_t pf_cols;
     const long long* counts4;  // no-allocation entry: the caller's counts [L][4]
     double lev[4];             // no-allocation entry: the code levels
-    const double2* tw;     // float32 bins: exp(-j 2 pi m/L)
-    const int4* twi;       // integer bins: the same in fixed point (rotator_fixed)
+    const double2* tw;     // exp(-j 2 pi m/L), or
+    const int4* twi;       // (kLarge plans, batches) the same in fixed point (rotator_fixed)
     const float2* twN;
     float4* P;     // P[b] as df re (x, y), df im (z, w)
     float2* T;     // FP32 tone phasors
@@ -83,6 +86,16 @@ struct FinArgs {
     double fs_hz;
     unsigned int* ticket;
 };
+
+// x mod L for 0 <= x < 2^40 (a 64-bit remainder is a subroutine of a hundred
+// instructions, and a finalize of few bins waited for three of them).
+__host__ __device__ inline unsigned long long reciprocal(int64_t L) { return ~0ull / (unsigned long long)L; }
+__device__ __forceinline__ int mod_L(const FinArgs& a, int64_t x) {
+    const unsigned int L = (unsigned int)a.L;
+    const unsigned int q = (unsigned int)__umul64hi((unsigned long long)x, a.rcp_L);  // the quotient or one less
+    const unsigned int r = (unsigned int)x - q * L;
+    return (int)(r >= L ? r - L : r);
+}
 
 // Decode bin k to its real value S[k] (FP64).  NoAlloc: the caller's
 // per-(bin, code) counts.
@@ -118,7 +131,7 @@ __device__ __forceinline__ double read_bin(const FinArgs& a, int64_t k) {
     df s{v.x, v.y};
     for (int e = 0; e < a.n_pf; ++e) {
         const int64_t R = a.pf_rg[e], stride = a.pf_cols;
-        for (int64_t c = ((k - a.pf_ka[e]) % a.L + a.L) % a.L; c < a.pf_cols; c += a.L) {
+        for (int64_t c = k >= a.pf_ka[e] ? k - a.pf_ka[e] : k - a.pf_ka[e] + a.L; c < a.pf_cols; c += a.L) {
             const float2* col = a.pf[e] + c;
             int64_t rg = 0;
             // eight loads in flight, then their additions in row-group order
@@ -566,6 +579,73 @@ __device__ __forceinline__ df warp_exclusive_scan_df(df v) {
     return lane == 0 ? df{0.f, 0.f} : prev;
 }
 
+// Threads per block sum of the products: the order of every sum over tones is
+// set by the lanes' contiguous chunks.  WARP order (short periods, batches,
+// long-period plans): 32 lanes; BLOCK order (LARGE plans): about 8 tones a lane.
+__host__ __device__ inline int product_lanes(int N, bool block_order) {
+    if (!block_order) return 32;
+    const int nt = ((N + 7) / 8 + 31) / 32 * 32;
+    return nt < kClusterThreads / 2 ? nt : kClusterThreads / 2;
+}
+
+// Per-tone arrays of the products are kept by (place in the chunk, lane), one
+// word of padding a row: lanes that walk their chunks together and threads
+// that take consecutive tones both spread over the banks.  (Lanes 32 tones
+// apart in plain arrays met in one bank: 57 us for 1024 tones.)
+struct ToneIndex {
+    int chunk, pitch;
+    __device__ __forceinline__ int operator()(int i) const {
+        const int l = i / chunk;
+        return (i - l * chunk) * pitch + l;
+    }
+};
+__host__ __device__ inline int tone_slots(int N) { return N + N / 32 + 144; }  // at least chunk * (lanes + 1)
+
+// Dynamic shared memory of the cluster finalize for N tones.  The partials and
+// the DFT's twiddles share their memory with the products that follow.
+struct ClusterSmem {
+    float2* sP;   // [N] P
+    float2* sT;   // [N] tone phasors
+    float4* Pr;   // [N] this CTA's partial P (df re, df im)
+    float2* sTw;  // [N rounded up to 16] DFT twiddles, swizzled (tw_slot)
+};
+
+// ... and of the products in the place of Pr and sTw.
+struct ProductsArea {
+    float2* un;    // [4][tone_slots]: unwrapped phase (df), then three arrays of terms of sums over tones (df)
+    float* psi;    // [tone_slots]
+    float* w;      // [tone_slots]
+    float2* red;   // [8 warps][3] partial sums
+    int slots;
+    __device__ __forceinline__ float2* term(int j) const { return un + (j + 1) * slots; }
+};
+
+__host__ __device__ inline size_t cluster_smem_bytes(int64_t N) {
+    const size_t both = (size_t)N * 16, parts = (size_t)N * 16 + (size_t)(N + 15) / 16 * 16 * 8,
+                 prod = (size_t)tone_slots((int)N) * 40 + 8 * 26;
+    return both + (parts > prod ? parts : prod) + 16;
+}
+
+__device__ inline ClusterSmem cluster_layout(uint8_t* base, int64_t N) {
+    ClusterSmem m;
+    m.sP = reinterpret_cast<float2*>(base);
+    m.sT = m.sP + N;
+    uint8_t* q = base + 16 * N;
+    m.Pr = reinterpret_cast<float4*>(q);
+    m.sTw = reinterpret_cast<float2*>(q + 16 * N);
+    return m;
+}
+
+__device__ inline ProductsArea products_area(uint8_t* base, int N) {
+    ProductsArea m;
+    m.slots = tone_slots(N);
+    m.un = reinterpret_cast<float2*>(base + 16 * (size_t)N);
+    m.psi = reinterpret_cast<float*>(m.un + 4 * m.slots);
+    m.w = m.psi + m.slots;
+    m.red = reinterpret_cast<float2*>(m.w + m.slots);
+    return m;
+}
+
 // K df sums over the 32 lanes by a fixed butterfly; every lane gets them.
 // The steps are a loop, not unrolled: this code runs once per finalize, so
 // its size (instruction fetch) costs more than its loop overhead.
@@ -575,41 +655,6 @@ __device__ __forceinline__ void warp_sums_df(df (&v)[K]) {
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
         for (int j = 0; j < K; ++j) v[j] = pcal_df::add(v[j], shfl_xor_df(v[j], o));
-}
-
-// Shared memory of tone_products_warp: per tone the phase, the weight and
-// the unwrapped phase (df).
-struct WarpProductsSmem {
-    float2* un;   // [N] unwrapped phase (df)
-    float2* out;  // [2] td, sigma (df)
-    float* psi;   // [N]
-    float* w;     // [N]
-};
-
-// Dynamic shared memory of the cluster finalize for N tones.
-struct ClusterSmem {
-    float4* Pr;   // [N] this CTA's partial P (df re, df im)
-    float2* sP;   // [N] P
-    float2* sTw;  // [N] DFT twiddles
-    float2* sT;   // [N] tone phasors
-    WarpProductsSmem pm;
-};
-
-__host__ __device__ inline size_t cluster_smem_bytes(int64_t N) { return (size_t)N * 56 + 16; }
-// ... and of its LARGE form, the block's products behind it.
-__host__ __device__ inline size_t large_smem_bytes(int64_t N) { return cluster_smem_bytes(N) + products_bytes(N); }
-
-__device__ inline ClusterSmem cluster_layout(uint8_t* base, int64_t N) {
-    ClusterSmem m;
-    m.Pr = reinterpret_cast<float4*>(base);
-    m.sP = reinterpret_cast<float2*>(base + 16 * N);
-    m.sTw = m.sP + N;
-    m.sT = m.sTw + N;
-    m.pm.un = m.sT + N;
-    m.pm.out = m.pm.un + N;
-    m.pm.psi = reinterpret_cast<float*>(m.pm.out + 2);
-    m.pm.w = m.pm.psi + N;
-    return m;
 }
 
 // The products of tone_products, by one warp with no block barrier: lane l
@@ -702,7 +747,7 @@ __device__ __noinline__ void tone_products_warp(const FinArgs& a, const float2* 
 }
 
 // The FP64 result vector from the products in shared memory, by the block.
-__device__ void write_results_block(const FinArgs& a, const float2* sT, const WarpProductsSmem& m) {
+__device__ void write_results_block(const FinArgs& a, const float2* sT, const ProductsArea& m) {
     const int N = (int)a.N;
     double* amp = a.res + 2 * N;
     double* ph = a.res + 3 * N;
@@ -716,8 +761,198 @@ __device__ void write_results_block(const FinArgs& a, const float2* sT, const Wa
         unw[i] = (double)m.un[i].x + (double)m.un[i].y;
     }
     if (threadIdx.x == 0) {
-        a.res[5 * N] = (double)m.out[0].x + (double)m.out[0].y;
-        a.res[5 * N + 1] = (double)m.out[1].x + (double)m.out[1].y;
+        a.res[5 * N] = (double)m.red[0].x + (double)m.red[0].y;
+        a.res[5 * N + 1] = (double)m.red[1].x + (double)m.red[1].y;
+        a.res[5 * N + 2] = a.M;
+    }
+}
+
+// Amplitude, phase, unwrapped phase, the weighted LS delay fit over all N
+// tones, the post-processing and the FP64 result vector, by one block of
+// kClusterThreads from T and P in shared memory.  Everything that belongs to
+// one tone is done by all threads; only the sums over tones run lane by lane in
+// their fixed order (add_f and add chains of ceil(N/lanes) steps and a
+// butterfly), the three sums of a fit side by side in different warps.  For
+// more than kWarpProductsN tones: with fewer its barriers and its size cost
+// more than the one-warp form takes (64 tones: 6.3 against 4 us).
+constexpr int kWarpProductsN = 128;
+
+template <bool BLOCK_ORDER>
+__device__ __noinline__ void tone_products_all(const FinArgs& a, uint8_t* base) {
+    const int N = (int)a.N, t = threadIdx.x, T = (int)blockDim.x;
+    const float2* sP = reinterpret_cast<const float2*>(base);
+    const float2* sT = sP + N;
+    const ProductsArea m = products_area(base, N);
+    const int nt = product_lanes(N, BLOCK_ORDER), nw = BLOCK_ORDER ? nt / 32 : 1;
+    const int chunk = (N + nt - 1) / nt;
+    const ToneIndex ix{chunk, nt + 1};
+    const int grp = t / nt, lt = t - grp * nt, G = T / nt;  // groups of nt threads
+    const int lane = t & 31, gw = lt >> 5;
+    const int n_mine = lt * chunk < N ? (N - lt * chunk < chunk ? N - lt * chunk : chunk) : 0;  // tones of this lane
+    // 1. phase and weight per tone, FP32
+#pragma unroll 1
+    for (int i = t; i < N; i += T) {
+        const float2 z = sT[i];
+        const int q = ix(i);
+        m.psi[q] = wrap_pi_f(atan2f(z.y, z.x) + 1.5707963267948966f);
+        m.w[q] = z.x * z.x + z.y * z.y;
+    }
+    __syncthreads();
+    float* step = reinterpret_cast<float*>(m.term(0));  // wrapped phase steps
+#pragma unroll 1
+    for (int i = t; i < N; i += T) step[ix(i)] = i > 0 ? wrap_pi_f(m.psi[ix(i)] - m.psi[ix(i - 1)]) : 0.f;
+    __syncthreads();
+    // 2. unwrap: u_i = psi_0 + sum_{j=1..i} wrap(psi_j - psi_{j-1}), df sums
+    df local{0.f, 0.f};
+    const int skip = lt == 0 ? 1 : 0;  // tone 0 has no step
+    if (grp == 0) {
+#pragma unroll 4
+        for (int j = skip; j < n_mine; ++j) local = pcal_df::add_f(local, step[j * ix.pitch + lt]);
+    } else if (t >= T - 32) {
+        if (a.extra) peak_delay_warp(a, sP);
+    }
+    df before;
+    if constexpr (BLOCK_ORDER) {
+        df inc = local;
+#pragma unroll 1
+        for (int o = 1; o < 32; o <<= 1) {
+            const df u{__shfl_up_sync(0xffffffffu, inc.hi, o), __shfl_up_sync(0xffffffffu, inc.lo, o)};
+            if (lane >= o) inc = pcal_df::add(inc, u);
+        }
+        if (grp == 0 && lane == 31) m.red[gw] = make_float2(inc.hi, inc.lo);
+        __syncthreads();
+        before = df{0.f, 0.f};
+        for (int w = 0; w < gw; ++w) before = pcal_df::add(before, df{m.red[w].x, m.red[w].y});
+        before = pcal_df::sub(pcal_df::add(before, inc), local);
+    } else {
+        before = warp_exclusive_scan_df(local);
+    }
+    if (grp == 0) {
+        df run = pcal_df::add_f(before, m.psi[0]);
+#pragma unroll 4
+        for (int j = 0; j < n_mine; ++j) {
+            if (j >= skip) run = pcal_df::add_f(run, step[j * ix.pitch + lt]);
+            m.un[j * ix.pitch + lt] = make_float2(run.hi, run.lo);
+        }
+    }
+    __syncthreads();
+    // Sum `j` of three by group j % G: red[warp * 3 + j], then everybody adds the warps in order.
+    auto three_sums = [&](auto&& chain, df (&out)[3]) {
+#pragma unroll 1
+        for (int j = grp; j < 3; j += G) {
+            df v = chain(j);
+#pragma unroll 1
+            for (int o = 16; o > 0; o >>= 1) v = pcal_df::add(v, shfl_xor_df(v, o));
+            if (lane == 0) m.red[gw * 3 + j] = make_float2(v.hi, v.lo);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            if (nw == 1) {
+                out[j] = df{m.red[j].x, m.red[j].y};
+            } else {
+                df v{0.f, 0.f};
+                for (int w = 0; w < nw; ++w) v = pcal_df::add(v, df{m.red[w * 3 + j].x, m.red[w * 3 + j].y});
+                out[j] = v;
+            }
+        }
+        __syncthreads();
+    };
+    // 3. weighted least squares of u_i against the tone index x_i = i (the
+    //    frequency is f_i = f_comb*i + f_offset), weights w_i = |T_i|^2
+#pragma unroll 1
+    for (int i = t; i < N; i += T) {
+        const int q = ix(i);
+        const df v = pcal_df::mul_f(df{m.un[q].x, m.un[q].y}, m.w[q]);
+        m.term(2)[q] = make_float2(v.hi, v.lo);
+    }
+    __syncthreads();
+    df s3[3], s2[3];
+    three_sums(
+        [&](int j) {
+            df v{0.f, 0.f};
+            if (j == 0) {
+#pragma unroll 4
+                for (int k = 0; k < n_mine; ++k) v = pcal_df::add_f(v, m.w[k * ix.pitch + lt]);
+            } else if (j == 1) {
+#pragma unroll 4
+                for (int k = 0; k < n_mine; ++k)
+                    v = pcal_df::add(v, pcal_df::two_prod(m.w[k * ix.pitch + lt], (float)(lt * chunk + k)));
+            } else {
+#pragma unroll 4
+                for (int k = 0; k < n_mine; ++k) {
+                    const float2 u = m.term(2)[k * ix.pitch + lt];
+                    v = pcal_df::add(v, df{u.x, u.y});
+                }
+            }
+            return v;
+        },
+        s3);
+    const df W = s3[0];
+    df td{__int_as_float(0x7fc00000), 0.f}, sig{__int_as_float(0x7fc00000), 0.f};  // NaN until fitted
+    df xbar{0.f, 0.f}, ubar{0.f, 0.f}, slope{0.f, 0.f};
+    bool fitted = false;
+    if (N >= 2 && W.hi > 0.f) {
+        xbar = pcal_df::div(s3[1], W);
+        ubar = pcal_df::div(s3[2], W);
+        // centred sums; the residual sum follows from Syy - slope*Sxu
+#pragma unroll 1
+        for (int i = t; i < N; i += T) {
+            const int q = ix(i);
+            const float w = m.w[q];
+            const df dx = pcal_df::sub(df{(float)i, 0.f}, xbar);
+            const df du = pcal_df::sub(df{m.un[q].x, m.un[q].y}, ubar);
+            const df wdx = pcal_df::mul_f(dx, w);
+            const df xx = pcal_df::mul(wdx, dx), xu = pcal_df::mul(wdx, du),
+                     uu = pcal_df::mul_f(pcal_df::mul(du, du), w);
+            m.term(0)[q] = make_float2(xx.hi, xx.lo);
+            m.term(1)[q] = make_float2(xu.hi, xu.lo);
+            m.term(2)[q] = make_float2(uu.hi, uu.lo);
+        }
+        __syncthreads();
+        three_sums(
+            [&](int j) {
+                df v{0.f, 0.f};
+#pragma unroll 4
+                for (int k = 0; k < n_mine; ++k) {
+                    const float2 u = m.term(j)[k * ix.pitch + lt];
+                    v = pcal_df::add(v, df{u.x, u.y});
+                }
+                return v;
+            },
+            s2);
+        if (s2[0].hi > 0.f) {
+            slope = pcal_df::div(s2[1], s2[0]);  // rad per tone index
+            fitted = true;
+            td = pcal_df::div(slope, a.two_pi_fc);
+            if (N > 2) {
+                df ssr = pcal_df::sub(s2[2], pcal_df::mul(slope, s2[1]));
+                if (ssr.hi < 0.f) ssr = df{0.f, 0.f};
+                sig = pcal_df::div(pcal_df::sqrt_df(pcal_df::div(ssr, pcal_df::mul_f(s2[0], (float)(N - 2)))),
+                                   a.two_pi_fc);
+            }
+        }
+    }
+    // 4. FP64 results and the bandpass phase with the fitted delay removed,
+    //    u_i - ubar - slope*(i - xbar)
+#pragma unroll 1
+    for (int i = t; i < N; i += T) {
+        const int q = ix(i);
+        const float2 z = sT[i], u = m.un[q];
+        a.res[2 * i] = (double)z.x;
+        a.res[2 * i + 1] = (double)z.y;
+        a.res[2 * N + i] = (double)(sqrtf(m.w[q]) * a.two_over_m);
+        a.res[3 * N + i] = (double)m.psi[q];
+        a.res[4 * N + i] = (double)u.x + (double)u.y;
+        if (a.extra) {
+            const df r = pcal_df::sub(pcal_df::sub(df{u.x, u.y}, ubar),
+                                      pcal_df::mul(slope, pcal_df::sub(df{(float)i, 0.f}, xbar)));
+            a.extra[2 + i] = fitted ? (double)r.hi + (double)r.lo : __longlong_as_double(0x7ff8000000000000ll);
+        }
+    }
+    if (t == 0) {
+        a.res[5 * N] = (double)td.hi + (double)td.lo;
+        a.res[5 * N + 1] = (double)sig.hi + (double)sig.lo;
         a.res[5 * N + 2] = a.M;
     }
 }
@@ -730,19 +965,42 @@ __device__ __forceinline__ double2 fold_residue(const FinArgs& a, int b, int m, 
     if (m >= m_end) return make_double2(0.0, 0.0);
     const int L = (int)a.L, N = (int)a.N;
     int k = b + m * N;
-    int idx = (int)((a.so * k) % L);  // rotator index (f_offset/g * k) mod L
+    int idx = mod_L(a, a.so * k);  // rotator index (f_offset/g * k) mod L
     const int kstep = step * N;
-    const int istep = (int)((a.so * kstep) % L);
+    const int istep = mod_L(a, a.so * kstep);
+    if (FMT == PCAL_2BIT && !a.spilled && !a.twi) {
+        // S = lev0*cnt + c_l*sum(l) + c_h*sum(h) + c_hl*sum(h AND l),
+        // cnt = q or q + 1; the fields are below 2^21
+        const double s_q = a.lev0 * (double)a.q, s_q1 = a.lev0 * (double)(a.q + 1);
+        const int a0 = (int)a.a0, rem = (int)a.rem;
+#pragma unroll 2
+        for (; m < m_end; m += step) {
+            const unsigned long long v = a.acc2[k];
+            const double2 w = a.tw[idx];
+            a.acc2[k] = 0;
+            int rr = k - a0;
+            if (rr < 0) rr += L;
+            const double S = fma(a.c_hl, (double)(int)((v >> 42) & PCAL_F21_MASK),
+                                 fma(a.c_h, (double)(int)((v >> 21) & PCAL_F21_MASK),
+                                     fma(a.c_l, (double)(int)(v & PCAL_F21_MASK), rr < rem ? s_q1 : s_q)));
+            re = fma(S, w.x, re);
+            im = fma(S, w.y, im);
+            k += kstep;
+            idx += istep;
+            if (idx >= L) idx -= L;
+        }
+    } else {
 #pragma unroll 1
-    for (; m < m_end; m += step) {
-        const double S = read_bin<false, FMT>(a, k);
-        const double2 w = rotator<false>(a, idx);
-        re = fma(S, w.x, re);
-        im = fma(S, w.y, im);
-        clear_bin<FMT>(a, k);
-        k += kstep;
-        idx += istep;
-        if (idx >= L) idx -= L;
+        for (; m < m_end; m += step) {
+            const double S = read_bin<false, FMT>(a, k);
+            const double2 w = rotator<false>(a, idx);
+            re = fma(S, w.x, re);
+            im = fma(S, w.y, im);
+            clear_bin<FMT>(a, k);
+            k += kstep;
+            idx += istep;
+            if (idx >= L) idx -= L;
+        }
     }
     return make_double2(re, im);
 }
@@ -791,72 +1049,81 @@ __device__ __forceinline__ void add_scaled(df& re, df& im, const IntSum& s, df k
 // 14.5 -> 13.1 us; wide plans (LARGE below) 35 us in two kernels over all SMs
 // after the fold -> one cluster beside the next fold (1024 tones: 91 -> 79 us a
 // step).
-template <int FMT>
+// SRC: 0 packed 2-bit words (or int8 sums), 1 packed and spilled, 2 the wide
+// arrays alone.  U: bins whose loads are in flight together (from clamped
+// addresses past the end: a load behind a branch waited for the one before it,
+// 3.5 us for eight).
+template <int FMT, int SRC, int U>
 __device__ __forceinline__ float4 residue_int(const FinArgs& a, int b, int m, int step, int m_end) {
-    const int fmt = FMT < 0 ? a.fmt : FMT;
     df re{0.f, 0.f}, im{0.f, 0.f};
     if (m >= m_end) return make_float4(0.f, 0.f, 0.f, 0.f);
     const int L = (int)a.L, N = (int)a.N;
+    // bin k = b + m N turns by so k mod L: by so N m here, which the lanes of a
+    // warp mostly share (their loads of the table are one), and by so b at the end
     int k = b + m * N;
-    int idx = (int)((a.so * k) % L);  // rotator index (f_offset/g * k) mod L
     const int kstep = step * N;
-    const int istep = (int)((a.so * kstep) % L);
+    const int4* __restrict__ twi = a.twi;
+    int idx = mod_L(a, a.so * ((int64_t)m * N));
+    const int istep = mod_L(a, a.so * kstep);
     const int q = (int)a.q, a0 = (int)a.a0, rem = (int)a.rem;
     const bool use_c = a.k_c.hi != 0.f, use_h = a.k_h.hi != 0.f;
-    constexpr int U = 4;  // bins in flight
     while (m < m_end) {
         const int end = (m_end - m) / step >= 512 ? m + 512 * step : m_end;  // (512: a multiple of U)
         IntSum A, B, Cn, H;
+#pragma unroll 1
         while (m < end) {
             int4 w[U];
-            int x[U], y[U], z[U], cnt[U];
-            int kk = k;
+            unsigned long long v[U], wl[U], wh[U], wb[U];
+            int at[U];
+            bool in[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const bool in = m + u * step < end;
-                w[u] = make_int4(0, 0, 0, 0);
-                x[u] = y[u] = z[u] = cnt[u] = 0;
-                if (in) {
-                    w[u] = a.twi[idx];
-                    if (fmt == PCAL_2BIT) {
-                        if (a.spilled != 2) {
-                            const unsigned long long v = a.acc2[kk];
-                            x[u] = (int)(v & PCAL_F21_MASK);
-                            y[u] = (int)((v >> 21) & PCAL_F21_MASK);
-                            z[u] = (int)((v >> 42) & PCAL_F21_MASK);
-                        }
-                        if (a.spilled) {
-                            x[u] += (int)a.wide2[kk];
-                            y[u] += (int)a.wide2[L + kk];
-                            if (use_h) z[u] += (int)a.wide2[2 * L + kk];
-                        }
-                        int rr = kk - a0;
-                        if (rr < 0) rr += L;
-                        cnt[u] = q + (rr < rem ? 1 : 0);
-                    } else {
-                        x[u] = (int)a.acc8[kk];
-                    }
+                in[u] = m + u * step < end;
+                at[u] = in[u] ? k + u * kstep : k;
+                w[u] = __ldg(twi + idx);
+                if (FMT == PCAL_I8) v[u] = (unsigned long long)a.acc8[at[u]];
+                if (FMT == PCAL_2BIT && SRC != 2) v[u] = a.acc2[at[u]];
+                if (FMT == PCAL_2BIT && SRC != 0) {
+                    wl[u] = a.wide2[at[u]];
+                    wh[u] = a.wide2[L + at[u]];
+                    wb[u] = use_h ? a.wide2[2 * L + at[u]] : 0ull;
                 }
-                kk += kstep;
                 idx += istep;
                 if (idx >= L) idx -= L;
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                if (m + u * step < end) clear_bin<FMT>(a, k);
-                k += kstep;
-                if (fmt == PCAL_2BIT) {
-                    A.add(x[u] + y[u] - cnt[u], w[u]);
-                    B.add(y[u] - x[u], w[u]);
-                    if (use_c) Cn.add(cnt[u], w[u]);
-                    if (use_h) H.add(z[u], w[u]);
+                if (in[u])
+                    clear_bin<FMT>(a, at[u]);
+                else
+                    w[u] = make_int4(0, 0, 0, 0);
+                if (FMT == PCAL_2BIT) {
+                    int x = 0, y = 0, z = 0;
+                    if (SRC != 2) {
+                        x = (int)(v[u] & PCAL_F21_MASK);
+                        y = (int)((v[u] >> 21) & PCAL_F21_MASK);
+                        z = (int)((v[u] >> 42) & PCAL_F21_MASK);
+                    }
+                    if (SRC != 0) {
+                        x += (int)wl[u];
+                        y += (int)wh[u];
+                        z += (int)wb[u];
+                    }
+                    int rr = at[u] - a0;
+                    if (rr < 0) rr += L;
+                    const int cnt = q + (rr < rem ? 1 : 0);
+                    A.add(x + y - cnt, w[u]);
+                    B.add(y - x, w[u]);
+                    if (use_c) Cn.add(cnt, w[u]);
+                    if (use_h) H.add(z, w[u]);
                 } else {
-                    A.add(x[u], w[u]);
+                    A.add((int)v[u], w[u]);
                 }
             }
+            k += U * kstep;
             m += U * step;
         }
-        if (fmt == PCAL_2BIT) {
+        if (FMT == PCAL_2BIT) {
             add_scaled(re, im, A, a.k_a);
             add_scaled(re, im, B, a.k_b);
             if (use_c) add_scaled(re, im, Cn, a.k_c);
@@ -866,7 +1133,11 @@ __device__ __forceinline__ float4 residue_int(const FinArgs& a, int b, int m, in
             im = pcal_df::add(im, int_df(A.ih, A.il));
         }
     }
-    return make_float4(re.hi, re.lo, im.hi, im.lo);
+    const int4 w = __ldg(twi + mod_L(a, a.so * b));
+    const df wr = int_df(w.x, w.y), wi = int_df(w.z, w.w);
+    const df r = pcal_df::sub(pcal_df::mul(re, wr), pcal_df::mul(im, wi));
+    const df i = pcal_df::add(pcal_df::mul(re, wi), pcal_df::mul(im, wr));
+    return make_float4(r.hi, r.lo, i.hi, i.lo);
 }
 
 // Whether a period's integer bins fit residue_int: samples per bin below 2^26
@@ -892,7 +1163,7 @@ __host__ __device__ inline df split_df(double x) {
 // Residue b over m = m, m + step, ... below m_end as double-float (re hi, re
 // lo, im hi, im lo).  kFmtRotated: the bins are rotated complex sums already
 // (the rows of a long-period plan), added in row order.
-template <int FMT>
+template <int FMT, int KIND>
 __device__ __forceinline__ float4 residue_df(const FinArgs& a, int b, int m, int step, int m_end) {
     if constexpr (FMT == kFmtRotated) {
         df re{0.f, 0.f}, im{0.f, 0.f};
@@ -906,48 +1177,138 @@ __device__ __forceinline__ float4 residue_df(const FinArgs& a, int b, int m, int
         }
         return make_float4(re.hi, re.lo, im.hi, im.lo);
     } else {
-        if constexpr (FMT != PCAL_F32)
-            if (a.exact) return residue_int<FMT>(a, b, m, step, m_end);
+        if constexpr (FMT < 0) {  // (two CTAs share an SM: fewer registers)
+            if (a.exact)
+                return a.fmt == PCAL_2BIT ? residue_int<PCAL_2BIT, 2, 4>(a, b, m, step, m_end)
+                                          : residue_int<PCAL_I8, 0, 8>(a, b, m, step, m_end);
+        } else if constexpr (FMT != PCAL_F32 && KIND == kLarge) {
+            if (a.exact)
+                return a.spilled ? residue_int<FMT, 1, 2>(a, b, m, step, m_end)
+                                 : residue_int<FMT, 0, 8>(a, b, m, step, m_end);
+        }
         const double2 z = fold_residue<FMT>(a, b, m, step, m_end);
         const df dre = df_of(z.x), dim = df_of(z.y);
         return make_float4(dre.hi, dre.lo, dim.hi, dim.lo);
     }
 }
 
-// Tones [i0, i1) of the N-point DFT of sP in FP32, written to dst[i] (shared
-// memory of this CTA or, through the cluster, of another).  The threads per
-// tone g, combined by a fixed butterfly, are as many as `share` tones leave
-// for each in the block: they set the order of a tone's FP32 sum.
-__device__ void dft_range(const float2* sP, const float2* sTw, int N, int i0, int i1, float2* dst, int share) {
-    const int t = threadIdx.x;
-    const int ntone = i1 - i0;
+// Slot of DFT twiddle ix in shared memory: the low four bits of its index are
+// mixed with the next eight, so that the strides i of tone i (powers of two
+// among them) spread over the banks.
+__device__ __forceinline__ int tw_slot(int ix) { return ix ^ ((ix >> 4) & 15) ^ ((ix >> 8) & 15); }
+
+// Threads per tone of a DFT that `share` tones split a block for (a power of
+// two, at most 32): they set the order of a tone's FP32 sum (thread gs takes
+// b = gs, gs + g, ...; then a fixed butterfly).
+__host__ __device__ inline int dft_threads(int share) {
     int g = 1;
-    while (g < 32 && g * 2 * share <= (int)blockDim.x) g *= 2;
+    while (g < 32 && g * 2 * share <= kClusterThreads) g *= 2;
+    return g;
+}
+
+// Tones [i0, i1) of the N-point DFT of sP in FP32, g threads each, written to
+// dst[i] (shared memory of this CTA or, through the cluster, of another).
+// PAIRS: i in [i0, i1) of 0 .. N/2, each with the tone N - i, whose twiddles
+// are the conjugates: one lookup serves both.  Eight steps at a time, their
+// twiddle indices from the first one's.
+template <bool PAIRS>
+__device__ __forceinline__ void dft_tones_smem(const float2* sP, const float2* sTw, int N, int i0, int i1, float2* dst,
+                                               int g) {
+    const int t = threadIdx.x;
+    const int n = i1 - i0;
     const int groups = blockDim.x / g;
     const int gs = t % g;
 #pragma unroll 1
-    for (int base = 0; base < ntone; base += groups) {
+    for (int base = 0; base < n; base += groups) {
         const int i = i0 + base + t / g;
-        float sre = 0.f, sim = 0.f;
+        float sre = 0.f, sim = 0.f, cre = 0.f, cim = 0.f;
+        auto add = [&](float2 p, float2 w) {
+            sre = fmaf(p.x, w.x, fmaf(-p.y, w.y, sre));
+            sim = fmaf(p.x, w.y, fmaf(p.y, w.x, sim));
+            if (PAIRS) {
+                cre = fmaf(p.x, w.x, fmaf(p.y, w.y, cre));
+                cim = fmaf(p.x, -w.y, fmaf(p.y, w.x, cim));
+            }
+        };
         if (i < i1) {
-            int ix = (int)(((int64_t)i * gs) % N);
-            const int step = (int)(((int64_t)i * g) % N);
-#pragma unroll 4
-            for (int bb = gs; bb < N; bb += g) {
-                const float2 p = sP[bb];
-                const float2 w = sTw[ix];
-                sre = fmaf(p.x, w.x, fmaf(-p.y, w.y, sre));
-                sim = fmaf(p.x, w.y, fmaf(p.y, w.x, sim));
+            const unsigned int un = (unsigned int)N;
+            unsigned int ix = (unsigned int)(i * gs) % un;  // i, g below 2^11
+            const unsigned int step = (unsigned int)(i * g) % un;
+            int bb = gs;
+            if (bb + 7 * g < N) {
+                unsigned int off[8];  // k steps on
+                off[0] = 0;
+#pragma unroll
+                for (int k = 1; k < 8; ++k) {
+                    off[k] = off[k - 1] + step;
+                    off[k] = min(off[k], off[k] - un);
+                }
+                unsigned int eight = off[7] + step;
+                eight = min(eight, eight - un);
+#pragma unroll 1
+                for (; bb + 7 * g < N; bb += 8 * g) {
+                    float2 p[8], w[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        unsigned int x = ix + off[k];
+                        x = min(x, x - un);
+                        p[k] = sP[bb + k * g];
+                        w[k] = sTw[tw_slot((int)x)];
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) add(p[k], w[k]);
+                    ix += eight;
+                    ix = min(ix, ix - un);
+                }
+            }
+#pragma unroll 1
+            for (; bb < N; bb += g) {
+                add(sP[bb], sTw[tw_slot((int)ix)]);
                 ix += step;
-                if (ix >= N) ix -= N;
+                ix = min(ix, ix - un);
             }
         }
+#pragma unroll 1
         for (int o = g / 2; o > 0; o >>= 1) {
             sre += __shfl_xor_sync(0xffffffffu, sre, o);
             sim += __shfl_xor_sync(0xffffffffu, sim, o);
+            if (PAIRS) {
+                cre += __shfl_xor_sync(0xffffffffu, cre, o);
+                cim += __shfl_xor_sync(0xffffffffu, cim, o);
+            }
         }
-        if (i < i1 && gs == 0) dst[i] = make_float2(sre, sim);
+        if (i < i1 && gs == 0) {
+            dst[i] = make_float2(sre, sim);
+            if (PAIRS && i > 0 && 2 * i != N) dst[N - i] = make_float2(cre, cim);
+        }
     }
+}
+
+// All tones of a DFT of at most kFewN: the same sums in a loop that is short
+// as code (16 steps at most), from twiddles in their plain order.
+__device__ __forceinline__ void dft_few(const float2* sP, const float2* sTw, int N, float2* dst, int g) {
+    const int t = threadIdx.x, gs = t % g, i = t / g;
+    float sre = 0.f, sim = 0.f;
+    if (i < N) {
+        const unsigned int un = (unsigned int)N;
+        unsigned int ix = (unsigned int)(i * gs) % un;
+        const unsigned int step = (unsigned int)(i * g) % un;
+#pragma unroll 4
+        for (int bb = gs; bb < N; bb += g) {
+            const float2 p = sP[bb];
+            const float2 w = sTw[ix];
+            sre = fmaf(p.x, w.x, fmaf(-p.y, w.y, sre));
+            sim = fmaf(p.x, w.y, fmaf(p.y, w.x, sim));
+            ix += step;
+            ix = min(ix, ix - un);
+        }
+    }
+#pragma unroll 1
+    for (int o = g / 2; o > 0; o >>= 1) {
+        sre += __shfl_xor_sync(0xffffffffu, sre, o);
+        sim += __shfl_xor_sync(0xffffffffu, sim, o);
+    }
+    if (i < N && gs == 0) dst[i] = make_float2(sre, sim);
 }
 
 // The whole finalize in one cluster of C CTAs.  Thread t of every CTA takes
@@ -961,11 +1322,18 @@ __device__ void dft_range(const float2* sP, const float2* sTw, int N, int i0, in
 // products.
 // Runs in every CTA of the cluster; returns true in the CTA that wrote the
 // results (rank 0), after it wrote them.
-// LARGE: plans of more than kClusterMaxN tones or of long periods.  Their DFT
-// and products keep the order of operations of fin_dft_kernel and
-// fin_fold_kernel: tones in groups of kDftTonesPerCta (the groups dealt to the
-// CTAs), and the products by the block.
-template <int FMT = -1, bool LARGE = false>
+// KIND: what the kernel has to hold.  A finalize runs once per step and its
+// instructions come from L2, slowly beside a streaming fold, so each kernel
+// leaves out what its plans never use (an integer decode and the wide paths
+// in the one kernel: C2 decode 4.7 -> 11.8 us beside the next fold).
+//   kFew, kMany  plans of at most kFewN, kClusterMaxN tones and short periods:
+//                FP64 decode (1 to 8 bins a thread), one-warp products up to
+//                kWarpProductsN tones
+//   kLarge       the other integer plans: integer decode; their DFT and products
+//                keep the order of fin_dft_kernel and fin_fold_kernel: tones in
+//                groups of kDftTonesPerCta, products in BLOCK order
+//   kAny         batches (integer decode) and long-period plans
+template <int FMT, int KIND>
 __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -978,10 +1346,11 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     float2 *sP = sm.sP, *sTw = sm.sTw, *sT = sm.sT;
     const int t = threadIdx.x;
     // N > blockDim: one lane per residue, the residues in turns
-    const bool big = N > (int)blockDim.x;
+    constexpr bool LARGE = KIND == kLarge;
+    const bool big = KIND >= kLarge && N > (int)blockDim.x;
     const int lanes = big ? 1 : (int)blockDim.x / N;
     if (r == 0 || N > kClusterMaxN)
-        for (int i = t; i < N; i += blockDim.x) sTw[i] = a.twN[i];
+        for (int i = t; i < N; i += blockDim.x) sTw[KIND == kFew ? i : tw_slot(i)] = a.twN[i];
     // L <= PCAL_MAX_L: bin and rotator indices fit 32 bits (so*k does not)
     const int L = (int)a.L;
     const int per = L / N;
@@ -990,7 +1359,7 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
         // thread t: residue t % N, every lanes-th m of this CTA's slice
         const int b = t % N, ml = t / N;
         if (ml < lanes) {
-            part[t] = residue_df<FMT>(a, b, per * r / C + ml, lanes, m1);
+            part[t] = residue_df<FMT, KIND>(a, b, per * r / C + ml, lanes, m1);
         }
         __syncthreads();
         if (t < N) {
@@ -1006,55 +1375,67 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     } else {
         // one thread per residue, the residues in turns
 #pragma unroll 1
-        for (int b = t; b < N; b += blockDim.x) Pr[b] = residue_df<FMT>(a, b, per * r / C, 1, m1);
+        for (int b = t; b < N; b += blockDim.x) Pr[b] = residue_df<FMT, KIND>(a, b, per * r / C, 1, m1);
     }
     cluster.sync();  // every CTA's partial P is complete
-    if (r == 0) {
+    if (big) {
+        // every CTA adds its share of the residues (the C partials in rank order,
+        // loads issued in fours) and hands the sums to all of them
+        for (int i = N * r / C + t; i < N * (r + 1) / C; i += blockDim.x) {
+            df sr{0.f, 0.f}, si{0.f, 0.f};
+#pragma unroll 1
+            for (int q0 = 0; q0 < C; q0 += 4) {
+                float4 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    v[u] = q0 + u < C ? *cluster.map_shared_rank(&Pr[i], q0 + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    sr = pcal_df::add(sr, df{v[u].x, v[u].y});
+                    si = pcal_df::add(si, df{v[u].z, v[u].w});
+                }
+            }
+            const float2 p = make_float2(sr.hi + sr.lo, si.hi + si.lo);
+            for (int q = 0; q < C; ++q) cluster.map_shared_rank(sP, q)[i] = p;
+        }
+    } else if (r == 0) {
         // residue i: the C partials in rank order, loads issued in fours;
         // G threads share a residue when N is small
-        const int G = big ? 1 : (lanes < C ? lanes : C);
-        const int g = big ? 0 : t / N;
+        const int G = lanes < C ? lanes : C;
+        const int g = t / N;
         if (g < G) {
+            const int i = t % N;
+            df sr{0.f, 0.f}, si{0.f, 0.f};
 #pragma unroll 1
-            for (int i = big ? t : t % N; i < N; i += big ? blockDim.x : N) {
-                df sr{0.f, 0.f}, si{0.f, 0.f};
-#pragma unroll 1
-                for (int q0 = g; q0 < C; q0 += 4 * G) {
-                    float4 v[4];
+            for (int q0 = g; q0 < C; q0 += 4 * G) {
+                float4 v[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int q = q0 + u * G;
-                        v[u] = q < C ? *cluster.map_shared_rank(&Pr[i], q) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        sr = pcal_df::add(sr, df{v[u].x, v[u].y});
-                        si = pcal_df::add(si, df{v[u].z, v[u].w});
-                    }
+                for (int u = 0; u < 4; ++u) {
+                    const int q = q0 + u * G;
+                    v[u] = q < C ? *cluster.map_shared_rank(&Pr[i], q) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
-                if (big)
-                    sP[i] = make_float2(sr.hi + sr.lo, si.hi + si.lo);
-                else
-                    part[t] = make_float4(sr.hi, sr.lo, si.hi, si.lo);
-                if (!big) break;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    sr = pcal_df::add(sr, df{v[u].x, v[u].y});
+                    si = pcal_df::add(si, df{v[u].z, v[u].w});
+                }
             }
+            part[t] = make_float4(sr.hi, sr.lo, si.hi, si.lo);
         }
-        if (!big) {
-            __syncthreads();
-            if (t < N) {
-                df sr{0.f, 0.f}, si{0.f, 0.f};
+        __syncthreads();
+        if (t < N) {
+            df sr{0.f, 0.f}, si{0.f, 0.f};
 #pragma unroll 1
-                for (int gg = 0; gg < G; ++gg) {
-                    const float4 v = part[gg * N + t];
-                    sr = pcal_df::add(sr, df{v.x, v.y});
-                    si = pcal_df::add(si, df{v.z, v.w});
-                }
-                sP[t] = make_float2(sr.hi + sr.lo, si.hi + si.lo);
+            for (int gg = 0; gg < G; ++gg) {
+                const float4 v = part[gg * N + t];
+                sr = pcal_df::add(sr, df{v.x, v.y});
+                si = pcal_df::add(si, df{v.z, v.w});
             }
+            sP[t] = make_float2(sr.hi + sr.lo, si.hi + si.lo);
         }
     }
-    cluster.sync();  // P is complete in CTA 0; the other CTAs' Pr is no longer read
-    if (a.Pout) {
+    cluster.sync();  // P is complete (in CTA 0; big: in all); the other CTAs' Pr is no longer read
+    if (KIND == kAny && a.Pout) {
         // the DFT runs elsewhere (the batched tensor-core DFT)
         if (r == 0)
             for (int i = t; i < N; i += blockDim.x) a.Pout[i] = sP[i];
@@ -1062,54 +1443,57 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     }
     if (!big) {
         if (r != 0) return false;
-        dft_range(sP, sTw, N, 0, N, sT, N);
+        if (KIND == kFew)
+            dft_few(sP, sTw, N, sT, dft_threads(N));
+        else
+            dft_tones_smem<true>(sP, sTw, N, 0, N / 2 + 1, sT, dft_threads(N));
     } else {
-        // every CTA: its share of the tones from a copy of P, into CTA 0's sT
-        if (r != 0) {
-            const float2* p0 = cluster.map_shared_rank(sP, 0);
-            for (int i = t; i < N; i += blockDim.x) sP[i] = p0[i];
-        }
-        __syncthreads();
+        // every CTA: its share of the tones, into CTA 0's sT
         float2* dst = cluster.map_shared_rank(sT, 0);
-        if constexpr (LARGE) {
+        // threads per tone: of LARGE groups of kDftTonesPerCta tones, of equal
+        // shares of the tones, or (long-period plans) of one CTA with all of them;
+        // where the last or the larger shares have another count, tone by tone
+        const int least = LARGE ? (N % kDftTonesPerCta ? N % kDftTonesPerCta : kDftTonesPerCta)
+                                : (FMT == kFmtRotated ? N : N / C);
+        const int most = LARGE ? kDftTonesPerCta : (FMT == kFmtRotated ? N : (N + C - 1) / C);
+        if (dft_threads(least) == dft_threads(most)) {
+            const int H = N / 2 + 1;
+            dft_tones_smem<true>(sP, sTw, N, H * r / C, H * (r + 1) / C, dst, dft_threads(most));
+        } else if constexpr (LARGE) {
             for (int i0 = r * kDftTonesPerCta; i0 < N; i0 += C * kDftTonesPerCta) {
                 const int n = N - i0 < kDftTonesPerCta ? N - i0 : kDftTonesPerCta;
-                dft_range(sP, sTw, N, i0, i0 + n, dst, n);
+                dft_tones_smem<false>(sP, sTw, N, i0, i0 + n, dst, dft_threads(n));
             }
         } else {
-            // (long-period plans: in the order of one CTA with all N tones)
             const int i0 = N * r / C, i1 = N * (r + 1) / C;
-            dft_range(sP, sTw, N, i0, i1, dst, FMT == kFmtRotated ? N : i1 - i0);
+            dft_tones_smem<false>(sP, sTw, N, i0, i1, dst, dft_threads(i1 - i0));
         }
-        cluster.sync();  // CTA 0 holds every tone; its sP is no longer read
+        cluster.sync();  // CTA 0 holds every tone
         if (r != 0) return false;
     }
     __syncthreads();
-    if constexpr (LARGE) {
-        const ProductsSmem pm = products_layout(dsm + cluster_smem_bytes(N), N);
-        for (int i = t; i < N; i += blockDim.x) pm.T[i] = sT[i];
+    if (LARGE || (KIND != kFew && N > kWarpProductsN)) {
+        tone_products_all<LARGE>(a, dsm);
+    } else {
+        const ProductsArea pm = products_area(dsm, N);
+        if (t < 32) tone_products_warp(a, sT, pm.psi, pm.w, pm.un, pm.red);
+        else if (t < 64 && a.extra) peak_delay_warp(a, sP);
         __syncthreads();
-        tone_products(a, pm);
-        if (a.extra && t < 32) peak_delay_warp(a, sP);
-        return true;
+        write_results_block(a, sT, pm);
     }
-    if (t < 32) tone_products_warp(a, sT, sm.pm.psi, sm.pm.w, sm.pm.un, sm.pm.out);
-    else if (t < 64 && a.extra) peak_delay_warp(a, sP);
-    __syncthreads();
-    write_results_block(a, sT, sm.pm);
     return true;
 }
 
 // One instantiation per sample format: the finalize runs once per step and its
 // instructions come from L2 (slow beside a streaming fold), so each plan's
 // kernel holds only its own format's decode.
-template <int FMT, bool LARGE = false>
+template <int FMT, int KIND>
 __global__ void __launch_bounds__(kClusterThreads, 1) fin_cluster_kernel(FinArgs a) {
     // The next fold may launch at once: it adds into the other set of bins
     // and waits for this kernel before its first atomic.
     allow_dependents();
     grid_dependency_wait();  // the bins of the preceding fold
-    cluster_finalize<FMT, LARGE>(a);
+    cluster_finalize<FMT, KIND>(a);
 }
 
 // Finalize arguments of one batched channel from its device state.
@@ -1119,6 +1503,7 @@ __device__ inline FinArgs batch_fin_args(const BatchChan& bc) {
     a.fmt = bc.fmt;
     a.spilled = 2;  // 2-bit sums live in the wide arrays
     a.L = bc.L;
+    a.rcp_L = bc.rcp_L;
     a.N = bc.N;
     a.so = bc.so;
     a.q = n_tot / bc.L;
@@ -1172,7 +1557,7 @@ __global__ void __launch_bounds__(kClusterThreads, 2) batch_fin_kernel(BatchChan
     __syncthreads();
     // every CTA has read the state above before the first cluster barrier
     // inside, and rank 0 returns after the last one
-    if (cluster_finalize(a) && threadIdx.x == 0) bc.period_start = bc.n_abs;
+    if (cluster_finalize<-1, kAny>(a) && threadIdx.x == 0) bc.period_start = bc.n_abs;
 }
 
 // After the batched DFT: block c runs channel c's products and
@@ -1190,10 +1575,15 @@ __global__ void __launch_bounds__(kClusterThreads, 1) batch_products_kernel(Batc
         sm.sP[i] = bc.Pslot[i];
     }
     __syncthreads();
-    if (t < 32) tone_products_warp(a, sm.sT, sm.pm.psi, sm.pm.w, sm.pm.un, sm.pm.out);
-    else if (t < 64 && a.extra) peak_delay_warp(a, sm.sP);
-    __syncthreads();
-    write_results_block(a, sm.sT, sm.pm);
+    if (bc.N > kWarpProductsN) {
+        tone_products_all<false>(a, dsm);
+    } else {
+        const ProductsArea pm = products_area(dsm, bc.N);
+        if (t < 32) tone_products_warp(a, sm.sT, pm.psi, pm.w, pm.un, pm.red);
+        else if (t < 64 && a.extra) peak_delay_warp(a, sm.sP);
+        __syncthreads();
+        write_results_block(a, sm.sT, pm);
+    }
     __syncthreads();
     if (t == 0) bc.period_start = bc.n_abs;
 }
@@ -1275,9 +1665,17 @@ cudaError_t launch_rotators(bool fixed, void* tw, int64_t L, float2* twN, int64_
     return cudaGetLastError();
 }
 
+// Integer plans that the short-period clusters do not take, up to kClusterBigN
+// tones: one cluster with the integer decode.  (float32 bins need an FP64
+// rotation, two operations per SM and clock: their wide plans spread over the
+// SMs.)
+static bool large_plan(const pcal_geometry& g) {
+    return g.format != PCAL_F32 && g.N <= kClusterBigN && (g.N > kClusterMaxN || g.L > kClusterMaxL);
+}
+
 cudaError_t launch_init_twiddles(pcal_plan* p, cudaStream_t s) {
     p->stats.kernel_launches += 1;
-    return launch_rotators(p->g.format != PCAL_F32, p->d_tw, p->g.L, p->d_twN, p->g.N, p->g.step_comb, s);
+    return launch_rotators(large_plan(p->g), p->d_tw, p->g.L, p->d_twN, p->g.N, p->g.step_comb, s);
 }
 
 namespace {
@@ -1335,14 +1733,16 @@ int cluster_size_for_device() {
     std::lock_guard<std::mutex> lock(mu);
     if (known[dev]) return cached[dev];
     int best = 0;
-    for (auto k : {fin_cluster_kernel<PCAL_2BIT>, fin_cluster_kernel<PCAL_I8>, fin_cluster_kernel<PCAL_F32>,
-                   fin_cluster_kernel<PCAL_2BIT, true>, fin_cluster_kernel<PCAL_I8, true>})
+    for (auto k : {fin_cluster_kernel<PCAL_2BIT, kFew>, fin_cluster_kernel<PCAL_I8, kFew>,
+                   fin_cluster_kernel<PCAL_F32, kFew>, fin_cluster_kernel<PCAL_2BIT, kMany>,
+                   fin_cluster_kernel<PCAL_I8, kMany>, fin_cluster_kernel<PCAL_F32, kMany>,
+                   fin_cluster_kernel<PCAL_2BIT, kLarge>, fin_cluster_kernel<PCAL_I8, kLarge>}) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
             (void)cudaGetLastError();
-    for (auto k : {fin_cluster_kernel<PCAL_2BIT, true>, fin_cluster_kernel<PCAL_I8, true>})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(large_smem_bytes(kClusterBigN) + kClusterPadSmem)) != cudaSuccess)
+                                 (int)(cluster_smem_bytes(kClusterBigN) + kClusterPadSmem)) != cudaSuccess)
             (void)cudaGetLastError();
+    }
     for (int c : {16, 8}) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(c);
@@ -1355,7 +1755,7 @@ int cluster_size_for_device() {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, fin_cluster_kernel<PCAL_2BIT>, &cfg) == cudaSuccess && n > 0) {
+        if (cudaOccupancyMaxActiveClusters(&n, fin_cluster_kernel<PCAL_2BIT, kFew>, &cfg) == cudaSuccess && n > 0) {
             best = c;
             break;
         }
@@ -1371,11 +1771,11 @@ int cluster_size_for_device() {
 // none of them fits on an SM beside a CTA of the fold that overlaps it (about
 // 205 KB each): sharing an SM with a fold CTA slowed the finalize 2-3x.  The
 // fold leaves kFinalizeReserveSms SMs for it.
-cudaError_t launch_cluster_finalize(const FinArgs& a, int C, bool large, cudaStream_t s) {
+cudaError_t launch_cluster_finalize(const FinArgs& a, int C, int kind, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C);
     cfg.blockDim = dim3(kClusterThreads);
-    cfg.dynamicSmemBytes = (large ? large_smem_bytes(a.N) : cluster_smem_bytes(a.N)) + kClusterPadSmem;
+    cfg.dynamicSmemBytes = cluster_smem_bytes(a.N) + kClusterPadSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1386,19 +1786,24 @@ cudaError_t launch_cluster_finalize(const FinArgs& a, int C, bool large, cudaStr
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (large)
-        return a.fmt == PCAL_2BIT ? cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT, true>, a)
-                                  : cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8, true>, a);
-    if (a.fmt == PCAL_2BIT) return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT>, a);
-    if (a.fmt == PCAL_I8) return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8>, a);
-    return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_F32>, a);
+    switch ((kind << 2) | a.fmt) {
+        case (kLarge << 2) | PCAL_2BIT: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT, kLarge>, a);
+        case (kLarge << 2) | PCAL_I8: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8, kLarge>, a);
+        case (kMany << 2) | PCAL_2BIT: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT, kMany>, a);
+        case (kMany << 2) | PCAL_I8: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8, kMany>, a);
+        case (kMany << 2) | PCAL_F32: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_F32, kMany>, a);
+        case (kFew << 2) | PCAL_2BIT: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT, kFew>, a);
+        case (kFew << 2) | PCAL_I8: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8, kFew>, a);
+        case (kFew << 2) | PCAL_F32: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_F32, kFew>, a);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // Finalize of a long-period plan: its rows of partial sums are added (and
 // cleared) by one cluster, then the DFT, the products and the post-processing
 // of the folded path.  (One CTA that added 9,728 rows of 16 bins took 115 us.)
 __global__ void __launch_bounds__(kClusterThreads, 1) rot_finalize_kernel(FinArgs a) {
-    cluster_finalize<kFmtRotated>(a);
+    cluster_finalize<kFmtRotated, kAny>(a);
 }
 
 }  // namespace
@@ -1495,6 +1900,7 @@ namespace {
 void set_common(FinArgs& a, const pcal_geometry& g, int64_t n_tot) {
     a.fs_hz = (double)g.fs;
     a.L = g.L;
+    a.rcp_L = reciprocal(g.L);
     a.N = g.N;
     a.so = g.step_offset;
     a.M = (double)n_tot;
@@ -1540,10 +1946,10 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
         a.n_pf = p->n_pending;
         a.pf_cols = g.row_samples / g.samples_per_byte_x4;
     }
-    if (g.format == PCAL_F32)
-        a.tw = static_cast<const double2*>(p->d_tw);
-    else
+    if (large_plan(g))
         a.twi = static_cast<const int4*>(p->d_tw);
+    else
+        a.tw = static_cast<const double2*>(p->d_tw);
     a.twN = p->d_twN;
     a.P = reinterpret_cast<float4*>(p->d_P);
     a.T = reinterpret_cast<float2*>(p->d_T);
@@ -1552,15 +1958,12 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
     a.ticket = p->d_ticket;
     cudaError_t e = cudaErrorUnknown;
     bool done = false;
-    // One cluster for every integer plan of up to kClusterBigN tones, and for
-    // float32 bins (FP64 rotation: two operations per SM and clock) of short
-    // periods only; the others spread over the SMs.
     const bool small = g.N <= kClusterMaxN && g.L <= kClusterMaxL;
-    if (small || (g.format != PCAL_F32 && g.N <= kClusterBigN)) {
+    if (small || large_plan(g)) {
         const int C = cluster_size_for_device();
         if (C > 0) {
             p->stats.kernel_launches += 1;
-            e = launch_cluster_finalize(a, C, !small, s);
+            e = launch_cluster_finalize(a, C, !small ? kLarge : g.N <= kFewN ? kFew : kMany, s);
             done = true;
         }
     }

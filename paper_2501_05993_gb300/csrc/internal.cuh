@@ -108,7 +108,7 @@ struct pcal_plan {
     PartSlot pending[kPartSlots]; // slots written by folds and not yet added into the bins
     int n_pending;
     int part_next;                // slot of the next float32 fold
-    void* d_tw;                   // exp(-j 2 pi m / L), m < L: double2 (float32), fixed-point int4 (integer bins)
+    void* d_tw;                   // exp(-j 2 pi m / L), m < L: double2, or fixed-point int4 (finalize.cu: large_plan)
     float2* d_twN;                // exp(-j 2 pi m / N), m < N (FP32)
     double2* d_P;                 // folded rotated bins P[b], b < N (scratch)
     double2* d_T;                 // tone phasors (scratch before products)
@@ -175,6 +175,7 @@ struct BatchChan {
     int N;
     int L;
     int64_t so;           // rotator index step per sample: f_offset/g (mod L)
+    unsigned long long rcp_L;  // floor((2^64 - 1) / L)
     int cols_total;       // words per bulk row
     int col_width;        // words per column group (the TMA box width)
     int col_groups;
