@@ -563,6 +563,9 @@ __global__ void fin_fold_kernel(FinArgs a) {
 constexpr int kClusterMaxN = 256;       // single plans: the cluster path up to here
 constexpr int kClusterBigN = 1024;      // batches: the cluster path up to here (DFT spread over the cluster)
 constexpr int kClusterThreads = 256;
+// kLarge plans decode up to thousands of bins a CTA: twice the warps hide the
+// loads (the DFT and the products keep the order of 256 threads).
+constexpr int kLargeThreads = 512;
 constexpr size_t kClusterPadSmem = 24 * 1024;
 constexpr int64_t kClusterMaxL = 32768;
 
@@ -1184,7 +1187,7 @@ __device__ __forceinline__ float4 residue_df(const FinArgs& a, int b, int m, int
         } else if constexpr (FMT != PCAL_F32 && KIND == kLarge) {
             if (a.exact)
                 return a.spilled ? residue_int<FMT, 1, 2>(a, b, m, step, m_end)
-                                 : residue_int<FMT, 0, 8>(a, b, m, step, m_end);
+                                 : residue_int<FMT, 0, 4>(a, b, m, step, m_end);
         }
         const double2 z = fold_residue<FMT>(a, b, m, step, m_end);
         const df dre = df_of(z.x), dim = df_of(z.y);
@@ -1208,9 +1211,11 @@ __host__ __device__ inline int dft_threads(int share) {
 
 // Tones [i0, i1) of the N-point DFT of sP in FP32, g threads each, written to
 // dst[i] (shared memory of this CTA or, through the cluster, of another).
-// PAIRS: i in [i0, i1) of 0 .. N/2, each with the tone N - i, whose twiddles
-// are the conjugates: one lookup serves both.  Eight steps at a time, their
-// twiddle indices from the first one's.
+// PAIRS: i in [i0, i1) of 1 .. N/2, each with the tone N - i, whose twiddles
+// are the conjugates: one lookup serves both.  (Tone 0 goes apart: with it in
+// the list, 256 tones took 129 threads, and the fifth warp shared a scheduler
+// with the first for the whole sum.)  Four steps at a time, their twiddle
+// indices from the first one's.
 template <bool PAIRS>
 __device__ __forceinline__ void dft_tones_smem(const float2* sP, const float2* sTw, int N, int i0, int i1, float2* dst,
                                                int g) {
@@ -1235,29 +1240,29 @@ __device__ __forceinline__ void dft_tones_smem(const float2* sP, const float2* s
             unsigned int ix = (unsigned int)(i * gs) % un;  // i, g below 2^11
             const unsigned int step = (unsigned int)(i * g) % un;
             int bb = gs;
-            if (bb + 7 * g < N) {
-                unsigned int off[8];  // k steps on
+            if (bb + 3 * g < N) {
+                unsigned int off[4];  // k steps on
                 off[0] = 0;
 #pragma unroll
-                for (int k = 1; k < 8; ++k) {
+                for (int k = 1; k < 4; ++k) {
                     off[k] = off[k - 1] + step;
                     off[k] = min(off[k], off[k] - un);
                 }
-                unsigned int eight = off[7] + step;
-                eight = min(eight, eight - un);
+                unsigned int four = off[3] + step;
+                four = min(four, four - un);
 #pragma unroll 1
-                for (; bb + 7 * g < N; bb += 8 * g) {
-                    float2 p[8], w[8];
+                for (; bb + 3 * g < N; bb += 4 * g) {
+                    float2 p[4], w[4];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
+                    for (int k = 0; k < 4; ++k) {
                         unsigned int x = ix + off[k];
                         x = min(x, x - un);
                         p[k] = sP[bb + k * g];
                         w[k] = sTw[tw_slot((int)x)];
                     }
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) add(p[k], w[k]);
-                    ix += eight;
+                    for (int k = 0; k < 4; ++k) add(p[k], w[k]);
+                    ix += four;
                     ix = min(ix, ix - un);
                 }
             }
@@ -1279,9 +1284,31 @@ __device__ __forceinline__ void dft_tones_smem(const float2* sP, const float2* s
         }
         if (i < i1 && gs == 0) {
             dst[i] = make_float2(sre, sim);
-            if (PAIRS && i > 0 && 2 * i != N) dst[N - i] = make_float2(cre, cim);
+            if (PAIRS && 2 * i != N) dst[N - i] = make_float2(cre, cim);
         }
     }
+}
+
+// Tone 0 the same way (every twiddle is the first one), by the g threads from
+// t0 on (within one warp).
+__device__ __forceinline__ void dft_zero(const float2* sP, float2 w, int N, float2* dst, int g, int t0) {
+    const int gs = (int)threadIdx.x - t0;
+    if (((int)threadIdx.x >> 5) != (t0 >> 5)) return;  // (whole warps)
+    float sre = 0.f, sim = 0.f;
+    if (gs >= 0 && gs < g) {
+#pragma unroll 4
+        for (int bb = gs; bb < N; bb += g) {
+            const float2 p = sP[bb];
+            sre = fmaf(p.x, w.x, fmaf(-p.y, w.y, sre));
+            sim = fmaf(p.x, w.y, fmaf(p.y, w.x, sim));
+        }
+    }
+#pragma unroll 1
+    for (int o = g / 2; o > 0; o >>= 1) {
+        sre += __shfl_xor_sync(0xffffffffu, sre, o);
+        sim += __shfl_xor_sync(0xffffffffu, sim, o);
+    }
+    if (gs == 0) dst[0] = make_float2(sre, sim);
 }
 
 // All tones of a DFT of at most kFewN: the same sums in a loop that is short
@@ -1337,7 +1364,8 @@ template <int FMT, int KIND>
 __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    __shared__ float4 part[kClusterThreads];  // per (lane, residue) df partials: re hi, re lo, im hi, im lo
+    // per (lane, residue) df partials: re hi, re lo, im hi, im lo
+    __shared__ float4 part[KIND == kLarge ? kLargeThreads : kClusterThreads];
     extern __shared__ __align__(16) uint8_t dsm[];
     const int C = (int)cluster.num_blocks(), r = (int)cluster.block_rank();
     const int N = (int)a.N;
@@ -1345,9 +1373,9 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
     float4* Pr = sm.Pr;
     float2 *sP = sm.sP, *sTw = sm.sTw, *sT = sm.sT;
     const int t = threadIdx.x;
-    // N > blockDim: one lane per residue, the residues in turns
+    // N > kClusterThreads: one lane per residue, the residues in turns
     constexpr bool LARGE = KIND == kLarge;
-    const bool big = KIND >= kLarge && N > (int)blockDim.x;
+    const bool big = KIND >= kLarge && N > kClusterThreads;
     const int lanes = big ? 1 : (int)blockDim.x / N;
     if (r == 0 || N > kClusterMaxN)
         for (int i = t; i < N; i += blockDim.x) sTw[KIND == kFew ? i : tw_slot(i)] = a.twN[i];
@@ -1446,7 +1474,11 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
         if (KIND == kFew)
             dft_few(sP, sTw, N, sT, dft_threads(N));
         else
-            dft_tones_smem<true>(sP, sTw, N, 0, N / 2 + 1, sT, dft_threads(N));
+{
+            const int g = dft_threads(N);
+            dft_tones_smem<true>(sP, sTw, N, 1, N / 2 + 1, sT, g);
+            dft_zero(sP, sTw[0], N, sT, g, kClusterThreads / 2);
+        }
     } else {
         // every CTA: its share of the tones, into CTA 0's sT
         float2* dst = cluster.map_shared_rank(sT, 0);
@@ -1457,8 +1489,9 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
                                 : (FMT == kFmtRotated ? N : N / C);
         const int most = LARGE ? kDftTonesPerCta : (FMT == kFmtRotated ? N : (N + C - 1) / C);
         if (dft_threads(least) == dft_threads(most)) {
-            const int H = N / 2 + 1;
-            dft_tones_smem<true>(sP, sTw, N, H * r / C, H * (r + 1) / C, dst, dft_threads(most));
+            const int H = N / 2, g = dft_threads(most);
+            dft_tones_smem<true>(sP, sTw, N, 1 + H * r / C, 1 + H * (r + 1) / C, dst, g);
+            if (r == C - 1) dft_zero(sP, sTw[0], N, dst, g, kClusterThreads / 2);
         } else if constexpr (LARGE) {
             for (int i0 = r * kDftTonesPerCta; i0 < N; i0 += C * kDftTonesPerCta) {
                 const int n = N - i0 < kDftTonesPerCta ? N - i0 : kDftTonesPerCta;
@@ -1488,7 +1521,7 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
 // instructions come from L2 (slow beside a streaming fold), so each plan's
 // kernel holds only its own format's decode.
 template <int FMT, int KIND>
-__global__ void __launch_bounds__(kClusterThreads, 1) fin_cluster_kernel(FinArgs a) {
+__global__ void __launch_bounds__(KIND == kLarge ? kLargeThreads : kClusterThreads, 1) fin_cluster_kernel(FinArgs a) {
     // The next fold may launch at once: it adds into the other set of bins
     // and waits for this kernel before its first atomic.
     allow_dependents();
@@ -1774,7 +1807,7 @@ int cluster_size_for_device() {
 cudaError_t launch_cluster_finalize(const FinArgs& a, int C, int kind, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(kClusterThreads);
+    cfg.blockDim = dim3(kind == kLarge ? kLargeThreads : kClusterThreads);
     cfg.dynamicSmemBytes = cluster_smem_bytes(a.N) + kClusterPadSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
