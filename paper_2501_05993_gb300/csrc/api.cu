@@ -13,6 +13,7 @@ namespace {
 // Inputs shorter than this many bulk rows (or bytes) go through the ragged
 // kernel alone: the bulk kernel's fixed cost does not pay off below it.
 constexpr int64_t kBulkMinBytes = 1 << 20;
+constexpr int64_t kShortMinBytes = 8 << 10, kShortMaxBytes = 1 << 28;
 constexpr size_t kStageBytes = 64ull << 20;
 
 int cuda_status(cudaError_t e) {
@@ -89,7 +90,9 @@ int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
     if (rows > 0 && bulk_tiling(p, rows, &probe) != 0) rows = 0;  // no tile plan: ragged only
     cudaError_t e = cudaSuccess;
     if (rows == 0) {
-        e = launch_ragged(p, d, n, k0, s);
+        // a few KB: one sample a thread does (and so would an input without a tile plan)
+        const int64_t b = bytes_of(p, n);
+        e = b < kShortMinBytes || b >= kShortMaxBytes ? launch_ragged(p, d, n, k0, s) : launch_short(p, d, n, k0, s);
     } else {
         if (head > 0) e = launch_ragged(p, d, head, k0, s);
         const uint8_t* body = d + bytes_of(p, head);
@@ -148,6 +151,7 @@ extern "C" int pcal_plan_create(double fs, double f_comb, double f_offset, int N
         memset(static_cast<void*>(p->h_hint), 0, kHintRing * sizeof(PrefetchHint));
         e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&p->d_hint), p->h_hint, 0);
     }
+    if (e == cudaSuccess) e = prepare_short();
     if (e == cudaSuccess) e = launch_init_twiddles(p, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
