@@ -94,14 +94,26 @@ int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
         const int64_t b = bytes_of(p, n);
         e = b < kShortMinBytes || b >= kShortMaxBytes ? launch_ragged(p, d, n, k0, s) : launch_short(p, d, n, k0, s);
     } else {
-        if (head > 0) e = launch_ragged(p, d, head, k0, s);
         const uint8_t* body = d + bytes_of(p, head);
+        const int64_t done = head + rows * row, tail = n - done;
+        const uint8_t* behind = body + bytes_of(p, rows * row);
+        // what is no whole row: with the rows where a thread each is enough,
+        // else launches of its own around them
+        BulkEdges edges{{d, behind}, {0, 0}, {k0, (k0 + done) % L}};
+        const bool inside = p->g.format != PCAL_F32 && bytes_of(p, head + tail) <=
+                                                           probe.col_groups * probe.row_groups * probe.threads;
+        if (inside) {
+            edges.n[0] = (int)bytes_of(p, head);
+            edges.n[1] = (int)bytes_of(p, tail);
+        } else if (head > 0) {
+            e = launch_ragged(p, d, head, k0, s);
+        }
         int launched = 0;
-        if (e == cudaSuccess) e = launch_bulk(p, body, rows, (k0 + head) % L, s, &launched);
+        if (e == cudaSuccess) e = launch_bulk(p, body, rows, (k0 + head) % L, inside ? &edges : nullptr, s, &launched);
         if (e == cudaSuccess) p->stats.bulk_launches += 1;
-        const int64_t done = head + rows * row;
-        if (e == cudaSuccess && done < n)
-            e = launch_ragged(p, body + bytes_of(p, rows * row), n - done, (k0 + done) % L, s);
+        if (e == cudaSuccess && tail > 0 && !inside)
+            e = bytes_of(p, tail) < kShortMinBytes ? launch_ragged(p, behind, tail, (k0 + done) % L, s)
+                                                   : launch_short(p, behind, tail, (k0 + done) % L, s);
     }
     if (e != cudaSuccess) return cuda_status(e);
     p->n_abs += n;

@@ -158,12 +158,20 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s);
 // Add a float32 plan's pending partial slots into its bins (one reduce launch; none when nothing is pending).
 cudaError_t flush_partials(pcal_plan* p, cudaStream_t s);
 
+// The bytes before a bulk launch's first row and behind its last one (2-bit
+// and int8), folded by the same launch: at most one a thread.
+struct BulkEdges {
+    const uint8_t* ptr[2];
+    int n[2];      // bytes
+    int64_t k[2];  // phase of the first sample
+};
+
 // Bulk fold of whole rows of row_samples samples starting at a 16-byte
 // aligned device address whose first sample has phase k_a = n mod L.
 // Returns cudaSuccess and sets *launched = the number of kernels launched,
-// or an error.  Rows must be >= 1.
-cudaError_t launch_bulk(pcal_plan* p, const void* d_rows, int64_t n_rows, int64_t k_a, cudaStream_t s,
-                        int* launched);
+// or an error.  Rows must be >= 1; edges may be null.
+cudaError_t launch_bulk(pcal_plan* p, const void* d_rows, int64_t n_rows, int64_t k_a, const BulkEdges* edges,
+                        cudaStream_t s, int* launched);
 
 int bulk_tiling(const pcal_plan* p, int64_t n_rows, BulkTiling* t);
 
