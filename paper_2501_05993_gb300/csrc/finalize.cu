@@ -1698,17 +1698,20 @@ cudaError_t launch_rotators(bool fixed, void* tw, int64_t L, float2* twN, int64_
     return cudaGetLastError();
 }
 
-// Integer plans that the short-period clusters do not take, up to kClusterBigN
-// tones: one cluster with the integer decode.  (float32 bins need an FP64
-// rotation, two operations per SM and clock: their wide plans spread over the
-// SMs.)
+// Plans that the short-period clusters do not take, up to kClusterBigN tones:
+// one cluster too, integer bins with the integer decode, float32 bins (an FP64
+// rotation, two operations per SM and clock) as long as 16 SMs decode them in
+// about 10 us.  The others spread over the SMs.
+constexpr int64_t kLargeF32L = 131072;
 static bool large_plan(const pcal_geometry& g) {
-    return g.format != PCAL_F32 && g.N <= kClusterBigN && (g.N > kClusterMaxN || g.L > kClusterMaxL);
+    return g.N <= kClusterBigN && (g.N > kClusterMaxN || g.L > kClusterMaxL) &&
+           (g.format != PCAL_F32 || g.L <= kLargeF32L);
 }
+static bool fixed_rotators(const pcal_geometry& g) { return g.format != PCAL_F32 && large_plan(g); }
 
 cudaError_t launch_init_twiddles(pcal_plan* p, cudaStream_t s) {
     p->stats.kernel_launches += 1;
-    return launch_rotators(large_plan(p->g), p->d_tw, p->g.L, p->d_twN, p->g.N, p->g.step_comb, s);
+    return launch_rotators(fixed_rotators(p->g), p->d_tw, p->g.L, p->d_twN, p->g.N, p->g.step_comb, s);
 }
 
 namespace {
@@ -1769,7 +1772,8 @@ int cluster_size_for_device() {
     for (auto k : {fin_cluster_kernel<PCAL_2BIT, kFew>, fin_cluster_kernel<PCAL_I8, kFew>,
                    fin_cluster_kernel<PCAL_F32, kFew>, fin_cluster_kernel<PCAL_2BIT, kMany>,
                    fin_cluster_kernel<PCAL_I8, kMany>, fin_cluster_kernel<PCAL_F32, kMany>,
-                   fin_cluster_kernel<PCAL_2BIT, kLarge>, fin_cluster_kernel<PCAL_I8, kLarge>}) {
+                   fin_cluster_kernel<PCAL_2BIT, kLarge>, fin_cluster_kernel<PCAL_I8, kLarge>,
+                   fin_cluster_kernel<PCAL_F32, kLarge>}) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
             (void)cudaGetLastError();
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1822,6 +1826,7 @@ cudaError_t launch_cluster_finalize(const FinArgs& a, int C, int kind, cudaStrea
     switch ((kind << 2) | a.fmt) {
         case (kLarge << 2) | PCAL_2BIT: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT, kLarge>, a);
         case (kLarge << 2) | PCAL_I8: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8, kLarge>, a);
+        case (kLarge << 2) | PCAL_F32: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_F32, kLarge>, a);
         case (kMany << 2) | PCAL_2BIT: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_2BIT, kMany>, a);
         case (kMany << 2) | PCAL_I8: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_I8, kMany>, a);
         case (kMany << 2) | PCAL_F32: return cudaLaunchKernelEx(&cfg, fin_cluster_kernel<PCAL_F32, kMany>, a);
@@ -1930,6 +1935,8 @@ cudaError_t launch_batch_finalize(BatchChan* d_ch, int n_ch, int max_n, const in
 
 namespace {
 
+constexpr int64_t kFlushFirstL = 6144;
+
 void set_common(FinArgs& a, const pcal_geometry& g, int64_t n_tot) {
     a.fs_hz = (double)g.fs;
     a.L = g.L;
@@ -1946,6 +1953,12 @@ void set_common(FinArgs& a, const pcal_geometry& g, int64_t n_tot) {
 }  // namespace
 
 cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
+    // float32 bins of a long period: the pending partials by all SMs first (16
+    // CTAs that add them bin by bin took 25 us for L 25600)
+    if (p->g.format == PCAL_F32 && p->g.L >= kFlushFirstL && p->n_pending > 0) {
+        const cudaError_t e = flush_partials(p, s);
+        if (e != cudaSuccess) return e;
+    }
     FinArgs a{};
     const pcal_geometry& g = p->g;
     const int64_t n_tot = p->n_abs - p->period_start;
@@ -1979,7 +1992,7 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
         a.n_pf = p->n_pending;
         a.pf_cols = g.row_samples / g.samples_per_byte_x4;
     }
-    if (large_plan(g))
+    if (fixed_rotators(g))
         a.twi = static_cast<const int4*>(p->d_tw);
     else
         a.tw = static_cast<const double2*>(p->d_tw);

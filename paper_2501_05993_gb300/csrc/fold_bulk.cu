@@ -544,6 +544,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1) bulk_fold_kernel(const __grid_co
 // only once every block of this one has started, so the grid is at most one
 // block per SM and its warps stride over the bins.
 constexpr int kReduceWarps = 16;  // warps per block
+constexpr int64_t kReduceBinsL = 6144;  // periods from which on the bins are a thread each
 
 struct PendingArgs {
     const float2* base[kPartSlots];
@@ -586,6 +587,40 @@ __global__ void __launch_bounds__(32 * kReduceWarps) reduce_f32_kernel(const __g
             s = pcal_df::add(pcal_df::df{a.x, a.y}, s);
             acc[k] = make_float2(s.hi, s.lo);
         }
+    }
+}
+
+// The same sums with one thread per bin, for long periods: their rows fill the
+// SMs with column groups, so a bin has few partials, a warp per bin leaves its
+// lanes idle (L 25600, four slots: 47 us), and consecutive bins' partials are
+// consecutive.  In slot, row group and column order.
+__global__ void __launch_bounds__(256) reduce_f32_bins_kernel(const __grid_constant__ PendingArgs pa, int cols_total,
+                                                              int L, float2* __restrict__ acc) {
+    allow_dependents();
+    grid_dependency_wait();
+    const int stride = (int)(gridDim.x * blockDim.x);
+    for (int k = (int)(blockIdx.x * blockDim.x + threadIdx.x); k < L; k += stride) {
+        const float2 a = acc[k];
+        pcal_df::df s{a.x, a.y};
+        for (int e = 0; e < pa.n; ++e) {
+            const int k_a = (int)pa.k_a[e], R = (int)pa.row_groups[e];
+            for (int c = k >= k_a ? k - k_a : k - k_a + L; c < cols_total; c += L) {
+                const float2* col = pa.base[e] + c;
+                int rg = 0;
+                for (; rg + 4 <= R; rg += 4) {
+                    float2 v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v[u] = col[(int64_t)(rg + u) * cols_total];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) s = pcal_df::add(s, pcal_df::two_sum(v[u].x, v[u].y));
+                }
+                for (; rg < R; ++rg) {
+                    const float2 v = col[(int64_t)rg * cols_total];
+                    s = pcal_df::add(s, pcal_df::two_sum(v.x, v.y));
+                }
+            }
+        }
+        acc[k] = make_float2(s.hi, s.lo);
     }
 }
 
@@ -793,17 +828,20 @@ cudaError_t flush_partials(pcal_plan* p, cudaStream_t s) {
     pa.n = p->n_pending;
     const int spw = p->g.samples_per_byte_x4;
     const int cols_total = (int)(p->g.row_samples / spw);
-    const int64_t blocks = (p->g.L + kReduceWarps - 1) / kReduceWarps;
+    const bool bins = p->g.L >= kReduceBinsL;
+    const int64_t per_block = bins ? 256 : kReduceWarps;
+    const int64_t blocks = (p->g.L + per_block - 1) / per_block;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(blocks < p->num_sms ? blocks : p->num_sms));
-    cfg.blockDim = dim3(32 * kReduceWarps);
+    cfg.blockDim = dim3(bins ? 256 : 32 * kReduceWarps);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, reduce_f32_kernel, pa, cols_total, (int64_t)p->g.L, cur_accf(p));
+    const cudaError_t e = bins ? cudaLaunchKernelEx(&cfg, reduce_f32_bins_kernel, pa, cols_total, (int)p->g.L, cur_accf(p))
+                               : cudaLaunchKernelEx(&cfg, reduce_f32_kernel, pa, cols_total, (int64_t)p->g.L, cur_accf(p));
     if (e == cudaSuccess) {
         p->n_pending = 0;
         p->stats.kernel_launches += 1;

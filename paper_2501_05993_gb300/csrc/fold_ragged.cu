@@ -55,17 +55,28 @@ __global__ void ragged_i8_kernel(const int8_t* __restrict__ x, int64_t n, int64_
     }
 }
 
-// One thread per bin k: sums the samples of this run that fall into bin k, in
-// order, in double-float, and adds the sum to the plan's double-float bin.
-__global__ void ragged_f32_kernel(const float* __restrict__ x, int64_t n, int64_t k0, int64_t L,
-                                  float2* __restrict__ acc) {
+// One thread per bin k: sums the samples of two runs (before and behind a bulk
+// launch's rows) that fall into bin k, in order, in double-float, and adds the
+// sum to the plan's double-float bin.
+struct FloatRun {
+    const float* x;
+    int64_t n, k0;  // samples, phase of the first one
+};
+
+__global__ void ragged_f32_kernel(FloatRun r0, FloatRun r1, int64_t L, float2* __restrict__ acc) {
     chain_in();
-    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= L) return;
-    int64_t t = (k - k0 % L + L) % L;  // first sample index of this run in bin k
-    if (t >= n) return;
     pcal_df::df s{0.f, 0.f};
-    for (; t < n; t += L) s = pcal_df::add_f(s, x[t]);
+    bool any = false;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const FloatRun& r = e ? r1 : r0;
+        int64_t t = k >= r.k0 ? k - r.k0 : k - r.k0 + L;  // first sample of the run in bin k
+        any = any || t < r.n;
+        for (; t < r.n; t += L) s = pcal_df::add_f(s, r.x[t]);
+    }
+    if (!any) return;
     const float2 a = acc[k];
     s = pcal_df::add(pcal_df::df{a.x, a.y}, s);
     acc[k] = make_float2(s.hi, s.lo);
@@ -254,6 +265,14 @@ inline int grid_for(int64_t work, int threads, int num_sms) {
 
 }  // namespace
 
+cudaError_t launch_ragged_f32(pcal_plan* p, const uint8_t* d0, int64_t n0, int64_t k0, const uint8_t* d1, int64_t n1,
+                              int64_t k1, cudaStream_t s) {
+    const int64_t L = p->g.L;
+    const FloatRun r0{reinterpret_cast<const float*>(d0), n0, k0 % L}, r1{reinterpret_cast<const float*>(d1), n1, k1 % L};
+    p->stats.kernel_launches += 1;
+    return launch_chained(ragged_f32_kernel, (int)((L + 255) / 256), 256, s, 0, r0, r1, L, cur_accf(p));
+}
+
 cudaError_t launch_ragged(pcal_plan* p, const uint8_t* d_bytes, int64_t n, int64_t k0, cudaStream_t s) {
     const int64_t L = p->g.L;
     if (n <= 0) return cudaSuccess;
@@ -269,10 +288,7 @@ cudaError_t launch_ragged(pcal_plan* p, const uint8_t* d_bytes, int64_t n, int64
             e = launch_chained(ragged_i8_kernel, grid_for(n, 256, p->num_sms), 256, s, 0,
                                reinterpret_cast<const int8_t*>(d_bytes), n, k0, L, cur_acc8(p));
             break;
-        default:
-            e = launch_chained(ragged_f32_kernel, (int)((L + 255) / 256), 256, s, 0,
-                               reinterpret_cast<const float*>(d_bytes), n, k0, L, cur_accf(p));
-            break;
+        default: return launch_ragged_f32(p, d_bytes, n, k0, nullptr, 0, 0, s);
     }
     p->stats.kernel_launches += 1;
     return e;

@@ -149,6 +149,9 @@ cudaError_t launch_init_twiddles(pcal_plan* p, cudaStream_t s);
 cudaError_t launch_rotators(bool fixed, void* tw, int64_t L, float2* twN, int64_t N, int64_t step_comb,
                             cudaStream_t s);
 cudaError_t launch_ragged(pcal_plan* p, const uint8_t* d_bytes, int64_t n_samples, int64_t k0, cudaStream_t s);
+// float32: two runs in one launch.
+cudaError_t launch_ragged_f32(pcal_plan* p, const uint8_t* d0, int64_t n0, int64_t k0, const uint8_t* d1, int64_t n1,
+                              int64_t k1, cudaStream_t s);
 // Fold of a run too short for the bulk kernel, at any alignment (one launch).
 cudaError_t launch_short(pcal_plan* p, const uint8_t* d_bytes, int64_t n_samples, int64_t k0, cudaStream_t s);
 cudaError_t prepare_short();
