@@ -233,7 +233,7 @@ typedef struct {
     int64_t n_abs;          /* samples accumulated since plan creation      */
     int64_t n_period;       /* samples in the current integration period    */
     int64_t kernel_launches;/* CUDA kernels this plan has launched          */
-    int64_t bulk_launches;  /* of which bulk (TMA bit-plane) fold kernels   */
+    int64_t bulk_launches;  /* of which folds of a call's whole rows, 1 MB+ */
     int64_t bytes_folded;   /* sample bytes folded on the device            */
 } pcal_stats;
 

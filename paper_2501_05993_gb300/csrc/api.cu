@@ -10,10 +10,11 @@
 
 namespace {
 
-// Inputs shorter than this many bulk rows (or bytes) go through the ragged
-// kernel alone: the bulk kernel's fixed cost does not pay off below it.
+// Inputs of fewer bytes in whole rows go through a short fold (or, a few KB, the
+// ragged kernel) alone: the bulk kernel's fixed cost does not pay off below it.
 constexpr int64_t kBulkMinBytes = 1 << 20;
 constexpr int64_t kShortMinBytes = 8 << 10, kShortMaxBytes = 1 << 28;
+constexpr int64_t kShortPeriods = 256, kShortRows = 128;
 constexpr size_t kStageBytes = 64ull << 20;
 
 int cuda_status(cudaError_t e) {
@@ -87,12 +88,23 @@ int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
     int64_t rows = (n - head) / row;
     if (bytes_of(p, rows * row) < kBulkMinBytes) rows = 0;
     BulkTiling probe;
-    if (rows > 0 && bulk_tiling(p, rows, &probe) != 0) rows = 0;  // no tile plan: ragged only
+    if (rows > 0 && bulk_tiling(p, rows, &probe) != 0) rows = 0;  // no tile plan: short or ragged only
+    // Few rows, each wider than the SMs have column groups for (long periods):
+    // the bulk kernel's CTAs would come in waves with a box or two each.  A step
+    // of L 1,024,000 int8: 3 MB 99 -> 69 us, 128 MB (125 rows) 112 -> 83; 2-bit 64 MB
+    // (250 rows) the same either way.  float32 (also no partials then): L 25,600
+    // 16 MB (156 periods) 33 -> 29 us, 32 MB 34 -> 32, 64 MB 28 -> 42; L 6,400 3 MB
+    // 14.8 -> 12.0, 8 MB (312) 16.0 -> 16.2; L 256,000 32 MB 96 -> 51.
+    const bool wide = rows > 0 && (p->g.format == PCAL_F32 ? n <= kShortPeriods * L
+                                                           : rows <= kShortRows && probe.col_groups > p->num_sms);
+    if (wide) rows = 0;
     cudaError_t e = cudaSuccess;
     if (rows == 0) {
         // a few KB: one sample a thread does (and so would an input without a tile plan)
         const int64_t b = bytes_of(p, n);
-        e = b < kShortMinBytes || b >= kShortMaxBytes ? launch_ragged(p, d, n, k0, s) : launch_short(p, d, n, k0, s);
+        const bool few = b < kShortMinBytes || (p->g.format != PCAL_F32 && b >= kShortMaxBytes);
+        e = few ? launch_ragged(p, d, n, k0, s) : launch_short(p, d, n, k0, s);
+        if (e == cudaSuccess && wide) p->stats.bulk_launches += 1;
     } else {
         const uint8_t* body = d + bytes_of(p, head);
         const int64_t done = head + rows * row, tail = n - done;

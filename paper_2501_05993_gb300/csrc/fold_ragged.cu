@@ -298,8 +298,10 @@ cudaError_t launch_short(pcal_plan* p, const uint8_t* d, int64_t n, int64_t k0, 
     using namespace pcal_direct;
     const int64_t L = p->g.L;
     if (p->g.format == PCAL_F32) {
-        // eight warps per 32 bins, 32 where each would still take many periods
-        const int warps = n / L > 512 ? 32 : 8;
+        // a warp per eight periods (its loads in flight together), at most eight,
+        // or 32 where each would still take many
+        const int64_t periods = (n + L - 1) / L;
+        const int warps = periods > 512 ? 32 : periods > 56 ? 8 : (int)((periods + 7) / 8);
         p->stats.kernel_launches += 1;
         return launch_chained(short_f32_kernel, (int)((L + 31) / 32), 32 * warps, s, 0,
                               reinterpret_cast<const float*>(d), n, k0, L, cur_accf(p));
@@ -316,8 +318,11 @@ cudaError_t launch_short(pcal_plan* p, const uint8_t* d, int64_t n, int64_t k0, 
     a.part = ShortBlock{reinterpret_cast<const uint32_t*>(d + at), 0, (int)(part / 4)};
     a.n_rows = (int)rows;
     a.blocks = (int)((row_bytes / 4 + cols - 1) / cols);
-    // one chunk of 128 2-bit or 64 int8 rows, more where whole ones fit
-    const int64_t least = p->g.format == PCAL_2BIT ? 128 : 64;
+    // chunks of at least 128 2-bit or 64 int8 rows (below that the atomic adds
+    // of 512 bins cost as much as the loads), of about eight per resident CTA
+    int64_t least = p->g.format == PCAL_2BIT ? 128 : 64;
+    const int64_t even = bytes / (8 * kDirectCtas * p->num_sms) / (4 * cols);
+    if (least < even) least = even < kDirectRows / 2 ? even : kDirectRows / 2;
     const int64_t chunks = rows / least > 0 ? rows / least : 1;
     a.chunk_rows = (int)((rows + chunks - 1) / chunks);
     if (a.chunk_rows < 1) a.chunk_rows = 1;
