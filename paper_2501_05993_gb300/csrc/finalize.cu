@@ -1840,14 +1840,16 @@ cudaError_t launch_cluster_finalize(const FinArgs& a, int C, int kind, cudaStrea
 // Finalize of a long-period plan: its rows of partial sums are added (and
 // cleared) by one cluster, then the DFT, the products and the post-processing
 // of the folded path.  (One CTA that added 9,728 rows of 16 bins took 115 us.)
-__global__ void __launch_bounds__(kClusterThreads, 1) rot_finalize_kernel(FinArgs a) {
-    cluster_finalize<kFmtRotated, kAny>(a);
+__global__ void __launch_bounds__(kClusterThreads, 1) rot_finalize_kernel(FinArgs a, const unsigned int* err) {
+    grid_dependency_wait();  // the rows of the preceding fold
+    if (cluster_finalize<kFmtRotated, kAny>(a) && threadIdx.x == 0)
+        *reinterpret_cast<unsigned int*>(a.res + 6 * a.N + 5) = *err;
 }
 
 }  // namespace
 
 cudaError_t launch_rot_finalize(float4* rows, int n_rows, int N, double fs, double fc, int64_t M,
-                                const float2* twN, double* res, cudaStream_t s) {
+                                const float2* twN, double* res, const unsigned int* err, cudaStream_t s) {
     FinArgs a{};
     a.N = N;
     a.L = (int64_t)N * n_rows;
@@ -1868,14 +1870,16 @@ cudaError_t launch_rot_finalize(float4* rows, int n_rows, int N, double fs, doub
     cfg.blockDim = dim3(kClusterThreads);
     cfg.dynamicSmemBytes = cluster_smem_bytes(N);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, rot_finalize_kernel, a);
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, rot_finalize_kernel, a, err);
 }
 
 cudaError_t prepare_rot_finalize() {

@@ -246,9 +246,10 @@ struct BatchPiece {
 
 cudaError_t prepare_batch_finalize();
 // Finalize of a long-period plan: rows = [n_rows][N] double-float bin sums
-// (re hi, re lo, im hi, im lo), added and cleared.
+// (re hi, re lo, im hi, im lo), added and cleared.  res: 6N+5 values, then the
+// error word *err.
 cudaError_t launch_rot_finalize(float4* rows, int n_rows, int N, double fs, double fc, int64_t M,
-                                const float2* twN, double* res, cudaStream_t s);
+                                const float2* twN, double* res, const unsigned int* err, cudaStream_t s);
 // The CUDA calls launch_rot_finalize needs once per device.
 cudaError_t prepare_rot_finalize();
 // Finalize channels list[i] (or i when list is null), i < n, with one cluster each.

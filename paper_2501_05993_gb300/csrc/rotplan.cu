@@ -387,6 +387,8 @@ __global__ void __launch_bounds__(MAXT, MINB) rotplan_fold_kernel(const __grid_c
             phase ^= 1u;
         }
     }
+    // the finalize may launch (it waits for this kernel before it reads a row)
+    allow_dependents();
     if (s_fail) {
         // copies in flight (of units u .. u + kStages - 1) land before the
         // CTA's shared memory is reused
@@ -510,10 +512,13 @@ struct pcal_rotplan {
     float4* d_W;          // weights of a block: float4 [K], or the digit words
     float4* d_E;          // [kBlocks]
     float4* d_F;          // [S]
-    unsigned int* d_err;  // behind the results
+    unsigned int* d_err;
     float2* d_twN;
-    double* d_res;  // 5N+3 results, N+2 post-processing values, the error bits
+    // 5N+3 results, N+2 post-processing values, the error bits: pinned memory that
+    // the finalize writes through its device address (a copy behind it cost the
+    // host's wait 5 us)
     double* h_res;
+    double* d_res;
     cudaStream_t last_stream;
     bool results_valid;
 };
@@ -561,11 +566,14 @@ extern "C" int pcal_rotplan_create(double fs, double f_comb, double f_offset, in
         e = cudaFuncSetAttribute(rot_kernel(r->g, sample_format), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kRotMaxSmem);
     if (e == cudaSuccess) e = cudaMalloc(&r->d_twN, sizeof(float2) * N);
-    // results, post-processing, and the device error bits behind them
-    if (e == cudaSuccess) e = cudaMalloc(&r->d_res, sizeof(double) * (6 * (size_t)N + 6));
-    if (e == cudaSuccess) e = cudaMemset(r->d_res, 0, sizeof(double) * (6 * (size_t)N + 6));
-    if (e == cudaSuccess) r->d_err = reinterpret_cast<unsigned int*>(r->d_res + 6 * (size_t)N + 5);
-    if (e == cudaSuccess) e = cudaMallocHost(&r->h_res, sizeof(double) * (6 * (size_t)N + 6));
+    if (e == cudaSuccess) e = cudaMalloc(&r->d_err, sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemset(r->d_err, 0, sizeof(unsigned int));
+    if (e == cudaSuccess)
+        e = cudaHostAlloc(reinterpret_cast<void**>(&r->h_res), sizeof(double) * (6 * (size_t)N + 6), cudaHostAllocMapped);
+    if (e == cudaSuccess) {
+        memset(static_cast<void*>(r->h_res), 0, sizeof(double) * (6 * (size_t)N + 6));
+        e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&r->d_res), r->h_res, 0);
+    }
     if (e == cudaSuccess) {
         rotplan_twiddles_kernel<<<(N + 255) / 256, 256>>>(r->d_twN, N);
         const int most = r->g.S > r->g.K ? r->g.S : r->g.K;
@@ -591,7 +599,7 @@ extern "C" int pcal_rotplan_destroy(pcal_rotplan* r) {
     cudaFree(r->d_E);
     cudaFree(r->d_F);
     cudaFree(r->d_twN);
-    cudaFree(r->d_res);
+    cudaFree(r->d_err);
     if (r->h_res) cudaFreeHost(r->h_res);
     (void)cudaGetLastError();
     delete r;
@@ -666,7 +674,7 @@ extern "C" int pcal_rotplan_finalize_device(pcal_rotplan* r, void* stream) {
     const int64_t M = r->n_abs - r->period_start;
     // adds the rows of partial sums and clears them for the next period
     const cudaError_t e = launch_rot_finalize(r->d_acc, r->g.ctas + 1, r->N, (double)r->fs, (double)r->fc, M,
-                                              r->d_twN, r->d_res, s);
+                                              r->d_twN, r->d_res, r->d_err, s);
     if (e != cudaSuccess) return PCAL_ECUDA;
     r->period_start = r->n_abs;
     r->last_stream = s;
@@ -680,10 +688,7 @@ extern "C" int pcal_rotplan_read_results(pcal_rotplan* r, double* phasors, doubl
     if (!r) return PCAL_EINVAL;
     if (!r->results_valid) return PCAL_EBUSY;
     const int64_t N = r->N;
-    cudaError_t e = cudaMemcpyAsync(r->h_res, r->d_res, sizeof(double) * (6 * N + 6), cudaMemcpyDeviceToHost,
-                                    r->last_stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(r->last_stream);
-    if (e != cudaSuccess) return PCAL_ECUDA;
+    if (cudaStreamSynchronize(r->last_stream) != cudaSuccess) return PCAL_ECUDA;
     const double* h = r->h_res;
     unsigned int err;
     memcpy(&err, h + 6 * N + 5, sizeof(err));
