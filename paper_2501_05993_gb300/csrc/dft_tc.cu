@@ -1,5 +1,5 @@
 // Batched tone DFT: the entry points of every mode, and the tensor-core
-// (tcgen05) contraction for the tone counts that dft_fft.cu does not take (a
+// (tcgen05) contraction for the tone counts that dft_fft.cuh does not take (a
 // prime factor above 7; at C 4096, N 1024 the contraction takes 176 us in split
 // TF32, the FFT 53).  The contraction: T_i = sum_b P[b] e^{-j2 pi ib/N}
 // for C channels at once (the "DFT(P)" step of Sec. 2 after the L-to-N fold of
@@ -568,7 +568,7 @@ __global__ void dft_fp32_kernel(const float2* __restrict__ P, float2* __restrict
 
 struct pcal_dft {
     int N, mode, n_cols, k_chunks, col_tiles, parts;
-    FftPlan fft;      // every mode, where N has small prime factors; the contraction's state is then not made
+    pcal_fft::FftPlan fft;      // every mode, where N has small prime factors; the contraction's state is then not made
     uint8_t* d_w;     // weight tiles (tensor-core modes)
     uint8_t* d_a;     // operand tiles of P (workspace)
     size_t a_cap;     // bytes of d_a
@@ -658,10 +658,10 @@ extern "C" int pcal_dft_create(int N, int mode, pcal_dft** out) {
     memset(static_cast<void*>(d), 0, sizeof(*d));
     d->N = N;
     d->mode = mode;
-    if (fft_factors(N, &d->fft)) {
+    if (pcal_fft::fft_factors(N, &d->fft)) {
         cudaError_t e = cudaMalloc(&d->d_err, sizeof(unsigned int));
         if (e == cudaSuccess) e = cudaMemset(d->d_err, 0, sizeof(unsigned int));
-        if (e == cudaSuccess) e = fft_create(N, mode != PCAL_DFT_FP32, &d->fft);
+        if (e == cudaSuccess) e = pcal_fft::fft_create(N, mode != PCAL_DFT_FP32, &d->fft);
         if (e != cudaSuccess) {
             pcal_dft_destroy(d);
             (void)cudaGetLastError();
@@ -729,7 +729,7 @@ extern "C" int pcal_dft_create(int N, int mode, pcal_dft** out) {
 extern "C" int pcal_dft_destroy(pcal_dft* d) {
     if (!d) return PCAL_OK;
     cudaDeviceSynchronize();
-    fft_destroy(&d->fft);
+    pcal_fft::fft_destroy(&d->fft);
     cudaFree(d->d_w);
     cudaFree(d->d_a);
     cudaFree(d->d_tw);
@@ -753,7 +753,7 @@ cudaError_t dft_reserve(pcal_dft* d, int64_t C) {
 
 cudaError_t launch_dft(pcal_dft* d, const float2* P, int64_t C, float2* T, cudaStream_t s, unsigned int* err) {
     if (C <= 0) return cudaSuccess;
-    if (d->fft.passes) return launch_fft(d->fft, P, C, T, s);
+    if (d->fft.passes) return pcal_fft::launch_fft(d->fft, P, C, T, s);
     if (d->mode == PCAL_DFT_FP32) {
         dft_fp32_kernel<<<(unsigned)C, 256, 2 * d->N * sizeof(float2), s>>>(P, T, d->N, d->d_tw);
         return cudaGetLastError();
