@@ -90,15 +90,6 @@ def read_peaks():
         return 6800.0, "fallback"
 
 
-def read_tensor_peak():
-    """Measured dense bf16 tensor throughput (burst, TFLOP/s), else the fallback."""
-    try:
-        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-            return float(json.load(f)["bf16_tflops"]), "measured"
-    except Exception:
-        return 1900.0, "fallback"
-
-
 def read_batch_traffic_ratio():
     """DRAM bytes per sample byte of the batched fold from its committed ncu
     summary (captured on a reduced batch), or None when batch.cu changed."""
@@ -548,7 +539,7 @@ BATCH_SEED = 2501059932 + 1
 BATCH_WORKLOAD = ("64 channels, length U[0.5, 8] s in whole 10 ms, fs in {32, 64, 128, 256} MHz, f_comb 1 MHz, "
                   "f_offset 10 kHz x U{0..99}, even channels 2-bit, odd int8 (sigma 20), tone amplitude "
                   "U[0.005, 0.02] sigma, t_d U[0, 50] ns")
-BATCH_METRIC = "PCal Gsamples/s, batched (one persistent fold launch + one finalize launch per step) vs plain"
+BATCH_METRIC = "PCal Gsamples/s, batched (one fold launch + one finalize launch per step) vs plain"
 BLOCK_SAMPLES = 32 * 1024 * 1024
 
 
@@ -660,7 +651,7 @@ def run_batch(args, emit=True):
     torch.cuda.synchronize()
     graph_ms = g0.elapsed_time(g1) / args.steps
 
-    # the persistent fold alone (roofline): accumulate-only steps
+    # the fold alone (roofline): accumulate-only steps
     f0, f1 = ev(), ev()
     f0.record(stream)
     for _ in range(args.steps):
@@ -731,7 +722,8 @@ def run_batch(args, emit=True):
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": int(ratio * total_bytes) if ratio else None,
                 "traffic_note": "scaled from a reduced batch capture (profiles/batch_fold_mixed.txt)",
-                "peak_kind": f"{peak_kind} (copy bandwidth)", "kernel": "batch_fold_kernel",
+                "peak_kind": f"{peak_kind} (copy bandwidth)",
+                "kernel": "batch_fold_kernel or batch_direct_kernel (the faster in the autotuner)",
                 "algorithmic_bytes_per_launch": total_bytes}
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline:  # the host baseline: N = 1 only
@@ -739,7 +731,7 @@ def run_batch(args, emit=True):
         cpu = {"value": v, "unit": UNIT, "cores": 1, "kind": "oracle",
                "sample": f"direct FP64 definition over the first {args.cpu_sample} samples of a 2-bit channel "
                          f"({dt:.1f} s)"}
-    # the finalize alone with each tone DFT (fused CUDA-core FP32 vs one tensor-core contraction per N)
+    # the finalize alone with each tone DFT (in the clusters, or one batched DFT launch per N)
     fin_modes = {}
     for mode in ("fp32", "tf32x3", "bf16x6"):
         batch.set_dft(mode)
@@ -855,7 +847,7 @@ DFT_WORKLOAD = "batched tone DFT, 4096 channels x N 1024 (complex64 P -> T), see
 
 def run_tensor_dft(args, emit=True, C=4096, N=1024, reps=20):
     """pcal_dft_execute in every mode on one batch of P: time per launch (CUDA events over back-to-back
-    launches), achieved TFLOP/s of the algorithmic contraction against the measured tensor peak, and the
+    launches), bandwidth of its one read and one write against the measured copy bandwidth, and the
     error against the DFT definition in FP64."""
     import torch
 
@@ -870,7 +862,7 @@ def run_tensor_dft(args, emit=True, C=4096, N=1024, reps=20):
     ref = np.fft.fft(P.astype(np.complex128), axis=1)
     dP = torch.from_numpy(P).cuda()
     dT = torch.empty((C, N), dtype=torch.complex64, device="cuda")
-    peak_bf16, peak_kind = read_tensor_peak()
+    peak, peak_kind = read_peaks()
     modes = {}
     method_flops = 8.0 * C * N * N  # the DFT itself: C x N x N complex multiply-adds
     for mode in ("fp32", "tf32x3", "bf16x6"):
@@ -887,19 +879,11 @@ def run_tensor_dft(args, emit=True, C=4096, N=1024, reps=20):
             flags = d.check()
         T = dT.cpu().numpy()
         err = np.max(np.abs(T - ref), axis=1) / np.max(np.abs(ref), axis=1)
-        roof = None
-        executed = method_flops
-        if mode != "fp32":
-            # real C x 2N x 2N products: three (split TF32) or six (split BF16)
-            executed = (3 if mode == "tf32x3" else 6) * 2.0 * C * (2 * N) * (2 * N)
-            # TF32 from the measured bf16 peak and the nominal dense ratio (1.1 / 2.25 PFLOP/s)
-            peak = peak_bf16 * (1.1 / 2.25) if mode == "tf32x3" else peak_bf16
-            ach = method_flops / (ms / 1e3) / 1e12
-            roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                    "traffic": None, "work": "method flops 8 C N^2 (the DFT itself)",
-                    "executed_tflops": executed / (ms / 1e3) / 1e12,
-                    "executed_frac": executed / (ms / 1e3) / 1e12 / peak,
-                    "peak_kind": f"{peak_kind} bf16 burst" + (" x 1.1/2.25 (tf32)" if mode == "tf32x3" else "")}
+        # N here has small prime factors only: every mode is the FFT, one read of P and one write of T
+        moved = 2.0 * 8 * C * N
+        gbs = moved / (ms / 1e3) / 1e9
+        roof = {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "traffic": None,
+                "algorithmic_bytes_per_launch": moved, "peak_kind": f"{peak_kind} (copy bandwidth)"}
         modes[mode] = {"ms": ms, "tflops": method_flops / (ms / 1e3) / 1e12, "max_rel_err": float(err.max()),
                        "median_rel_err": float(np.median(err)), "device_error_bits": flags, "roofline": roof}
     out = {"metric": "batched tone DFT time per launch", "value": modes["tf32x3"]["ms"], "unit": "ms",
@@ -1282,7 +1266,7 @@ def compact_summary(out: dict) -> dict:
     if td:
         sm["dft"] = {m: [_sig(v["ms"], 3), _sig(v["max_rel_err"], 2), _sig(get(v, "roofline", "frac"), 3)]
                      for m, v in td.items()}
-        sm["dft"]["fmt"] = "[ms, max err, method-work frac]"
+        sm["dft"]["fmt"] = "[ms, max err, HBM frac]"
     return sm
 
 

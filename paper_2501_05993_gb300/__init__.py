@@ -577,7 +577,7 @@ def pcal_batch_autotune(batch: int, samples, n, stream=None) -> Schedule:
 
 
 class Batch:
-    """Many channels (2-bit or int8) folded by one persistent launch per call."""
+    """Many channels (2-bit or int8) folded by one launch per call."""
 
     def __init__(self, channels):
         self.channels = [tuple(c) for c in channels]
@@ -659,7 +659,7 @@ class Batch:
 
     def set_dft(self, mode: str):
         """Tone DFT of the finalize: "fp32" (inside each channel's cluster), "tf32x3" or "bf16x6"
-        (one tensor-core contraction per distinct N)."""
+        (one batched DFT launch per distinct N)."""
         _check(load().pcal_batch_set_dft(self.handle, DFT_MODES[mode]), "pcal_batch_set_dft")
 
     def autotune(self, samples, n, stream=None) -> dict:

@@ -1,5 +1,5 @@
 // Batched extraction (pcal_batch_*): many channels of mixed sample format,
-// sample rate, comb offset, period L and length, folded by ONE persistent
+// sample rate, comb offset, period L and length, folded by ONE
 // launch and finalized by one launch with a thread-block cluster per channel.
 //
 // Two folds.  The direct fold (below) takes every call of a batch whose
