@@ -67,3 +67,27 @@ def test_direct_fold_bins_are_exact(pcal):
             bins = b.bins(c)
             assert np.array_equal(bins, ref), (c, np.argwhere(bins != ref)[:4].tolist())
             assert np.array_equal(bins, p.bins(c))
+
+
+def test_finalize_order_of_many_channels(pcal):
+    """45 channels whose clusters cannot all run at once, the shortest finalizes first in channel order (the launch
+    starts the longest first): every channel gets its own results, twice.  Bound: the phasor bound of the other
+    paths, 1e-5 of the largest."""
+    chans = [(fs, 1_000_000, 10_000 * (1 + i % 3), "i8" if i % 2 else "2bit")
+             for fs in (16_000_000, 64_000_000, 1_024_000_000) for i in range(15)]
+    n = [400_000 + 4 * i for i in range(len(chans))]
+    hosts = [synth.Stream(fs=c[0], fc=c[1], fo=c[2], amp=0.05, td=1e-9, seed=90 + i).samples(c[3], 0, n[i])
+             for i, c in enumerate(chans)]
+    dev = [_dev(h, 0) for h in hosts]
+    with pcal.Batch(chans) as b:
+        plans = [pcal.Plan(*c[:3], fmt=c[3]) for c in chans]
+        for _ in range(2):
+            b.accumulate([a for _, a in dev], n)
+            b.finalize_device()
+            for i, p in enumerate(plans):
+                pcal.pcal_accumulate(p.handle, dev[i][1], n[i], 0)
+                T = p.finalize()
+                got = b.results(i)["phasors"]
+                assert np.max(np.abs(got - T)) <= 1e-5 * np.max(np.abs(T)), i
+        for p in plans:
+            p.close()
