@@ -353,7 +353,7 @@ int pcal_batch_set_schedule(pcal_batch* batch, const pcal_schedule* sched);
 /* How the batch finalize runs the tone DFT (the PCAL_DFT_* modes of the
  * batched tone DFT below): PCAL_DFT_FP32 (default) inside each channel's
  * finalize cluster on CUDA cores; PCAL_DFT_TC_TF32X3 / PCAL_DFT_TC_BF16X6 as
- * one tensor-core contraction per distinct N over all channels of that N (the
+ * one batched DFT launch per distinct N over all channels of that N (the
  * clusters stop at P, then a products kernel finishes every channel).
  * Synchronises the device; drops captured step graphs. */
 int pcal_batch_set_dft(pcal_batch* batch, int mode);
@@ -576,9 +576,10 @@ int pcal_rotplan_read_results(pcal_rotplan* plan, double* phasors, double* amp, 
  * Sec. 2, after the L-to-N fold of Eq. 2).  P and T: DEVICE, C x N complex
  * float32 (re, im interleaved, channel-major), owned by the caller; T may not
  * alias P.  Where N has no prime factor above 7 every mode is a mixed-radix
- * FFT: PCAL_DFT_FP32 in FP32, the tensor-core modes with double-float values
- * inside each pass (errors vs FP64 at N = 1024, rms over rms: 1.1e-7 and
- * 0.4e-7; the contractions below 2.0e-7 and 1.7e-7, the direct sum 8e-7).
+ * FFT: PCAL_DFT_FP32 in FP32, the tensor-core modes in FP32 from 500 tones on
+ * and with double-float values inside each pass below (and at every N inside a
+ * batch's finalize).  Errors vs FP64 at N = 1024, rms over rms: 1.1e-7 and
+ * 0.4e-7; the contractions below 2.0e-7 and 1.7e-7, the direct sum 8e-7.
  * For the other N:
  *   PCAL_DFT_FP32       CUDA cores, FP32 sums
  *   PCAL_DFT_TC_TF32X3  tensor cores (tcgen05): [Re P | Im P] . W as one real

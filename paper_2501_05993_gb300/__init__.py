@@ -888,7 +888,8 @@ DFT_CHUNK_BYTES = {"tf32x3": 128, "bf16x6": 64}  # bytes of K per weight tile ro
 
 class Dft:
     """Batched N-point tone DFT of C channels: T[c, i] = sum_b P[c, b] e^{-j 2 pi i b / N}
-    (device complex64 arrays [C][N]); mode "fp32" (CUDA cores), "tf32x3" or "bf16x6" (tensor cores)."""
+    (device complex64 arrays [C][N]); mode "fp32", "tf32x3" or "bf16x6" (an FFT where
+    N has no prime factor above 7; else CUDA cores, or tensor cores in split operands)."""
 
     def __init__(self, N: int, mode: str = "tf32x3"):
         self.N, self.mode = int(N), mode

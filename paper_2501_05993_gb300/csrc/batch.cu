@@ -1213,7 +1213,7 @@ extern "C" int pcal_batch_set_dft(pcal_batch* b, int mode) {
             if (!g) {
                 b->dft.push_back(DftGroup{b->h_ch[c].N, 0, nullptr, nullptr, nullptr});
                 g = &b->dft.back();
-                rc = pcal_dft_create(g->N, mode, &g->dft);
+                rc = dft_create(g->N, mode, true, &g->dft);
             }
             ++g->count;
         }

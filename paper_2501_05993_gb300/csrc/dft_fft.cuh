@@ -11,18 +11,23 @@
 // The twiddles of a pass lie in the order its threads read them (N - 1 in
 // all, from FP64, through L1).
 //
-// Two precisions.  The CUDA-core mode works in FP32.  The tensor-core modes
-// carry double-float values through each pass and round to FP32 between
-// passes, because FP32 butterflies alone (rms error 1.1e-7 at N = 1024,
-// 0.6e-7 at N = 20) are no better than the split-BF16 contraction at small N
-// (0.5e-7 at N = 20) and moved the delay of a strong comb by 1.07e-3 of its
-// sigma; rounding once per pass gives 0.4 to 0.5e-7 at every N.
+// Two precisions.  The CUDA-core mode works in FP32.  The tensor-core modes are
+// to be no less accurate than the contraction.  Its rms error grows with N (split
+// BF16 0.55e-7 at N = 20, 1.08e-7 at 256, 1.72e-7 at 1024; split TF32 1.2 to
+// 2.0e-7), that of FP32 butterflies hardly (0.66e-7, 0.92e-7, 1.07e-7): from
+// kFftSingleN tones on FP32 is the more accurate in every measure (rms, worst
+// channel, worst tone; at 486 tones the worst channel was not).  Below it, and
+// wherever a delay follows (a batch's finalize), they carry double-float values
+// through each pass and round to FP32 between passes (0.35 to 0.5e-7): with FP32
+// alone the delay of a strong comb of 1024 tones moved by 1.07e-3 of its sigma.
 //
 // Why not the dense contraction of dft_tc.cu here: that does 8 N^2 operations a
 // channel, this one 5 N log2 N, and its sums are log2 N long instead of N.
 // C 4096, N 1024, 67 MB: FP32 direct sum 2930 us, split-TF32 contraction 176 us,
-// this kernel with double-float passes 50 us, bound by the FP32 pipes (about
-// 300 operations a value; HBM alone would take 10 us).
+// this kernel 23 us in FP32 (bound by latency and issue slots, index arithmetic
+// and shared-memory exchanges beside the butterflies; HBM alone would take
+// 10 us) and 50 us with double-float passes (the FP32 pipes: about 300
+// operations a value).  N 256, C 4096, double-float: 33 -> 12.5 us.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -34,6 +39,7 @@
 namespace pcal_fft {
 
 constexpr int kFftMaxPasses = 12;
+constexpr int kFftSingleN = 500;  // tensor-core modes: FP32 inside passes from here on
 
 struct FftPlan {
     int N, passes;             // passes == 0: N has a prime factor above 7 (or is 1)

@@ -1,7 +1,7 @@
 // Batched tone DFT: the entry points of every mode, and the tensor-core
 // (tcgen05) contraction for the tone counts that dft_fft.cuh does not take (a
 // prime factor above 7; at C 4096, N 1024 the contraction takes 176 us in split
-// TF32, the FFT 53).  The contraction: T_i = sum_b P[b] e^{-j2 pi ib/N}
+// TF32, the FFT 23).  The contraction: T_i = sum_b P[b] e^{-j2 pi ib/N}
 // for C channels at once (the "DFT(P)" step of Sec. 2 after the L-to-N fold of
 // Eq. 2), as one real contraction
 //
@@ -650,7 +650,9 @@ extern "C" int pcal_dft_weights_host(int N, int mode, int tile, int chunk, void*
     return PCAL_OK;
 }
 
-extern "C" int pcal_dft_create(int N, int mode, pcal_dft** out) {
+extern "C" int pcal_dft_create(int N, int mode, pcal_dft** out) { return dft_create(N, mode, false, out); }
+
+int dft_create(int N, int mode, bool delays, pcal_dft** out) {
     if (!out || N < 1 || N > PCAL_BATCH_MAX_N) return PCAL_EINVAL;
     if (mode != PCAL_DFT_FP32 && mode != PCAL_DFT_TC_TF32X3 && mode != PCAL_DFT_TC_BF16X6) return PCAL_EINVAL;
     pcal_dft* d = new (std::nothrow) pcal_dft();
@@ -661,7 +663,8 @@ extern "C" int pcal_dft_create(int N, int mode, pcal_dft** out) {
     if (pcal_fft::fft_factors(N, &d->fft)) {
         cudaError_t e = cudaMalloc(&d->d_err, sizeof(unsigned int));
         if (e == cudaSuccess) e = cudaMemset(d->d_err, 0, sizeof(unsigned int));
-        if (e == cudaSuccess) e = pcal_fft::fft_create(N, mode != PCAL_DFT_FP32, &d->fft);
+        const bool wide = mode != PCAL_DFT_FP32 && (delays || N < pcal_fft::kFftSingleN);
+        if (e == cudaSuccess) e = pcal_fft::fft_create(N, wide, &d->fft);
         if (e != cudaSuccess) {
             pcal_dft_destroy(d);
             (void)cudaGetLastError();

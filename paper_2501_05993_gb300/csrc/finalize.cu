@@ -34,7 +34,7 @@
 // large N a second kernel spreads the DFT over CTAs and its last CTA runs the
 // products.  What bounds a cluster is its chain of dependent steps, the
 // instructions of each fetched from L2 once; alone 9 to 11 us at 64 tones and
-// L 6400, 29 us at 256 tones and L 1,024,000 beside a fold.
+// L 6400, 29 us at 256 tones and L 256,000 beside a fold.
 #include <cooperative_groups.h>
 #include <math.h>
 

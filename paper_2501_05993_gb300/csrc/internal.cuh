@@ -263,6 +263,10 @@ struct pcal_dft;
 // DFT object's own).
 cudaError_t launch_dft(pcal_dft* d, const float2* P, int64_t C, float2* T, cudaStream_t s,
                        unsigned int* err = nullptr);
+// pcal_dft_create; delays: the phasors go on to a delay whose error counts in
+// units of its sigma, so the FFT of the tensor-core modes is the accurate one
+// at every N.
+int dft_create(int N, int mode, bool delays, pcal_dft** out);
 // Operand workspace of launch_dft for up to C channels (allocates).
 cudaError_t dft_reserve(pcal_dft* d, int64_t C);
 
