@@ -174,7 +174,9 @@ __device__ int grab_boxes(unsigned long long* ctr, unsigned int epoch, int take,
 // waits for its uses in order.  Every thread of the group arrives on the
 // stage's empty barrier once it holds the box's words in registers (2-bit)
 // or has folded them (int8, float32).
-template <int FMT, int U>
+// EDGES: the call has bytes before or behind its rows (kept out of the kernel
+// of aligned calls, which they cost 0.1 us of 20.5: 128 MB of 2-bit).
+template <int FMT, int U, bool EDGES>
 __global__ void __launch_bounds__(kMaxBlock, 1) bulk_fold_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                  const BulkArgs a) {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -210,7 +212,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1) bulk_fold_kernel(const __grid_co
     // and adds its samples with the CTA's flush.  (As two launches of their own,
     // one after this one, they cost an int8 step of 12.8 MB 2 us.)
     uint32_t edge = 0, edge_k = 0;
-    if (FMT != PCAL_F32 && a.edges.n[0] + a.edges.n[1] > 0) {
+    if constexpr (EDGES) {
         const int g = (int)(blockIdx.x * blockDim.x) + tid, i = g < a.edges.n[0] ? 0 : 1;
         const int at = i ? g - a.edges.n[0] : g;
         if (at < a.edges.n[i]) {
@@ -449,7 +451,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1) bulk_fold_kernel(const __grid_co
         const int S = a.merge_stride;
         const int tasks = a.col_width * 16;
         const uint32_t Lu = (uint32_t)a.L;
-        if (edge) {
+        if (EDGES && edge) {
 #pragma unroll 1
             for (int j = 0; j < 4; ++j) {
                 const uint32_t c = (edge >> (2 * j)) & 3u, k = edge_k + j < Lu ? edge_k + j : (edge_k + j) % Lu;
@@ -489,7 +491,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1) bulk_fold_kernel(const __grid_co
         }
         __syncthreads();
         grid_dependency_wait();  // as for the 2-bit flush
-        if (edge)
+        if (EDGES && edge)
             atomicAdd(reinterpret_cast<unsigned long long*>(&a.acc8[edge_k]),
                       (unsigned long long)(long long)(int8_t)edge);
         const int tasks = a.col_width * 4;
@@ -647,9 +649,9 @@ int bits_for(int64_t v) {
 // start while that kernel finishes.  Nothing it touches depends on that
 // kernel (new counter epoch; atomics into the current bin set, which a
 // preceding finalize does not touch); it waits for it only at its very end.
-template <int FMT, int U>
+template <int FMT, int U, bool EDGES>
 cudaError_t launch_one(const CUtensorMap& map, const BulkArgs& a, int grid, int block, size_t smem, cudaStream_t s) {
-    auto k = bulk_fold_kernel<FMT, U>;
+    auto k = bulk_fold_kernel<FMT, U, EDGES>;
     static size_t smem_set = 0;  // per instantiation; the attribute only grows
     if (smem > smem_set) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -667,6 +669,19 @@ cudaError_t launch_one(const CUtensorMap& map, const BulkArgs& a, int grid, int 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, map, a);
+}
+
+// int8 and 2-bit launches (2-bit: a kernel per number of upper counter planes).
+template <bool EDGES>
+cudaError_t launch_int(const pcal_plan* p, const CUtensorMap& map, const BulkArgs& a, const BulkTiling& t,
+                       cudaStream_t s) {
+    const int grid = (int)(t.col_groups * t.row_groups), u = t.upper_planes;
+    if (p->g.format == PCAL_I8) return launch_one<PCAL_I8, 1, EDGES>(map, a, grid, t.threads, t.smem_bytes, s);
+    if (u <= 3) return launch_one<PCAL_2BIT, 3, EDGES>(map, a, grid, t.threads, t.smem_bytes, s);
+    if (u <= 5) return launch_one<PCAL_2BIT, 5, EDGES>(map, a, grid, t.threads, t.smem_bytes, s);
+    if (u <= 7) return launch_one<PCAL_2BIT, 7, EDGES>(map, a, grid, t.threads, t.smem_bytes, s);
+    if (u <= 9) return launch_one<PCAL_2BIT, 9, EDGES>(map, a, grid, t.threads, t.smem_bytes, s);
+    return launch_one<PCAL_2BIT, 11, EDGES>(map, a, grid, t.threads, t.smem_bytes, s);
 }
 
 }  // namespace
@@ -949,7 +964,7 @@ cudaError_t launch_bulk(pcal_plan* p, const void* d_rows, int64_t n_rows, int64_
         }
         const int slot = p->part_next;
         a.partf = p->d_partf + (size_t)slot * p->partf_cap;
-        e = launch_one<PCAL_F32, 1>(map, a, grid, t.threads, t.smem_bytes, s);
+        e = launch_one<PCAL_F32, 1, false>(map, a, grid, t.threads, t.smem_bytes, s);
         if (e != cudaSuccess) {
             unpublish_hint(p, a.epoch);
             return e;
@@ -960,21 +975,8 @@ cudaError_t launch_bulk(pcal_plan* p, const void* d_rows, int64_t n_rows, int64_
         p->stats.kernel_launches += 1;
         return cudaSuccess;
     }
-    if (p->g.format == PCAL_I8) {
-        e = launch_one<PCAL_I8, 1>(map, a, grid, t.threads, t.smem_bytes, s);
-    } else {
-        const int u = t.upper_planes;
-        if (u <= 3)
-            e = launch_one<PCAL_2BIT, 3>(map, a, grid, t.threads, t.smem_bytes, s);
-        else if (u <= 5)
-            e = launch_one<PCAL_2BIT, 5>(map, a, grid, t.threads, t.smem_bytes, s);
-        else if (u <= 7)
-            e = launch_one<PCAL_2BIT, 7>(map, a, grid, t.threads, t.smem_bytes, s);
-        else if (u <= 9)
-            e = launch_one<PCAL_2BIT, 9>(map, a, grid, t.threads, t.smem_bytes, s);
-        else
-            e = launch_one<PCAL_2BIT, 11>(map, a, grid, t.threads, t.smem_bytes, s);
-    }
+    const bool with_edges = a.edges.n[0] + a.edges.n[1] > 0;
+    e = with_edges ? launch_int<true>(p, map, a, t, s) : launch_int<false>(p, map, a, t, s);
     if (e == cudaSuccess) {
         *launched = 1;
         p->stats.kernel_launches += 1;
