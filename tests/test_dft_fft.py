@@ -3,8 +3,8 @@ contraction or the direct sum for the others, at the smallest counts, one of eac
 radix lists, the largest counts, and channel counts around a block's tile.
 
 Tolerance (max over channels of max|T - T_ref| / max|T_ref|, FP64 reference): the FFT makes at most about 20
-consecutive FP32 roundings of 2^-24 (two per level of a butterfly) or, in the tensor-core modes, one per pass;
-both stay below 20 * 2^-24 = 1.2e-6.  The other counts keep the bounds of the existing paths."""
+consecutive FP32 roundings of 2^-24 (two per level of a butterfly) or, in the tensor-core modes below 500 tones,
+one per pass; both stay below 20 * 2^-24 = 1.2e-6.  The other counts keep the bounds of the existing paths."""
 import numpy as np
 import pytest
 
