@@ -53,7 +53,7 @@ constexpr int kBulkMapCache = 16;
 // SMs the bulk fold leaves free (on GPUs with at least 64 SMs) for the
 // one-cluster finalize that overlaps it.
 constexpr int kFinalizeReserveSms = 16;
-constexpr int kSchedCounters = 8192;  // dynamic box counters (one per column group) + 1
+constexpr int kSchedCounters = 8192;  // dynamic box counters, one per column group that several CTAs share
 
 // Where a plan's bulk launch with epoch e starts reading, published by the
 // host in ring slot e % kHintRing (pinned, mapped) when it enqueues that
