@@ -233,13 +233,29 @@ typedef struct {
     int64_t n_abs;          /* samples accumulated since plan creation      */
     int64_t n_period;       /* samples in the current integration period    */
     int64_t kernel_launches;/* CUDA kernels this plan has launched          */
-    int64_t bulk_launches;  /* of which folds of a call's whole rows, 1 MB+ */
+    int64_t bulk_launches;  /* of which folds of a call's whole rows, 1 MB+, */
+                            /* by whichever kernel (see pcal_fold_counts)    */
     int64_t bytes_folded;   /* sample bytes folded on the device            */
 } pcal_stats;
 
 /* Copy the plan's counters into *out (host bookkeeping; no CUDA call, no
  * synchronisation).  PCAL_EINVAL for a NULL argument. */
 int pcal_get_stats(const pcal_plan* plan, pcal_stats* out);
+
+/* Fold kernels launched so far, by kind: which of its folds the library took
+ * for the calls of a plan (the first three) or a batch (the last two; a
+ * replayed step counts as its fold). */
+typedef struct {
+    int64_t bulk;        /* bulk folds (TMA tiles of whole rows)                */
+    int64_t short_folds; /* short folds: small calls, and few, wide rows        */
+    int64_t ragged;      /* sample by sample: a few KB, and edges of bulk folds */
+    int64_t persistent;  /* batches under a schedule                            */
+    int64_t direct;      /* batches without one                                 */
+} pcal_fold_counts;
+
+/* Copy the counts into *out (host bookkeeping; no CUDA call, no
+ * synchronisation).  PCAL_EINVAL for a NULL argument. */
+int pcal_get_fold_counts(const pcal_plan* plan, pcal_fold_counts* out);
 
 /*
  * Work split of the bulk fold kernel (host only, no CUDA call), for tests and
@@ -404,6 +420,9 @@ int pcal_batch_get_bins(pcal_batch* batch, int channel, int64_t* host_out);
  * n_period is not kept and stays 0): host bookkeeping, no synchronisation.
  * PCAL_EINVAL for a NULL argument. */
 int pcal_batch_get_stats(const pcal_batch* batch, pcal_stats* out);
+
+/* Its folds by kind (pcal_fold_counts above), likewise. */
+int pcal_batch_get_fold_counts(const pcal_batch* batch, pcal_fold_counts* out);
 
 /*
  * Time candidate schedules on these inputs, accumulate only, and keep the

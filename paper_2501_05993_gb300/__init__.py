@@ -43,6 +43,13 @@ class Stats(ctypes.Structure):
         return {k: getattr(self, k) for k, _ in self._fields_}
 
 
+class FoldCounts(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_int64) for k in ("bulk", "short_folds", "ragged", "persistent", "direct")]
+
+    def as_dict(self) -> dict:
+        return {k: getattr(self, k) for k, _ in self._fields_}
+
+
 class Tiling(ctypes.Structure):
     _fields_ = [("cols_total", ctypes.c_int32), ("col_width", ctypes.c_int32), ("col_groups", ctypes.c_int32),
                 ("replicas", ctypes.c_int32), ("box_rows", ctypes.c_int32), ("stages", ctypes.c_int32),
@@ -135,6 +142,7 @@ def load(path: str | None = None):
         "pcal_result_device": ([vp], vp),
         "pcal_get_bins": ([vp, vp], ci),
         "pcal_get_stats": ([vp, P(Stats)], ci),
+        "pcal_get_fold_counts": ([vp, P(FoldCounts)], ci),
         "pcal_strerror": ([ci], ctypes.c_char_p),
         "pcal_bulk_tiling": ([dbl, dbl, dbl, ci, ci, ci, i64, P(Tiling)], ci),
         "pcal_tones_from_counts_noalloc": ([dbl, dbl, dbl, ci, vp, i64, P(dbl), vp, vp], ci),
@@ -152,6 +160,7 @@ def load(path: str | None = None):
         "pcal_batch_read_post": ([vp, ci, vp, vp, vp], ci),
         "pcal_batch_get_bins": ([vp, ci, vp], ci),
         "pcal_batch_get_stats": ([vp, P(Stats)], ci),
+        "pcal_batch_get_fold_counts": ([vp, P(FoldCounts)], ci),
         "pcal_batch_autotune": ([vp, P(vp), P(i64), vp, P(Schedule)], ci),
         "pcal_server_stream_bytes": ([P(ServerConfig), P(ChannelDesc), P(i64)], ci),
         "pcal_rotfold_create": ([dbl, dbl, dbl, ci, ci, ci, ci, P(vp)], ci),
@@ -469,6 +478,12 @@ class Plan:
     def stats(self) -> dict:
         return pcal_get_stats(self.handle).as_dict()
 
+    def fold_counts(self) -> dict:
+        """Fold kernels launched so far, by kind."""
+        f = FoldCounts()
+        _check(load().pcal_get_fold_counts(self.handle, ctypes.byref(f)), "pcal_get_fold_counts")
+        return f.as_dict()
+
     @property
     def result_device_ptr(self) -> int:
         return pcal_result_device(self.handle)
@@ -633,6 +648,12 @@ class Batch:
 
     def stats(self) -> dict:
         return pcal_batch_get_stats(self.handle).as_dict()
+
+    def fold_counts(self) -> dict:
+        """Fold kernels launched so far, by kind (a replayed step counts as its fold)."""
+        f = FoldCounts()
+        _check(load().pcal_batch_get_fold_counts(self.handle, ctypes.byref(f)), "pcal_batch_get_fold_counts")
+        return f.as_dict()
 
     @property
     def schedule(self) -> dict:

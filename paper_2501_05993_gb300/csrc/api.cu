@@ -442,6 +442,12 @@ extern "C" int pcal_get_bins(pcal_plan* p, void* host_out) {
     return cuda_status(e);
 }
 
+extern "C" int pcal_get_fold_counts(const pcal_plan* p, pcal_fold_counts* out) {
+    if (!p || !out) return PCAL_EINVAL;
+    *out = p->folds;
+    return PCAL_OK;
+}
+
 extern "C" int pcal_get_stats(const pcal_plan* p, pcal_stats* out) {
     if (!p || !out) return PCAL_EINVAL;
     *out = p->stats;

@@ -622,6 +622,8 @@ struct BatchGraph {
     void* d_desc;
     unsigned long long* d_ctr;
     cudaGraphExec_t exec;
+    bool direct;  // its fold
+    int folds;    // ... launches (none without samples)
 };
 
 // Channels of one N that share a batched tone DFT: rows of P and of the
@@ -662,6 +664,7 @@ struct pcal_batch {
     cudaStream_t last_stream;
     std::vector<BatchGraph> graphs;
     pcal_stats stats;
+    pcal_fold_counts folds;
     int dft_mode;                 // PCAL_DFT_FP32: the DFT inside each channel's cluster
     std::vector<DftGroup> dft;    // tensor-core modes: one group per distinct N
     bool sched_set;               // the schedule was set or tuned: every call takes the persistent fold
@@ -1054,12 +1057,17 @@ int build_call(pcal_batch* b, const void* const* samples, const int64_t* n, cons
     return batch_build(b->h_ch.data(), b->n, regions, sh, std::vector<int>(), out);
 }
 
+void count_fold(pcal_batch* b, bool direct, int launches) {
+    (direct ? b->folds.direct : b->folds.persistent) += launches;
+}
+
 cudaError_t launch_call(pcal_batch* b, const BatchCallDesc& d, void* d_desc, unsigned long long* d_ctr,
                         const BatchShape& sh, cudaStream_t s) {
     int launches = 0;
     const cudaError_t e = batch_launch_fold(d, d_desc, b->d_ch, b->n, d_ctr, sh, b->d_err, s, &launches);
     b->stats.kernel_launches += launches;
     if (d.total_boxes > 0 || d.total_tasks > 0) b->stats.bulk_launches += 1;
+    count_fold(b, d.total_tasks > 0, launches);
     return e;
 }
 
@@ -1453,10 +1461,14 @@ extern "C" int pcal_batch_step_graph(pcal_batch* b, const void* const* samples, 
         if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             const pcal_stats keep = b->stats;
+            const pcal_fold_counts keep_folds = b->folds;
             cudaError_t el = launch_call(b, d, gr.d_desc, gr.d_ctr, sh, cap);
             int fl = 0;
             if (el == cudaSuccess) el = batch_finalize_all(b, cap, &fl);
             b->stats = keep;
+            b->folds = keep_folds;
+            gr.direct = d.total_tasks > 0;
+            gr.folds = d.total_boxes > 0 || d.total_tasks > 0 || d.n_pieces > 0;
             e = cudaStreamEndCapture(cap, &graph);
             if (el != cudaSuccess) e = el;
         }
@@ -1473,6 +1485,7 @@ extern "C" int pcal_batch_step_graph(pcal_batch* b, const void* const* samples, 
         hit = &b->graphs.back();
     }
     if (cudaGraphLaunch(hit->exec, s) != cudaSuccess) return PCAL_ECUDA;
+    count_fold(b, hit->direct, hit->folds);
     b->last_stream = s;
     for (int c = 0; c < b->n; ++c) {
         b->n_abs[c] += n[c];
@@ -1556,6 +1569,12 @@ extern "C" int pcal_batch_get_bins(pcal_batch* b, int channel, int64_t* host_out
         host_out[4 * k + 1] = sl - shl;
         host_out[4 * k + 0] = cnt - sl - sh + shl;
     }
+    return PCAL_OK;
+}
+
+extern "C" int pcal_batch_get_fold_counts(const pcal_batch* b, pcal_fold_counts* out) {
+    if (!b || !out) return PCAL_EINVAL;
+    *out = b->folds;
     return PCAL_OK;
 }
 

@@ -978,6 +978,7 @@ cudaError_t launch_bulk(pcal_plan* p, const void* d_rows, int64_t n_rows, int64_
         p->pending[p->n_pending++] = PartSlot{a.partf, (int64_t)t.row_groups, k_a};
         *launched = 1;
         p->stats.kernel_launches += 1;
+        p->folds.bulk += 1;
         return cudaSuccess;
     }
     const bool with_edges = a.edges.n[0] + a.edges.n[1] > 0;
@@ -985,6 +986,7 @@ cudaError_t launch_bulk(pcal_plan* p, const void* d_rows, int64_t n_rows, int64_
     if (e == cudaSuccess) {
         *launched = 1;
         p->stats.kernel_launches += 1;
+        p->folds.bulk += 1;
     } else {
         unpublish_hint(p, a.epoch);
     }

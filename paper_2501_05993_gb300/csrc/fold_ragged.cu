@@ -270,6 +270,7 @@ cudaError_t launch_ragged_f32(pcal_plan* p, const uint8_t* d0, int64_t n0, int64
     const int64_t L = p->g.L;
     const FloatRun r0{reinterpret_cast<const float*>(d0), n0, k0 % L}, r1{reinterpret_cast<const float*>(d1), n1, k1 % L};
     p->stats.kernel_launches += 1;
+    p->folds.ragged += 1;
     return launch_chained(ragged_f32_kernel, (int)((L + 255) / 256), 256, s, 0, r0, r1, L, cur_accf(p));
 }
 
@@ -291,12 +292,14 @@ cudaError_t launch_ragged(pcal_plan* p, const uint8_t* d_bytes, int64_t n, int64
         default: return launch_ragged_f32(p, d_bytes, n, k0, nullptr, 0, 0, s);
     }
     p->stats.kernel_launches += 1;
+    p->folds.ragged += 1;
     return e;
 }
 
 cudaError_t launch_short(pcal_plan* p, const uint8_t* d, int64_t n, int64_t k0, cudaStream_t s) {
     using namespace pcal_direct;
     const int64_t L = p->g.L;
+    p->folds.short_folds += 1;
     if (p->g.format == PCAL_F32) {
         // a warp per eight periods (its loads in flight together), at most eight,
         // or 32 where each would still take many

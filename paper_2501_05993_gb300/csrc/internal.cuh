@@ -132,6 +132,7 @@ struct pcal_plan {
     cudaStream_t copy_stream;     // H2D copies of pcal_accumulate_host
     bool results_valid;
     pcal_stats stats;
+    pcal_fold_counts folds;
     BulkMapEntry map_cache[kBulkMapCache];
     int map_next;
 };

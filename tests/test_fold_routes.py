@@ -1,0 +1,131 @@
+"""Which fold takes a call (Plan.fold_counts, Batch.fold_counts), on both sides of the lines between them, and the
+bulk fold of long float32 periods, whose partial sums go through four slots and a reduction with one thread per bin."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+MHZ = 1_000_000
+
+
+@pytest.fixture(scope="module")
+def pcal():
+    import torch
+
+    from paper_2501_05993_gb300 import build as libbuild
+
+    libbuild.build()
+    import paper_2501_05993_gb300 as pkg
+
+    pkg.load()
+    torch.cuda.set_device(0)
+    return pkg
+
+
+def counts(**kw):
+    return dict({"bulk": 0, "short_folds": 0, "ragged": 0, "persistent": 0, "direct": 0}, **kw)
+
+
+# fmt, fs, f_offset, samples, byte offset, folds
+ROUTES = [
+    ("i8", 64 * MHZ, 10_000, 8_191, 0, counts(ragged=1)),                # under 8 KB
+    ("i8", 64 * MHZ, 10_000, 8_192, 0, counts(short_folds=1)),
+    ("2bit", 64 * MHZ, 10_000, 640_000, 3, counts(short_folds=1)),       # 10 ms
+    ("f32", 16 * MHZ, 10_000, 160_000, 4, counts(short_folds=1)),
+    ("2bit", 64 * MHZ, 10_000, 4 * 1_100_000, 1, counts(bulk=1)),        # 1 MB of rows, edges inside
+    ("i8", 64 * MHZ, 10_000, 1_100_000, 0, counts(bulk=1)),
+    ("f32", 64 * MHZ, 10_000, 256 * 6_400, 0, counts(short_folds=1)),    # at most 256 periods
+    ("f32", 64 * MHZ, 10_000, 257 * 6_400 + 1, 0, counts(bulk=1, ragged=1)),
+    ("i8", 256 * MHZ, 7_000, 128 * 256_000, 0, counts(short_folds=1)),   # at most 128 wide rows
+    ("i8", 256 * MHZ, 7_000, 129 * 256_000, 0, counts(bulk=1)),
+]
+
+
+@pytest.mark.parametrize("route", ROUTES, ids=[f"{r[0]}-L{r[1] // np.gcd.reduce([r[1], MHZ, r[2]])}-{r[3]}" for r in ROUTES])
+def test_fold_of_a_call(pcal, route):
+    import torch
+
+    fmt, fs, fo, n, offset, expect = route
+    nbytes = {"2bit": n // 4, "i8": n, "f32": 4 * n}[fmt]
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    if fmt == "f32":
+        buf = torch.randn(n + 8, generator=gen, device="cuda").view(torch.uint8)
+    else:
+        buf = torch.randint(0, 256, (nbytes + 32,), dtype=torch.uint8, generator=gen, device="cuda")
+    with pcal.Plan(fs, MHZ, fo, fmt) as p:
+        p.accumulate(buf.data_ptr() + offset, n)
+        assert p.fold_counts() == expect
+        bins = p.bins()
+        host = buf[offset:offset + nbytes].cpu().numpy()
+        if fmt == "2bit":
+            assert np.array_equal(bins, oracle.counts_2bit(host, 0, p.L))
+        elif fmt == "i8":
+            assert np.array_equal(bins, oracle.sums_i8(host.view(np.int8), 0, p.L))
+        else:
+            x = host.view(np.float32)
+            # compensated FP32 sums of at most 257 samples a bin: 257^2 * 2^-48 < 2^-31 of their magnitudes
+            mag = oracle.fold_real(np.abs(x), "f32", 0, p.L)
+            assert np.all(np.abs(bins - oracle.sums_f32(x, 0, p.L)) <= 2.0**-31 * mag)
+
+
+@pytest.mark.parametrize("geom", [(64 * MHZ, 10_000), (256 * MHZ, 10_000), (1024 * MHZ, 10_000), (256 * MHZ, 1_000)],
+                         ids=["L6400", "L25600", "L102400", "L256000"])
+def test_bulk_float32_of_long_periods(pcal, geom):
+    """Six bulk folds of 257 periods and a few samples each: the slots fill, are reduced, and fill again; then the
+    bins (a reduction of what is pending), and the same once more through the finalize."""
+    import torch
+
+    fs, fo = geom
+    with pcal.Plan(fs, MHZ, fo, "f32") as p:
+        L, calls = p.L, 6
+        n = 257 * L + 37
+        x = np.random.default_rng(L).standard_normal(n).astype(np.float32)
+        dev = torch.from_numpy(x).cuda()
+        for _ in range(calls):
+            p.accumulate(dev)
+        f = p.fold_counts()
+        assert f["bulk"] == calls and f["short_folds"] == 0, f
+        bins = p.bins()
+        ref, mag = np.zeros(L), np.zeros(L)
+        once, once_mag = oracle.sums_f32(x, 0, L), oracle.fold_real(np.abs(x), "f32", 0, L)
+        for c in range(2 * calls):  # (a call's bins start at its first sample's)
+            if c == calls:
+                # compensated FP32 sums of at most 258 samples a bin and call (258^2 * 2^-48 < 2^-31 of their
+                # magnitudes), added in double-float
+                assert np.all(np.abs(bins - ref) <= 2.0**-31 * mag)
+                p.finalize_device()
+                for _ in range(calls):
+                    p.accumulate(dev)
+                ref, mag = np.zeros(L), np.zeros(L)
+            ref += np.roll(once, c * n % L)
+            mag += np.roll(once_mag, c * n % L)
+        T = p.finalize()
+        want = oracle.tones_from_bins(ref, fs, MHZ, fo)
+        assert np.max(np.abs(T - want)) <= 1e-5 * np.max(np.abs(want))  # the library's bound for phasors
+
+
+def test_fold_of_a_batch(pcal):
+    import torch
+
+    chans = [(64 * MHZ, MHZ, 10_000, "2bit"), (32 * MHZ, MHZ, 30_000, "i8")]
+    n = [4 * 300_000, 500_001]
+    xs = [torch.randint(0, 256, (300_000,), dtype=torch.uint8, device="cuda"),
+          torch.randint(-128, 128, (500_001,), dtype=torch.int8, device="cuda")]
+    with pcal.Batch(chans) as b:
+        b.accumulate(xs, n)
+        assert b.fold_counts() == counts(direct=1)
+        b.finalize_device()
+        for _ in range(3):
+            b.step_graph(xs, n)
+        assert b.fold_counts() == counts(direct=4)
+        want = [b.results(c)["phasors"] for c in range(2)]
+        b.set_schedule(min_chunk=4)
+        b.accumulate(xs, n)
+        assert b.fold_counts() == counts(direct=4, persistent=1)
+        assert all(np.all(np.isfinite(w)) for w in want)
+    with pcal.Batch(chans) as b:
+        b.accumulate(xs, [0, 0])  # no samples: no fold
+        b.step_graph(xs, [0, 0])
+        assert b.fold_counts() == counts()
