@@ -261,7 +261,7 @@ int pcal_get_fold_counts(const pcal_plan* plan, pcal_fold_counts* out);
  * Work split of the bulk fold kernel (host only, no CUDA call), for tests and
  * diagnostics: how `n_rows` rows of `row_samples` samples are tiled over
  * `num_sms` SMs for a plan with these parameters.  PCAL_EINVAL when no tile
- * plan exists (such inputs are folded by the ragged kernel instead).
+ * plan exists (such inputs take a short fold instead).
  */
 typedef struct {
     int32_t cols_total, col_width, col_groups, replicas, box_rows, stages;

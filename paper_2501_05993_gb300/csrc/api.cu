@@ -13,7 +13,7 @@ namespace {
 // Inputs of fewer bytes in whole rows go through a short fold (or, a few KB, the
 // ragged kernel) alone: the bulk kernel's fixed cost does not pay off below it.
 constexpr int64_t kBulkMinBytes = 1 << 20;
-constexpr int64_t kShortMinBytes = 8 << 10, kShortMaxBytes = 1 << 28;
+constexpr int64_t kShortMinBytes = 8 << 10, kShortFloatBytes = 6 << 20;
 constexpr int64_t kShortPeriods = 256, kShortRows = 128;
 constexpr size_t kStageBytes = 64ull << 20;
 
@@ -88,22 +88,31 @@ int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
     int64_t rows = (n - head) / row;
     if (bytes_of(p, rows * row) < kBulkMinBytes) rows = 0;
     BulkTiling probe;
-    if (rows > 0 && bulk_tiling(p, rows, &probe) != 0) rows = 0;  // no tile plan: short or ragged only
+    if (rows > 0 && bulk_tiling(p, rows, &probe) != 0) rows = 0;  // no tile plan: a short fold
     // Few rows, each wider than the SMs have column groups for (long periods):
-    // the bulk kernel's CTAs would come in waves with a box or two each.  A step
-    // of L 1,024,000 int8: 3 MB 99 -> 69 us, 128 MB (125 rows) 112 -> 83; 2-bit 64 MB
-    // (250 rows) the same either way.  float32 (also no partials then): L 25,600
-    // 16 MB (156 periods) 33 -> 29 us, 32 MB 34 -> 32, 64 MB 28 -> 42; L 6,400 3 MB
-    // 14.8 -> 12.0, 8 MB (312) 16.0 -> 16.2; L 256,000 32 MB 96 -> 51.
-    const bool wide = rows > 0 && (p->g.format == PCAL_F32 ? n <= kShortPeriods * L
-                                                           : rows <= kShortRows && probe.col_groups > p->num_sms);
+    // the bulk kernel's CTAs come in waves with a box or two each, and int8 and
+    // float32 take a short fold.  Steps in us, bulk against short: int8 L 1,024,000
+    // 64 MB 89 / 74, 128 MB (125 rows) 97 / 81; L 390,625 64 MB 178 / 79, 300 MB 204 / 89,
+    // 760 MB 288 / 164; L 140,625 260 MB (115 rows) 132 / 90; L 512,000 64 MB (125 rows)
+    // 55 / 48.  float32 (no partials to reduce then) L 50,000 128 periods 36 / 35, 256 39 / 41;
+    // L 102,400 256 periods 61 / 60, 320 64 / 65; L 256,000 256 periods 125 / 92; L 1,024,000
+    // 256 periods (1 GB) 352 / 289; L 703,125 64 periods 398 / 191.
+    // float32 rows of fewer groups leave the bulk kernel less to wait for: L 6,400
+    // 5 MB 13.9 / 13.6, 6.6 MB 14.4 / 14.5, 8 MB 14.2 / 15.6; L 12,800 6.6 MB 20.1 / 19.1, 9.8 MB
+    // 20.0 / 20.6; L 25,600 6.6 MB 27.6 / 27.2, 13 MB 27.7 / 28.8, 26 MB 28.7 / 31.8.
+    // 2-bit rows go either way (L 140,625 64 MB 141 / 167, 200 MB 223 / 214; L 390,625 128 MB
+    // 317 / 376, 300 MB 306 / 284; L 1,024,000 16 MB 78 / 82): they stay with the bulk kernel.
+    const bool many_groups = rows > 0 && probe.col_groups > p->num_sms;
+    bool wide = false;
+    if (rows > 0 && p->g.format == PCAL_F32)
+        wide = n <= kShortPeriods * L && (many_groups || 4 * n <= kShortFloatBytes);
+    else if (p->g.format == PCAL_I8)
+        wide = many_groups && rows <= kShortRows;
     if (wide) rows = 0;
     cudaError_t e = cudaSuccess;
     if (rows == 0) {
-        // a few KB: one sample a thread does (and so would an input without a tile plan)
-        const int64_t b = bytes_of(p, n);
-        const bool few = b < kShortMinBytes || (p->g.format != PCAL_F32 && b >= kShortMaxBytes);
-        e = few ? launch_ragged(p, d, n, k0, s) : launch_short(p, d, n, k0, s);
+        // a few KB: one sample a thread does
+        e = bytes_of(p, n) < kShortMinBytes ? launch_ragged(p, d, n, k0, s) : launch_short(p, d, n, k0, s);
         if (e == cudaSuccess && wide) p->stats.bulk_launches += 1;
     } else {
         const uint8_t* body = d + bytes_of(p, head);

@@ -36,8 +36,14 @@ ROUTES = [
     ("f32", 16 * MHZ, 10_000, 160_000, 4, counts(short_folds=1)),
     ("2bit", 64 * MHZ, 10_000, 4 * 1_100_000, 1, counts(bulk=1)),        # 1 MB of rows, edges inside
     ("i8", 64 * MHZ, 10_000, 1_100_000, 0, counts(bulk=1)),
-    ("f32", 64 * MHZ, 10_000, 256 * 6_400, 0, counts(short_folds=1)),    # at most 256 periods
+    ("f32", 64 * MHZ, 10_000, 245 * 6_400, 0, counts(short_folds=1)),
     ("f32", 64 * MHZ, 10_000, 257 * 6_400 + 1, 0, counts(bulk=1, ragged=1)),
+    ("f32", 256 * MHZ, 10_000, 61 * 25_600, 0, counts(short_folds=1)),   # up to 6 MB where the rows fit the SMs
+    ("f32", 256 * MHZ, 10_000, 62 * 25_600, 0, counts(bulk=1)),
+    ("f32", 64 * MHZ, 10_000, 246 * 6_400, 0, counts(bulk=1)),
+    ("f32", 256 * MHZ, 7_000, 256 * 256_000, 0, counts(short_folds=1)),  # at most 256 periods of wider rows
+    ("f32", 256 * MHZ, 7_000, 257 * 256_000, 0, counts(bulk=1)),
+    ("2bit", 1024 * MHZ, 7_000, 4 * 18 * 256_000, 0, counts(bulk=1)),    # wide 2-bit rows all the same
     ("i8", 256 * MHZ, 7_000, 128 * 256_000, 0, counts(short_folds=1)),   # at most 128 wide rows
     ("i8", 256 * MHZ, 7_000, 129 * 256_000, 0, counts(bulk=1)),
 ]
@@ -68,6 +74,48 @@ def test_fold_of_a_call(pcal, route):
             # compensated FP32 sums of at most 257 samples a bin: 257^2 * 2^-48 < 2^-31 of their magnitudes
             mag = oracle.fold_real(np.abs(x), "f32", 0, p.L)
             assert np.all(np.abs(bins - oracle.sums_f32(x, 0, p.L)) <= 2.0**-31 * mag)
+
+
+# fmt, fs, f_offset (L 390625, 140625 and 703125: rows of 6.25, 2.25 and 11.25 MB), samples, fold
+LARGE = [
+    ("i8", 25 * MHZ, 64, 300_000_007, "short_folds"),      # 256 MB and more of few wide rows
+    ("i8", 1125 * MHZ, 8_000, 270_000_000, "short_folds"),
+    ("i8", 25 * MHZ, 64, 130 * 6_250_000, "bulk"),
+    ("i8", 45 * MHZ, 64, 130 * 11_250_000, "bulk"),        # 10,987 column groups
+    ("f32", 45 * MHZ, 64, 257 * 703_125, "bulk"),
+    ("f32", 45 * MHZ, 64, 256 * 703_125, "short_folds"),
+]
+
+
+@pytest.mark.parametrize("case", LARGE, ids=[f"{c[0]}-{c[3]}" for c in LARGE])
+def test_large_calls_of_wide_rows(pcal, case):
+    import torch
+
+    fmt, fs, fo, n, fold = case
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    if fmt == "i8":
+        x = torch.randint(-128, 128, (n + 3,), dtype=torch.int8, generator=gen, device="cuda")[3:]
+    else:
+        x = torch.randn(n, generator=gen, device="cuda")
+    with pcal.Plan(fs, MHZ, fo, fmt) as p:
+        p.accumulate(x.data_ptr(), n)
+        f = p.fold_counts()
+        assert f[fold] == 1 and f["bulk"] + f["short_folds"] - f[fold] <= (fold == "bulk"), f  # (its tail: a short fold)
+        assert f["ragged"] <= 2
+        bins, L = torch.from_numpy(p.bins()).cuda(), p.L
+
+    def fold_of(v, dtype):
+        s = torch.zeros(L, dtype=dtype, device="cuda")
+        for at in range(0, n // L * L, 32 * L):
+            s += v[at:min(at + 32 * L, n // L * L)].view(-1, L).sum(0, dtype=dtype)
+        s[:n % L] += v[n // L * L:].to(dtype)
+        return s
+
+    if fmt == "i8":
+        assert torch.equal(bins, fold_of(x, torch.int64))
+    else:
+        # compensated FP32 sums of at most 257 samples a bin: 257^2 * 2^-48 < 2^-31 of their magnitudes
+        assert bool(torch.all((bins - fold_of(x, torch.float64)).abs() <= 2.0**-31 * fold_of(x.abs(), torch.float64)))
 
 
 @pytest.mark.parametrize("geom", [(64 * MHZ, 10_000), (256 * MHZ, 10_000), (1024 * MHZ, 10_000), (256 * MHZ, 1_000)],
