@@ -365,6 +365,8 @@ typedef struct pcal_batch pcal_batch;
 int pcal_batch_create(const pcal_channel_desc* channels, int n_channels, pcal_batch** out);
 int pcal_batch_destroy(pcal_batch* batch);
 int pcal_batch_get_geometry(const pcal_batch* batch, int channel, pcal_geometry* out);
+/* Takes effect with the next call; a schedule other than the current one drops
+ * captured step graphs (and synchronises the device if there are any). */
 int pcal_batch_set_schedule(pcal_batch* batch, const pcal_schedule* sched);
 /* How the batch finalize runs the tone DFT (the PCAL_DFT_* modes of the
  * batched tone DFT below): PCAL_DFT_FP32 (default) inside each channel's
@@ -395,7 +397,7 @@ int pcal_batch_finalize_device(pcal_batch* batch, void* stream);
  * pcal_batch_accumulate + pcal_batch_finalize_device as one CUDA graph: the
  * first call with a given set of (samples, n) captures the step, later calls
  * with the same pointers and counts replay it (the buffers' contents may
- * change).  Every per-step quantity lives on the device, so replays continue
+ * change; a change of the schedule or of the DFT mode captures anew).  Every per-step quantity lives on the device, so replays continue
  * the channels' sample indices correctly.  Asynchronous.
  */
 int pcal_batch_step_graph(pcal_batch* batch, const void* const* samples, const int64_t* n, void* stream);

@@ -1171,6 +1171,19 @@ extern "C" int pcal_batch_create(const pcal_channel_desc* channels, int n_channe
 
 namespace {
 
+// Captured steps hold the fold, the schedule and the finalize of their time.
+int drop_graphs(pcal_batch* b) {
+    if (b->graphs.empty()) return PCAL_OK;
+    if (cudaDeviceSynchronize() != cudaSuccess) return PCAL_ECUDA;
+    for (BatchGraph& gr : b->graphs) {
+        cudaGraphExecDestroy(gr.exec);
+        cudaFree(gr.d_desc);
+        cudaFree(gr.d_ctr);
+    }
+    b->graphs.clear();
+    return PCAL_OK;
+}
+
 void free_dft_groups(pcal_batch* b) {
     for (DftGroup& g : b->dft) {
         pcal_dft_destroy(g.dft);
@@ -1203,13 +1216,8 @@ extern "C" int pcal_batch_set_dft(pcal_batch* b, int mode) {
     if (mode != PCAL_DFT_FP32 && mode != PCAL_DFT_TC_TF32X3 && mode != PCAL_DFT_TC_BF16X6) return PCAL_EINVAL;
     if (mode == b->dft_mode) return PCAL_OK;
     if (cudaDeviceSynchronize() != cudaSuccess) return PCAL_ECUDA;
-    // captured steps hold the old finalize
-    for (BatchGraph& gr : b->graphs) {
-        cudaGraphExecDestroy(gr.exec);
-        cudaFree(gr.d_desc);
-        cudaFree(gr.d_ctr);
-    }
-    b->graphs.clear();
+    const int dropped = drop_graphs(b);
+    if (dropped != PCAL_OK) return dropped;
     free_dft_groups(b);
     for (BatchChan& c : b->h_ch) c.Pslot = c.Tslot = nullptr;
     int rc = PCAL_OK;
@@ -1312,8 +1320,9 @@ extern "C" int pcal_batch_set_schedule(pcal_batch* b, const pcal_schedule* s) {
         apply_col_caps(b, old);
         return PCAL_EINVAL;
     }
+    const bool same = b->sched_set && memcmp(s, &old, sizeof(old)) == 0;
     b->sched_set = true;
-    return PCAL_OK;
+    return same ? PCAL_OK : drop_graphs(b);
 }
 
 extern "C" int pcal_batch_channel_tiling(const pcal_batch* b, int channel, int* bucket, int* col_width,
@@ -1700,7 +1709,10 @@ extern "C" int pcal_batch_autotune(pcal_batch* b, const void* const* samples, co
     if (e != cudaSuccess) return PCAL_ECUDA;
     if (rc != PCAL_OK) return rc;
     rc = pcal_batch_set_schedule(b, &best_s);
-    if (rc == PCAL_OK && direct_ms >= 0.f && direct_ms <= best) b->sched_set = false;
+    if (rc == PCAL_OK && direct_ms >= 0.f && direct_ms <= best) {
+        b->sched_set = false;
+        rc = drop_graphs(b);
+    }
     if (rc == PCAL_OK && chosen) *chosen = best_s;
     return rc;
 }

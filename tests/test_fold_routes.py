@@ -177,3 +177,38 @@ def test_fold_of_a_batch(pcal):
         b.accumulate(xs, [0, 0])  # no samples: no fold
         b.step_graph(xs, [0, 0])
         assert b.fold_counts() == counts()
+
+
+def test_captured_steps_follow_the_schedule(pcal):
+    """A step that was captured before its batch's schedule changed is captured again: it runs the new fold, with the
+    same exact bins and so the same phasors."""
+    import torch
+
+    chans = [(64 * MHZ, MHZ, 10_000, "2bit"), (32 * MHZ, MHZ, 30_000, "i8")]
+    n = [64 * 80_000, 32 * 20_000]  # whole periods: every step's phasors are the first one's
+    xs = [torch.randint(0, 256, (n[0] // 4,), dtype=torch.uint8, device="cuda"),
+          torch.randint(-128, 128, (n[1],), dtype=torch.int8, device="cuda")]
+    with pcal.Batch(chans) as b:
+        def step():
+            before = b.fold_counts()
+            b.step_graph(xs, n)
+            torch.cuda.synchronize()
+            now = b.fold_counts()
+            got = [b.results(c)["phasors"] for c in range(2)]
+            return {k for k in now if now[k] != before[k]}, got
+
+        kind, want = step()
+        assert kind == {"direct"}
+        for kw in (dict(min_chunk=4), dict(box_rows=64), dict(box_rows=64)):
+            b.set_schedule(**kw)
+            kind, got = step()
+            assert kind == {"persistent"}
+            assert all(np.array_equal(x, y) for x, y in zip(got, want))
+        b.autotune(xs, n)
+        kind, got = step()
+        b.accumulate(xs, n)  # the fold of an uncaptured call is the one that autotune kept
+        last = b.fold_counts()
+        b.accumulate(xs, n)
+        now = b.fold_counts()
+        assert kind == {k for k in now if now[k] != last[k]}
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
