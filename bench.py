@@ -90,9 +90,10 @@ def read_peaks():
         return 6800.0, "fallback"
 
 
-def read_batch_traffic_ratio():
-    """DRAM bytes per sample byte of the batched fold from its committed ncu
-    summary (captured on a reduced batch), or None when batch.cu changed."""
+def read_batch_traffic_ratio(fold: str = "schedule"):
+    """DRAM bytes per sample byte of the batched fold that runs ("direct" or
+    "schedule", the persistent one) from its committed ncu summary (captured
+    on a reduced batch), or None when batch.cu changed."""
     import hashlib
 
     try:
@@ -101,7 +102,7 @@ def read_batch_traffic_ratio():
         src = open(os.path.join(ROOT, "paper_2501_05993_gb300", "csrc", "batch.cu"), "rb").read()
         if kv.get("source_sha256", "").strip() != hashlib.sha256(src).hexdigest():
             return None
-        return float(kv["traffic_per_algorithmic_byte"])
+        return float(kv[("direct_" if fold == "direct" else "") + "traffic_per_algorithmic_byte"])
     except Exception:
         return None
 
@@ -617,6 +618,7 @@ def run_batch(args, emit=True):
     total_bytes = sum(b.numel() for b in bufs)
     stream = torch.cuda.current_stream()
     chosen = batch.autotune(ptrs, n, stream)
+    fold = batch.fold  # the one that the autotuner kept
 
     def ev():
         return torch.cuda.Event(enable_timing=True)
@@ -718,12 +720,12 @@ def run_batch(args, emit=True):
 
     peak, peak_kind = read_peaks()
     achieved = total_bytes / (fold_ms / 1e3) / 1e9
-    ratio = read_batch_traffic_ratio()
+    ratio = read_batch_traffic_ratio(fold)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": int(ratio * total_bytes) if ratio else None,
                 "traffic_note": "scaled from a reduced batch capture (profiles/batch_fold_mixed.txt)",
                 "peak_kind": f"{peak_kind} (copy bandwidth)",
-                "kernel": "batch_fold_kernel or batch_direct_kernel (the faster in the autotuner)",
+                "kernel": {"schedule": "batch_fold_kernel", "direct": "batch_direct_kernel"}[fold],
                 "algorithmic_bytes_per_launch": total_bytes}
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline:  # the host baseline: N = 1 only
@@ -756,7 +758,7 @@ def run_batch(args, emit=True):
             "vs_baseline": None, "dtype": "u32", "data": "synthetic",
             "config": {"workload": BATCH_WORKLOAD, "channels": len(chans), "two_bit_channels": n2,
                        "samples_per_step": total_samples, "bytes_per_step": total_bytes,
-                       "max_L": max(int(g.L) for g in batch.geometry), "schedule": chosen,
+                       "max_L": max(int(g.L) for g in batch.geometry), "fold": fold, "schedule": chosen,
                        "parallelism": f"replicas x{world}" if world > 1 else "single GPU",
                        "l2": f"{total_bytes / 1e9:.2f} GB of inputs per step > L2",
                        "fold_ms": fold_ms, "batched_vs_plain_max_phasor_diff": worst,

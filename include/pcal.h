@@ -335,7 +335,7 @@ typedef struct {
 
 /* Launch schedule of the persistent fold, which takes the calls of a batch once
  * a schedule was set (or pcal_batch_autotune found one faster than the fold
- * without a schedule that takes them otherwise; it picks one all the same).
+ * without a schedule that takes them otherwise: pcal_batch_get_fold).
  * A channel's tile is a column group of its rows (one row = a whole number of
  * periods L); its width is capped by the channel's bucket -- sample format x
  * row width -- or, where the bucket's cap is 0, by col_cap.  Bucket index =
@@ -375,8 +375,18 @@ int pcal_batch_set_schedule(pcal_batch* batch, const pcal_schedule* sched);
  * clusters stop at P, then a products kernel finishes every channel).
  * Synchronises the device; drops captured step graphs. */
 int pcal_batch_set_dft(pcal_batch* batch, int mode);
+/* The schedule of the persistent fold: it runs while pcal_batch_get_fold says PCAL_FOLD_SCHEDULE. */
 int pcal_batch_get_schedule(const pcal_batch* batch, pcal_schedule* out);
-/* The tile a channel's rows are cut into under the current schedule (host only): its bucket (the
+/* Which fold takes a batch's calls: PCAL_FOLD_DIRECT, the fold without a
+ * schedule (the one a batch starts with), or PCAL_FOLD_SCHEDULE, the
+ * persistent fold under the current schedule.  pcal_batch_set_schedule and
+ * pcal_batch_set_fold choose it, and pcal_batch_autotune keeps the faster.  A
+ * change drops captured step graphs, as pcal_batch_set_schedule does. */
+#define PCAL_FOLD_DIRECT 0
+#define PCAL_FOLD_SCHEDULE 1
+int pcal_batch_get_fold(const pcal_batch* batch, int* fold);
+int pcal_batch_set_fold(pcal_batch* batch, int fold);
+/* The tile a channel's rows are cut into by the persistent fold under the current schedule (host only): its bucket (the
  * index into col_cap_bucket), the column-group width in 32-bit words and the number of groups. */
 int pcal_batch_channel_tiling(const pcal_batch* batch, int channel, int* bucket, int* col_width, int* col_groups);
 
@@ -428,8 +438,9 @@ int pcal_batch_get_fold_counts(const pcal_batch* batch, pcal_fold_counts* out);
 
 /*
  * Time candidate schedules on these inputs, accumulate only, and keep the
- * fastest; writes it to *chosen when not NULL.  Where the fold without a
- * schedule is at least as fast, calls go on to take that.  Three passes: the batch-wide
+ * fastest; writes it to *chosen when not NULL.  The fold without a schedule is
+ * timed too, and takes the calls where it is at least as fast
+ * (pcal_batch_get_fold).  Three passes: the batch-wide
  * choices (column-width cap, box rows, static share, chunk size; the four
  * fastest timed again), then the CTA count (one per SM, or 8 or 16 fewer),
  * then, one bucket at a time for the buckets the batch's channels occupy, the

@@ -79,6 +79,7 @@ class Schedule(ctypes.Structure):
 
 
 PCAL_MAX_BATCH, PCAL_BATCH_MAX_N = 4096, 1024
+FOLDS = ("direct", "schedule")  # PCAL_FOLD_*
 
 
 class ServerConfig(ctypes.Structure):
@@ -160,6 +161,8 @@ def load(path: str | None = None):
         "pcal_batch_read_post": ([vp, ci, vp, vp, vp], ci),
         "pcal_batch_get_bins": ([vp, ci, vp], ci),
         "pcal_batch_get_stats": ([vp, P(Stats)], ci),
+        "pcal_batch_get_fold": ([vp, P(ci)], ci),
+        "pcal_batch_set_fold": ([vp, ci], ci),
         "pcal_batch_get_fold_counts": ([vp, P(FoldCounts)], ci),
         "pcal_batch_autotune": ([vp, P(vp), P(i64), vp, P(Schedule)], ci),
         "pcal_server_stream_bytes": ([P(ServerConfig), P(ChannelDesc), P(i64)], ci),
@@ -670,6 +673,16 @@ class Batch:
             else:
                 setattr(s, k, int(v))
         pcal_batch_set_schedule(self.handle, s)
+
+    @property
+    def fold(self) -> str:
+        """The fold that takes the calls: "direct", or "schedule" (the persistent one under `schedule`)."""
+        f = ctypes.c_int()
+        _check(load().pcal_batch_get_fold(self.handle, ctypes.byref(f)), "pcal_batch_get_fold")
+        return FOLDS[f.value]
+
+    def set_fold(self, fold: str):
+        _check(load().pcal_batch_set_fold(self.handle, FOLDS.index(fold)), "pcal_batch_set_fold")
 
     def channel_tiling(self, channel: int) -> dict:
         """The bucket, column-group width (32-bit words) and group count of a channel's rows."""

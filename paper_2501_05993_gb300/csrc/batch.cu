@@ -1325,6 +1325,20 @@ extern "C" int pcal_batch_set_schedule(pcal_batch* b, const pcal_schedule* s) {
     return same ? PCAL_OK : drop_graphs(b);
 }
 
+extern "C" int pcal_batch_get_fold(const pcal_batch* b, int* fold) {
+    if (!b || !fold) return PCAL_EINVAL;
+    *fold = b->sched_set ? PCAL_FOLD_SCHEDULE : PCAL_FOLD_DIRECT;
+    return PCAL_OK;
+}
+
+extern "C" int pcal_batch_set_fold(pcal_batch* b, int fold) {
+    if (!b || (fold != PCAL_FOLD_DIRECT && fold != PCAL_FOLD_SCHEDULE)) return PCAL_EINVAL;
+    const bool sched = fold == PCAL_FOLD_SCHEDULE;
+    if (b->sched_set == sched) return PCAL_OK;
+    b->sched_set = sched;
+    return drop_graphs(b);
+}
+
 extern "C" int pcal_batch_channel_tiling(const pcal_batch* b, int channel, int* bucket, int* col_width,
                                          int* col_groups) {
     if (!b || channel < 0 || channel >= b->n || !bucket || !col_width || !col_groups) return PCAL_EINVAL;
@@ -1709,10 +1723,7 @@ extern "C" int pcal_batch_autotune(pcal_batch* b, const void* const* samples, co
     if (e != cudaSuccess) return PCAL_ECUDA;
     if (rc != PCAL_OK) return rc;
     rc = pcal_batch_set_schedule(b, &best_s);
-    if (rc == PCAL_OK && direct_ms >= 0.f && direct_ms <= best) {
-        b->sched_set = false;
-        rc = drop_graphs(b);
-    }
+    if (rc == PCAL_OK && direct_ms >= 0.f && direct_ms <= best) rc = pcal_batch_set_fold(b, PCAL_FOLD_DIRECT);
     if (rc == PCAL_OK && chosen) *chosen = best_s;
     return rc;
 }

@@ -212,3 +212,35 @@ def test_captured_steps_follow_the_schedule(pcal):
         now = b.fold_counts()
         assert kind == {k for k in now if now[k] != last[k]}
         assert all(np.array_equal(x, y) for x, y in zip(got, want))
+
+
+def test_the_fold_that_runs_is_the_one_reported(pcal):
+    import torch
+
+    chans = [(64 * MHZ, MHZ, 10_000, "2bit"), (32 * MHZ, MHZ, 30_000, "i8")]
+    n = [64 * 80_000, 32 * 20_000]
+    xs = [torch.randint(0, 256, (n[0] // 4,), dtype=torch.uint8, device="cuda"),
+          torch.randint(-128, 128, (n[1],), dtype=torch.int8, device="cuda")]
+    with pcal.Batch(chans) as b:
+        def runs():
+            before = b.fold_counts()
+            b.step_graph(xs, n)
+            b.accumulate(xs, n)
+            now = b.fold_counts()
+            b.finalize_device()
+            return {k: now[k] - before[k] for k in now if now[k] != before[k]}
+
+        kernel = {"direct": "direct", "schedule": "persistent"}
+        assert b.fold == "direct"
+        assert runs() == {"direct": 2}
+        for change in (lambda: b.autotune(xs, n), lambda: b.set_schedule(min_chunk=8), lambda: b.set_fold("direct"),
+                       lambda: b.set_fold("schedule"), lambda: b.autotune(xs, n)):
+            change()
+            assert runs() == {kernel[b.fold]: 2}
+        b.set_schedule(min_chunk=8)
+        assert b.fold == "schedule"
+        b.set_fold("direct")
+        assert b.fold == "direct" and b.schedule["min_chunk"] == 8
+        with pytest.raises(ValueError):
+            b.set_fold("fast")
+        assert pcal.load().pcal_batch_set_fold(b.handle, 2) == pcal.PCAL_EINVAL
