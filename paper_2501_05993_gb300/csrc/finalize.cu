@@ -1868,8 +1868,8 @@ cudaError_t launch_rot_finalize(float4* rows, int n_rows, int N, double fs, doub
     a.twN = twN;
     a.res = res;
     a.extra = res + 5 * (int64_t)N + 3;
-    const int C = cluster_size_for_device();
-    if (C == 0) return cudaErrorNotSupported;
+    // (one CTA where no larger cluster fits: slower, and all that a part of a GPU may have)
+    const int fits = cluster_size_for_device(), C = fits > 0 ? fits : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C);
     cfg.blockDim = dim3(kClusterThreads);
@@ -1888,10 +1888,11 @@ cudaError_t launch_rot_finalize(float4* rows, int n_rows, int N, double fs, doub
 }
 
 cudaError_t prepare_rot_finalize() {
-    if (cluster_size_for_device() == 0) return cudaErrorNotSupported;
+    const int C = cluster_size_for_device();
     cudaError_t e = cudaFuncSetAttribute(rot_finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)cluster_smem_bytes(kClusterBigN));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(rot_finalize_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess && C > 8)
+        e = cudaFuncSetAttribute(rot_finalize_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
