@@ -80,7 +80,7 @@ struct FinArgs {
     const long long* counts4;  // no-allocation entry: the caller's counts [L][4]
     double lev[4];             // no-allocation entry: the code levels
     const double2* tw;     // exp(-j 2 pi m/L), or
-    const int4* twi;       // (kLarge plans, batches) the same in fixed point (rotator_fixed)
+    const int4* twi;       // (integer kLarge plans, batches) the same in fixed point (rotator_fixed)
     const float2* twN;
     float4* P;     // P[b] as df re (x, y), df im (z, w)
     float2* T;     // FP32 tone phasors
@@ -166,15 +166,16 @@ __device__ __forceinline__ int2 rotator_fixed(double x) {
     return make_int2((int)(W >> kRotHalf), (int)(W & ((1ll << kRotHalf) - 1)));
 }
 
-// exp(-j*2*pi*m/L): the plan's table; NoAlloc evaluates it here.
-template <bool NoAlloc>
+// exp(-j*2*pi*m/L): the plan's table, FP64 or (FIXED) fixed point; NoAlloc
+// evaluates it here.
+template <bool NoAlloc, bool FIXED = false>
 __device__ __forceinline__ double2 rotator(const FinArgs& a, int64_t m) {
     if constexpr (NoAlloc) {
         double sn, cs;
         sincospi(2.0 * (double)m / (double)a.L, &sn, &cs);
         return make_double2(cs, -sn);
     }
-    if (a.twi) {
+    if constexpr (FIXED) {
         const int4 w = a.twi[m];
         constexpr double kHi = 1.0 / (double)(1ll << (kRotBits - kRotHalf)), kLo = 1.0 / (double)(1ll << kRotBits);
         return make_double2(fma((double)w.x, kHi, (double)w.y * kLo), fma((double)w.z, kHi, (double)w.w * kLo));
@@ -967,7 +968,9 @@ __device__ __noinline__ void tone_products_all(const FinArgs& a, uint8_t* base) 
 
 // Decode, rotate (FP64, Eq. 3) and fold residue b over m = m, m + step, ...
 // below m_end (bins k = b + m*N), clearing each bin; returns the FP64 sum.
-template <int FMT = -1>
+// FIXED: the rotators are the fixed-point table (a test of it in the loop cost
+// float32 plans of 128 tones and L 25,600 2 us of 25).
+template <int FMT, bool FIXED>
 __device__ __forceinline__ double2 fold_residue(const FinArgs& a, int b, int m, int step, int m_end) {
     double re = 0.0, im = 0.0;
     if (m >= m_end) return make_double2(0.0, 0.0);
@@ -976,7 +979,7 @@ __device__ __forceinline__ double2 fold_residue(const FinArgs& a, int b, int m, 
     int idx = mod_L(a, a.so * k);  // rotator index (f_offset/g * k) mod L
     const int kstep = step * N;
     const int istep = mod_L(a, a.so * kstep);
-    if (FMT == PCAL_2BIT && !a.spilled && !a.twi) {
+    if (FMT == PCAL_2BIT && !FIXED && !a.spilled) {
         // S = lev0*cnt + c_l*sum(l) + c_h*sum(h) + c_hl*sum(h AND l),
         // cnt = q or q + 1; the fields are below 2^21
         const double s_q = a.lev0 * (double)a.q, s_q1 = a.lev0 * (double)(a.q + 1);
@@ -1001,7 +1004,7 @@ __device__ __forceinline__ double2 fold_residue(const FinArgs& a, int b, int m, 
 #pragma unroll 1
         for (; m < m_end; m += step) {
             const double S = read_bin<false, FMT>(a, k);
-            const double2 w = rotator<false>(a, idx);
+            const double2 w = rotator<false, FIXED>(a, idx);
             re = fma(S, w.x, re);
             im = fma(S, w.y, im);
             clear_bin<FMT>(a, k);
@@ -1194,7 +1197,8 @@ __device__ __forceinline__ float4 residue_df(const FinArgs& a, int b, int m, int
                 return a.spilled ? residue_int<FMT, 1, 2>(a, b, m, step, m_end)
                                  : residue_int<FMT, 0, 4>(a, b, m, step, m_end);
         }
-        const double2 z = fold_residue<FMT>(a, b, m, step, m_end);
+        constexpr bool kFixed = FMT < 0 || (FMT != PCAL_F32 && KIND == kLarge);
+        const double2 z = fold_residue<FMT, kFixed>(a, b, m, step, m_end);
         const df dre = df_of(z.x), dim = df_of(z.y);
         return make_float4(dre.hi, dre.lo, dim.hi, dim.lo);
     }
@@ -1712,12 +1716,6 @@ static bool large_plan(const pcal_geometry& g) {
     return g.N <= kClusterBigN && (g.N > kClusterMaxN || g.L > kClusterMaxL) &&
            (g.format != PCAL_F32 || g.L <= kLargeF32L);
 }
-static bool fixed_rotators(const pcal_geometry& g) { return g.format != PCAL_F32 && large_plan(g); }
-
-cudaError_t launch_init_twiddles(pcal_plan* p, cudaStream_t s) {
-    p->stats.kernel_launches += 1;
-    return launch_rotators(fixed_rotators(p->g), p->d_tw, p->g.L, p->d_twN, p->g.N, p->g.step_comb, s);
-}
 
 namespace {
 
@@ -1807,6 +1805,17 @@ int cluster_size_for_device() {
     known[dev] = true;
     return best;
 }
+
+}  // namespace
+
+cudaError_t launch_init_twiddles(pcal_plan* p, cudaStream_t s) {
+    p->stats.kernel_launches += 1;
+    // (fixed point for the plans whose finalize is the cluster's integer decode)
+    p->fixed_tw = p->g.format != PCAL_F32 && large_plan(p->g) && cluster_size_for_device() > 0;
+    return launch_rotators(p->fixed_tw, p->d_tw, p->g.L, p->d_twN, p->g.N, p->g.step_comb, s);
+}
+
+namespace {
 
 // One cluster of C CTAs as a programmatic dependent of the preceding kernel.
 // The CTAs ask for kClusterPadSmem more shared memory than they use, so that
@@ -2002,7 +2011,7 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
         a.n_pf = p->n_pending;
         a.pf_cols = g.row_samples / g.samples_per_byte_x4;
     }
-    if (fixed_rotators(g))
+    if (p->fixed_tw)
         a.twi = static_cast<const int4*>(p->d_tw);
     else
         a.tw = static_cast<const double2*>(p->d_tw);
@@ -2015,7 +2024,8 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
     cudaError_t e = cudaErrorUnknown;
     bool done = false;
     const bool small = g.N <= kClusterMaxN && g.L <= kClusterMaxL;
-    if (small || large_plan(g)) {
+    const bool large = large_plan(g) && (g.format == PCAL_F32 || p->fixed_tw);
+    if (small || large) {
         const int C = cluster_size_for_device();
         if (C > 0) {
             p->stats.kernel_launches += 1;
@@ -2024,6 +2034,7 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
         }
     }
     if (!done) {
+        if (p->fixed_tw) return cudaErrorNotSupported;  // (its clusters fit when it was created)
         int launches = 0;
         e = launch_finalize_args<false>(a, p->num_sms, s, &launches);
         p->stats.kernel_launches += launches;

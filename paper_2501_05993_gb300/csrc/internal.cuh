@@ -108,7 +108,8 @@ struct pcal_plan {
     PartSlot pending[kPartSlots]; // slots written by folds and not yet added into the bins
     int n_pending;
     int part_next;                // slot of the next float32 fold
-    void* d_tw;                   // exp(-j 2 pi m / L), m < L: double2, or fixed-point int4 (finalize.cu: large_plan)
+    void* d_tw;                   // exp(-j 2 pi m / L), m < L: double2, or (fixed_tw) fixed-point int4
+    bool fixed_tw;
     float2* d_twN;                // exp(-j 2 pi m / N), m < N (FP32)
     double2* d_P;                 // folded rotated bins P[b], b < N (scratch)
     double2* d_T;                 // tone phasors (scratch before products)
