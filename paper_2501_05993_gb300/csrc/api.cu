@@ -127,15 +127,15 @@ int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
         if (inside) {
             edges.n[0] = (int)bytes_of(p, head);
             edges.n[1] = (int)bytes_of(p, tail);
-        } else if (f32 && head + tail > 0) {
-            e = launch_ragged_f32(p, d, head, k0, behind, tail, (k0 + done) % L, s);
-        } else if (head > 0) {
+        } else if (head > 0 && !f32) {
             e = launch_ragged(p, d, head, k0, s);
         }
         int launched = 0;
         if (e == cudaSuccess) e = launch_bulk(p, body, rows, (k0 + head) % L, inside ? &edges : nullptr, s, &launched);
         if (e == cudaSuccess) p->stats.bulk_launches += 1;
-        if (e == cudaSuccess && tail > 0 && !inside && !f32)
+        if (e == cudaSuccess && f32 && head + tail > 0)
+            e = launch_ragged_f32(p, d, head, k0, behind, tail, (k0 + done) % L, s);
+        else if (e == cudaSuccess && tail > 0 && !inside)
             e = bytes_of(p, tail) < kShortMinBytes ? launch_ragged(p, behind, tail, (k0 + done) % L, s)
                                                    : launch_short(p, behind, tail, (k0 + done) % L, s);
     }
