@@ -155,15 +155,17 @@ __global__ void __launch_bounds__(pcal_direct::kDirectThreads) short_fold_kernel
         });
 }
 
-// float32: a CTA owns 32 bins; its warps take the periods in turn (eight loads
-// in flight each), sum in double-float, and the warps' sums are added in order
-// to the bins.  Deterministic: nothing depends on timing.
+// float32: blockDim.y groups of warps, 32 bins each; a group's warps take the
+// periods in turn (eight loads in flight each), sum in double-float, and the
+// warps' sums are added in order to the bins.  Deterministic: nothing depends
+// on timing.
 __global__ void __launch_bounds__(1024) short_f32_kernel(const float* __restrict__ x, int64_t n, int64_t k0, int64_t L,
                                                          float2* __restrict__ acc) {
     __shared__ float2 s_sum[32][32];
     chain_in();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    const int64_t c = (int64_t)blockIdx.x * 32 + lane;  // place within a period of the run
+    float2(*const sums)[32] = s_sum + threadIdx.y * warps;
+    const int64_t c = ((int64_t)blockIdx.x * blockDim.y + threadIdx.y) * 32 + lane;  // place within a period of the run
     pcal_df::df s{0.f, 0.f};
     if (c < L) {
         const int64_t step = (int64_t)warps * L;
@@ -182,12 +184,12 @@ __global__ void __launch_bounds__(1024) short_f32_kernel(const float* __restrict
         for (int u = 0; u < 7; ++u)
             if (t + u * step < n) s = pcal_df::add_f(s, v[u]);
     }
-    s_sum[warp][lane] = make_float2(s.hi, s.lo);
+    sums[warp][lane] = make_float2(s.hi, s.lo);
     __syncthreads();
     if (warp == 0 && c < L && c < n) {
-        const int64_t k = (k0 + c) % L;
+        const int64_t k = k0 + c < L ? k0 + c : k0 + c - L;
         const float2 a = acc[k];
-        for (int w = 1; w < warps; ++w) s = pcal_df::add(s, pcal_df::df{s_sum[w][lane].x, s_sum[w][lane].y});
+        for (int w = 1; w < warps; ++w) s = pcal_df::add(s, pcal_df::df{sums[w][lane].x, sums[w][lane].y});
         s = pcal_df::add(pcal_df::df{a.x, a.y}, s);
         acc[k] = make_float2(s.hi, s.lo);
     }
@@ -242,10 +244,10 @@ __global__ void wait_timeout_kernel(uint64_t limit_ns, unsigned int* flags) {
 
 // Launch with programmatic stream serialization (see chain_in).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*k)(KArgs...), int grid, int block, cudaStream_t s, size_t smem, Args&&... args) {
+cudaError_t launch_chained(void (*k)(KArgs...), int grid, dim3 block, cudaStream_t s, size_t smem, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
+    cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -305,8 +307,12 @@ cudaError_t launch_short(pcal_plan* p, const uint8_t* d, int64_t n, int64_t k0, 
         // or 32 where each would still take many
         const int64_t periods = (n + L - 1) / L;
         const int warps = periods > 512 ? 32 : periods > 56 ? 8 : (int)((periods + 7) / 8);
+        // CTAs of up to eight warps, for the bins that the run reaches (a CTA of one
+        // warp for every 32 bins of the period: 32 us for 1 of its 1,000,000 bins' periods)
+        const int groups = warps < 8 ? 8 / warps : 1;
+        const int64_t places = n < L ? n : L, per_cta = 32 * groups;
         p->stats.kernel_launches += 1;
-        return launch_chained(short_f32_kernel, (int)((L + 31) / 32), 32 * warps, s, 0,
+        return launch_chained(short_f32_kernel, (int)((places + per_cta - 1) / per_cta), dim3(32 * warps, groups), s, 0,
                               reinterpret_cast<const float*>(d), n, k0, L, cur_accf(p));
     }
     const int spb = p->g.format == PCAL_2BIT ? 4 : 1;  // samples per byte
