@@ -10,8 +10,8 @@
 
 namespace {
 
-// Inputs of fewer bytes in whole rows go through a short fold (or, a few KB, the
-// ragged kernel) alone: the bulk kernel's fixed cost does not pay off below it.
+// Inputs of fewer bytes in whole rows go through a short fold (or the ragged
+// kernel: few_samples) alone: the bulk kernel's fixed cost does not pay off below it.
 constexpr int64_t kBulkMinBytes = 1 << 20;
 constexpr int64_t kShortMinBytes = 8 << 10, kShortFloatBytes = 6 << 20;
 constexpr int64_t kShortPeriods = 256, kShortRows = 128;
@@ -77,6 +77,29 @@ int64_t samples_of(const pcal_plan* p, int64_t b) {
     }
 }
 
+// Whether a run goes to the ragged kernel: one sample (2-bit: byte) a thread, or
+// float32 one bin.
+//   2-bit, int8  runs of fewer than three whole rows, where a short fold has next to
+//                nothing to add up before its atomics.  Accumulates, ragged / short:
+//                2-bit L 1,024,000 4M samples 13.7 / 17.8 us, L 256,000 640,000 (2.5 rows) 4.5 / 5.3,
+//                800,000 (3.1) 4.7 / 4.1; int8 L 1,024,000 1M 3.8 / 6.3; and without a whole
+//                row (a row of an odd L is 64 or 16 periods) 2-bit L 390,625 4M 10.6 / 34,
+//                int8 11 / 20.  Beyond that while few atomics meet in a bin and the run is
+//                short: 2-bit steps L 6,400 30 KB 12.4 / 13.0, 40 KB 12.8 / 12.9, 60 KB 13.6 / 12.9,
+//                L 1,600 20 KB (50 periods) 11.5 / 11.9, 30 KB 12.3 / 11.9; int8 L 3,200 240 KB
+//                10.9 / 11.2, L 6,400 400 KB 12.3 / 12.2, L 1,600 160 KB (100 periods) 11.2 / 12.0,
+//                400 KB 12.3 / 11.6, L 256 24 KB (94) 17.9 / 18.3, 64 KB (250) 18.8 / 18.3.
+//   float32      up to four periods: steps L 256,000 4 MB 35.5 / 41.7, L 200,000 0.8 MB 28.3 /
+//                31.7, L 64,000 1 MB 20.4 / 20.9, six periods 40 / 40; not for the longest,
+//                whose every bin gets a thread (L 1,000,000 80 KB 82 / 67).
+bool few_samples(const pcal_plan* p, int64_t n, int64_t rows) {
+    const int64_t L = p->g.L, b = bytes_of(p, n);
+    if (b < kShortMinBytes) return true;
+    if (p->g.format == PCAL_F32) return n <= 4 * L && L <= 1 << 19;
+    if (rows < (b <= 4 << 20 ? 3 : 1)) return true;
+    return p->g.format == PCAL_2BIT ? n <= 48 * L && b <= 40 << 10 : n <= 128 * L && b <= 240 << 10;
+}
+
 // Fold one run of samples (n small enough for the packed 2-bit fields).
 int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
     const int64_t L = p->g.L;
@@ -85,7 +108,8 @@ int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
     int64_t head = samples_of(p, (int64_t)((16 - addr % 16) % 16));
     if (head > n) head = n;
     const int64_t row = p->g.row_samples;
-    int64_t rows = (n - head) / row;
+    const int64_t whole = (n - head) / row;
+    int64_t rows = whole;
     if (bytes_of(p, rows * row) < kBulkMinBytes) rows = 0;
     BulkTiling probe;
     if (rows > 0 && bulk_tiling(p, rows, &probe) != 0) rows = 0;  // no tile plan: a short fold
@@ -111,8 +135,7 @@ int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
     if (wide) rows = 0;
     cudaError_t e = cudaSuccess;
     if (rows == 0) {
-        // a few KB: one sample a thread does
-        e = bytes_of(p, n) < kShortMinBytes ? launch_ragged(p, d, n, k0, s) : launch_short(p, d, n, k0, s);
+        e = few_samples(p, n, whole) ? launch_ragged(p, d, n, k0, s) : launch_short(p, d, n, k0, s);
         if (e == cudaSuccess && wide) p->stats.bulk_launches += 1;
     } else {
         const uint8_t* body = d + bytes_of(p, head);

@@ -30,10 +30,30 @@ def counts(**kw):
 
 # fmt, fs, f_offset, samples, byte offset, folds
 ROUTES = [
-    ("i8", 64 * MHZ, 10_000, 8_191, 0, counts(ragged=1)),                # under 8 KB
-    ("i8", 64 * MHZ, 10_000, 8_192, 0, counts(short_folds=1)),
+    ("i8", 16, 1, 8_191, 0, counts(ragged=1)),                           # under 8 KB (L 16)
+    ("i8", 16, 1, 8_192, 0, counts(short_folds=1)),
     ("2bit", 64 * MHZ, 10_000, 640_000, 3, counts(short_folds=1)),       # 10 ms
     ("f32", 16 * MHZ, 10_000, 160_000, 4, counts(short_folds=1)),
+    ("i8", 64 * MHZ, 10_000, 245_760, 1, counts(ragged=1)),              # short calls and few samples a bin
+    ("i8", 64 * MHZ, 10_000, 245_761, 1, counts(short_folds=1)),
+    ("i8", 16 * MHZ, 10_000, 128 * 1_600, 0, counts(ragged=1)),
+    ("i8", 16 * MHZ, 10_000, 128 * 1_600 + 1, 0, counts(short_folds=1)),
+    ("2bit", 64 * MHZ, 10_000, 4 * 40_960, 0, counts(ragged=1)),
+    ("2bit", 64 * MHZ, 10_000, 4 * 40_961, 0, counts(short_folds=1)),
+    ("2bit", 16 * MHZ, 10_000, 48 * 1_600, 5, counts(ragged=1)),
+    ("2bit", 16 * MHZ, 10_000, 48 * 1_600 + 4, 5, counts(short_folds=1)),
+    ("f32", 64 * MHZ, 10_000, 4 * 6_400, 4, counts(ragged=1)),           # up to four periods
+    ("f32", 64 * MHZ, 10_000, 4 * 6_400 + 1, 4, counts(short_folds=1)),
+    ("f32", 256 * MHZ, 7_000, 4 * 256_000, 0, counts(ragged=1)),
+    ("f32", 256 * MHZ, 7_000, 4 * 256_000 + 1, 0, counts(short_folds=1)),
+    ("f32", 1024 * MHZ, 1_000, 40_000, 0, counts(short_folds=1)),        # (not of the longest)
+    ("i8", 1024 * MHZ, 1_000, 3 * 1_024_000 - 1, 0, counts(ragged=1)),   # fewer than three whole rows
+    ("i8", 1024 * MHZ, 1_000, 3 * 1_024_000, 0, counts(short_folds=1)),
+    ("2bit", 1024 * MHZ, 1_000, 4 * 767_999, 0, counts(ragged=1)),
+    ("2bit", 1024 * MHZ, 1_000, 4 * 768_000, 0, counts(short_folds=1)),
+    ("2bit", 25 * MHZ, 64, 4 * 1_000_000, 2, counts(ragged=1)),          # (rows of 6.25 MB)
+    ("i8", 25 * MHZ, 64, 6_249_999, 0, counts(ragged=1)),                # none, however long
+    ("i8", 25 * MHZ, 64, 6_250_000, 0, counts(short_folds=1)),
     ("2bit", 64 * MHZ, 10_000, 4 * 1_100_000, 1, counts(bulk=1)),        # 1 MB of rows, edges inside
     ("i8", 64 * MHZ, 10_000, 1_100_000, 0, counts(bulk=1)),
     ("f32", 64 * MHZ, 10_000, 245 * 6_400, 0, counts(short_folds=1)),
@@ -49,7 +69,7 @@ ROUTES = [
 ]
 
 
-@pytest.mark.parametrize("route", ROUTES, ids=[f"{r[0]}-L{r[1] // np.gcd.reduce([r[1], MHZ, r[2]])}-{r[3]}" for r in ROUTES])
+@pytest.mark.parametrize("route", ROUTES, ids=[f"{r[0]}-fs{r[1]}-{r[2]}-{r[3]}" for r in ROUTES])
 def test_fold_of_a_call(pcal, route):
     import torch
 
@@ -60,7 +80,7 @@ def test_fold_of_a_call(pcal, route):
         buf = torch.randn(n + 8, generator=gen, device="cuda").view(torch.uint8)
     else:
         buf = torch.randint(0, 256, (nbytes + 32,), dtype=torch.uint8, generator=gen, device="cuda")
-    with pcal.Plan(fs, MHZ, fo, fmt) as p:
+    with pcal.Plan(fs, MHZ if fs > 16 else 4, fo, fmt) as p:
         p.accumulate(buf.data_ptr() + offset, n)
         assert p.fold_counts() == expect
         bins = p.bins()
