@@ -91,11 +91,12 @@ int64_t samples_of(const pcal_plan* p, int64_t b) {
 //                400 KB 12.3 / 11.6, L 256 24 KB (94) 17.9 / 18.3, 64 KB (250) 18.8 / 18.3.
 //   float32      up to four periods: steps L 256,000 4 MB 35.5 / 41.7, L 200,000 0.8 MB 28.3 /
 //                31.7, L 64,000 1 MB 20.4 / 20.9, six periods 40 / 40; not for the longest,
-//                whose every bin gets a thread (L 1,000,000 80 KB 82 / 67).
+//                whose every bin gets a thread (L 1,000,000 80 KB 82 / 67).  L 16 8 KB (125
+//                periods) 30 / 11.
 bool few_samples(const pcal_plan* p, int64_t n, int64_t rows) {
     const int64_t L = p->g.L, b = bytes_of(p, n);
-    if (b < kShortMinBytes) return true;
     if (p->g.format == PCAL_F32) return n <= 4 * L && L <= 1 << 19;
+    if (b < kShortMinBytes) return true;
     if (rows < (b <= 4 << 20 ? 3 : 1)) return true;
     return p->g.format == PCAL_2BIT ? n <= 48 * L && b <= 40 << 10 : n <= 128 * L && b <= 240 << 10;
 }

@@ -47,6 +47,8 @@ ROUTES = [
     ("f32", 256 * MHZ, 7_000, 4 * 256_000, 0, counts(ragged=1)),
     ("f32", 256 * MHZ, 7_000, 4 * 256_000 + 1, 0, counts(short_folds=1)),
     ("f32", 1024 * MHZ, 1_000, 40_000, 0, counts(short_folds=1)),        # (not of the longest)
+    ("f32", 16, 1, 64, 0, counts(ragged=1)),
+    ("f32", 16, 1, 65, 0, counts(short_folds=1)),
     ("i8", 1024 * MHZ, 1_000, 3 * 1_024_000 - 1, 0, counts(ragged=1)),   # fewer than three whole rows
     ("i8", 1024 * MHZ, 1_000, 3 * 1_024_000, 0, counts(short_folds=1)),
     ("2bit", 1024 * MHZ, 1_000, 4 * 767_999, 0, counts(ragged=1)),
