@@ -1708,14 +1708,21 @@ cudaError_t launch_rotators(bool fixed, void* tw, int64_t L, float2* twN, int64_
 }
 
 // Plans that the short-period clusters do not take, up to kClusterBigN tones:
-// one cluster too, integer bins with the integer decode, float32 bins (an FP64
-// rotation, two operations per SM and clock) as long as 16 SMs decode them in
-// about 10 us.  The others spread over the SMs.
+// one cluster too, integer bins with the integer decode; float32 bins (an FP64
+// rotation, two operations per SM and clock) of more than 256 tones, which
+// would need a second kernel for their DFT, at shorter periods, and, where no
+// partials wait to be added (f32_cluster), up to kLargeF32L.  The others spread
+// over the SMs.  float32 finalizes with a short call, spread / cluster: 256 tones and
+// fewer L 50,000 17.6 / 19.4 us, L 64,000 17.7 / 20.4, L 100,000 19.5 / 24.9, L 128,000 (128 tones)
+// 20.4 / 27.5; N 512 L 51,200 30 / 26, L 102,400 32 / 29; N 1024 L 102,400 50 / 39; N 700 L 140,000
+// 39 / 41.  Behind bulk folds (one a finalize, 256 MB): N 300 L 30,000 52 / 44, N 700 L 35,000 64 / 66,
+// N 1000 L 100,000 76 / 81.
 constexpr int64_t kLargeF32L = 131072;
 static bool large_plan(const pcal_geometry& g) {
     return g.N <= kClusterBigN && (g.N > kClusterMaxN || g.L > kClusterMaxL) &&
-           (g.format != PCAL_F32 || g.L <= kLargeF32L);
+           (g.format != PCAL_F32 || (g.N > kClusterMaxN && g.L <= kLargeF32L));
 }
+static bool f32_cluster(const pcal_plan* p) { return p->g.L <= kClusterMaxL || p->n_pending == 0; }
 
 namespace {
 
@@ -1954,7 +1961,6 @@ cudaError_t launch_batch_finalize(BatchChan* d_ch, int n_ch, int max_n, const in
 
 namespace {
 
-constexpr int64_t kFlushFirstL = 6144;
 
 void set_common(FinArgs& a, const pcal_geometry& g, int64_t n_tot) {
     a.fs_hz = (double)g.fs;
@@ -1972,14 +1978,20 @@ void set_common(FinArgs& a, const pcal_geometry& g, int64_t n_tot) {
 }  // namespace
 
 cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
-    // float32 bins of a long period: the pending partials by all SMs first (16
-    // CTAs that add them bin by bin took 25 us for L 25600)
-    if (p->g.format == PCAL_F32 && p->g.L >= kFlushFirstL && p->n_pending > 0) {
+    const pcal_geometry& g = p->g;
+    const bool f32 = g.format == PCAL_F32;
+    const bool small = g.N <= kClusterMaxN && g.L <= kClusterMaxL;
+    const bool large = large_plan(g) && (f32 ? f32_cluster(p) : p->fixed_tw);
+    // float32 bins of a long period, several folds' partials: added by all SMs
+    // first (a cluster's 16 CTAs add them bin by bin).  Three folds of 16 MB and a
+    // finalize, with / without: L 6,400 28.6 / 28.6 us, L 10,000 29 / 33, L 25,600 38 / 45, L 32,000
+    // 28 / 39.  One fold's stay for the decode, which then starts beside the next
+    // fold: 64 MB L 6,400 16.9 / 15.7, L 16,000 19.2 / 17.7, 256 MB L 25,600 42.9 / 40.3.
+    if (f32 && (small || large) && g.L >= kLongPeriodL && p->n_pending > 1) {
         const cudaError_t e = flush_partials(p, s);
         if (e != cudaSuccess) return e;
     }
     FinArgs a{};
-    const pcal_geometry& g = p->g;
     const int64_t n_tot = p->n_abs - p->period_start;
     set_common(a, g, n_tot);
     a.fmt = g.format;
@@ -2023,8 +2035,6 @@ cudaError_t launch_finalize(pcal_plan* p, cudaStream_t s) {
     a.ticket = p->d_ticket;
     cudaError_t e = cudaErrorUnknown;
     bool done = false;
-    const bool small = g.N <= kClusterMaxN && g.L <= kClusterMaxL;
-    const bool large = large_plan(g) && (g.format == PCAL_F32 || p->fixed_tw);
     if (small || large) {
         const int C = cluster_size_for_device();
         if (C > 0) {

@@ -546,7 +546,6 @@ __global__ void __launch_bounds__(kMaxBlock, 1) bulk_fold_kernel(const __grid_co
 // only once every block of this one has started, so the grid is at most one
 // block per SM and its warps stride over the bins.
 constexpr int kReduceWarps = 16;  // warps per block
-constexpr int64_t kReduceBinsL = 6144;  // periods from which on the bins are a thread each
 
 struct PendingArgs {
     const float2* base[kPartSlots];
@@ -595,7 +594,9 @@ __global__ void __launch_bounds__(32 * kReduceWarps) reduce_f32_kernel(const __g
 // The same sums with one thread per bin, for long periods: their rows fill the
 // SMs with column groups, so a bin has few partials, a warp per bin leaves its
 // lanes idle (L 25600, four slots: 47 us), and consecutive bins' partials are
-// consecutive.  In slot, row group and column order.
+// consecutive.  In slot, row group and column order.  Back-to-back folds of 2M
+// samples, a reduction every fourth, a warp / a thread a bin: L 1,600 7.1 / 8.9 us a
+// fold, L 3,200 7.7 / 7.1, L 4,800 8.3 / 6.5, L 6,400 9.0 / 6.0, L 25,600 20.8 / 8.0.
 __global__ void __launch_bounds__(256) reduce_f32_bins_kernel(const __grid_constant__ PendingArgs pa, int cols_total,
                                                               int L, float2* __restrict__ acc) {
     allow_dependents();
@@ -848,7 +849,7 @@ cudaError_t flush_partials(pcal_plan* p, cudaStream_t s) {
     pa.n = p->n_pending;
     const int spw = p->g.samples_per_byte_x4;
     const int cols_total = (int)(p->g.row_samples / spw);
-    const bool bins = p->g.L >= kReduceBinsL;
+    const bool bins = p->g.L >= kLongPeriodL;
     const int64_t per_block = bins ? 256 : kReduceWarps;
     const int64_t blocks = (p->g.L + per_block - 1) / per_block;
     cudaLaunchConfig_t cfg = {};

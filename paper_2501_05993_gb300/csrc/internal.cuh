@@ -78,6 +78,9 @@ __host__ __device__ inline unsigned long long hint_tag(unsigned long long epoch)
 // bins, so consecutive folds (and a fold and its finalize) follow each other
 // with no kernel in between.
 constexpr int kPartSlots = 4;
+// float32 periods from which on a reduction gives every bin a thread, and several
+// folds' partials are reduced before a cluster finalize.
+constexpr int64_t kLongPeriodL = 6144;
 struct PartSlot {
     const float2* base;  // [row_groups][cols_total]
     int64_t row_groups;

@@ -176,6 +176,51 @@ def test_bulk_float32_of_long_periods(pcal, geom):
         assert np.max(np.abs(T - want)) <= 1e-5 * np.max(np.abs(want))  # the library's bound for phasors
 
 
+# fs, f_offset, bulk folds before the finalize (0: one short fold), kernels of the finalize
+FINALIZES = [
+    (128 * MHZ, 10_000, 1, 1),   # L 12800: one fold's partials are added by the finalize,
+    (128 * MHZ, 10_000, 2, 2),   # more by a reduction before it
+    (48 * MHZ, 10_000, 3, 1),    # (not for short periods)
+    (64 * MHZ, 1_000, 2, 1),     # L 64000: the finalize of all SMs adds them
+    (300 * MHZ, 10_000, 1, 1),   # L 30000, 300 tones: one cluster
+    (300 * MHZ, 10_000, 3, 2),
+    (512 * MHZ, 10_000, 0, 1),   # L 51200, 512 tones: one cluster where no partials wait,
+    (512 * MHZ, 10_000, 1, 2),   # else two kernels on all SMs
+    (512 * MHZ, 5_000, 0, 1),    # L 102400
+    (512 * MHZ, 1_000, 0, 2),    # L 512000
+]
+
+
+@pytest.mark.parametrize("case", FINALIZES, ids=[f"L{c[0] // np.gcd(MHZ, c[1])}-{c[2]}" for c in FINALIZES])
+def test_float32_finalizes(pcal, case):
+    """The finalize that a float32 period takes, and its phasors (the library's bound, 1e-5 of the largest), twice."""
+    import torch
+
+    fs, fo, folds, kernels = case
+    with pcal.Plan(fs, MHZ, fo, "f32") as p:
+        L = p.L
+        n = 257 * L + 3 * L // 7 if folds else 5 * L // 2
+        gen = torch.Generator(device="cuda").manual_seed(L)
+        x = torch.randn(n, generator=gen, device="cuda")
+        once = torch.zeros(L, dtype=torch.float64, device="cuda")
+        once += x[:n // L * L].view(-1, L).sum(0, dtype=torch.float64)
+        once[:n % L] += x[n // L * L:]
+        once = once.cpu().numpy()
+        at = 0
+        for _ in range(2):
+            S = np.zeros(L)
+            for _ in range(max(folds, 1)):
+                p.accumulate(x)
+                S += np.roll(once, at % L)
+                at += n
+            assert (p.fold_counts()["bulk"] > 0) == (folds > 0)
+            before = p.stats()["kernel_launches"]
+            T = p.finalize()
+            assert p.stats()["kernel_launches"] - before == kernels
+            ref = oracle.tones_from_bins(S, fs, MHZ, fo)
+            assert np.max(np.abs(T - ref)) <= 1e-5 * np.max(np.abs(ref))
+
+
 def test_fold_of_a_batch(pcal):
     import torch
 
