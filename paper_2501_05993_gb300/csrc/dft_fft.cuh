@@ -8,8 +8,9 @@
 // pass reads P and the last one writes T (both runs of consecutive values);
 // the passes between go through two buffers in shared memory, one value of
 // padding after 16 so that strides of 2, 4, 8 and 16 spread over the banks.
-// The twiddles of a pass lie in the order its threads read them (N - 1 in
-// all, from FP64, through L1).
+// The twiddles of a pass lie in the order its threads read them (N less the
+// first radix in all, from FP64): through L1, or (CHAIN) from shared memory,
+// where they arrive with the first pass's values.
 //
 // Two precisions.  The CUDA-core mode works in FP32.  The tensor-core modes are
 // to be no less accurate than the contraction.  Its rms error grows with N (split
@@ -46,10 +47,19 @@ struct FftPlan {
     int radix[kFftMaxPasses];  // their product is N
     bool wide;                 // double-float inside a pass
     void* tw;                  // twiddles of the passes after the first, [q - 1][k] each
+    uint32_t by_nb[kFftMaxPasses], by_m[kFftMaxPasses];  // division by N / radix and by m (over)
 };
 
 constexpr int kThreads = 128;
 constexpr int kTileValues = 2048;  // values a CTA holds, where N allows (35 KB in two buffers)
+// FP32 transforms whose calls of few channels are one chain of latencies: their
+// kernel stages the twiddles and divides by multiplication, as a load of
+// twiddles behind each pass's barrier and two divisions a butterfly were links of
+// it.  300 channels, a call in a graph, without / with: N 32 2.55 / 2.38 us, N 50 3.00 /
+// 2.74, N 96 3.17 / 2.83, N 128 3.70 / 2.75 (the direct sum 1.8, 2.3, 3.0, 4.3; 4096 channels
+// 4.9, 10, 21, 41 and the FFT 2.8, 4.8, 5.3, 4.1).  With more tones the butterflies
+// outweigh both (and N 512 got slower: 4096 channels 11.2 / 12.9).
+constexpr int kChainMinN = 32, kChainMaxN = 128;
 
 __host__ __device__ constexpr int pad(int i) { return i + (i >> 4); }
 
@@ -235,24 +245,35 @@ __device__ __forceinline__ void dft_small(V (&v)[R]) {
     }
 }
 
+// x / d as the high word of x * over(d), for d > 1 and x d < 2^32.
+inline uint32_t over(int d) { return d > 1 ? (uint32_t)((1ull << 32) / (uint64_t)d + 1) : 0; }
+
 struct FftArgs {
     FftPlan p;
     const float2* P;
     float2* T;
     int64_t C;
     int G;  // channels per CTA
+    uint32_t tw_at;  // staged twiddles: bytes into shared memory
 };
 
 // One pass over the CTA's channels: radix R, m = product of the radices
 // before; from and to are a shared buffer, or null for P and T.
-template <int R, class V>
-__device__ __forceinline__ void fft_pass(const FftArgs& a, int m, const typename V::Twiddle* tw, const float2* from,
+template <int R, class V, bool CHAIN>
+__device__ __forceinline__ void fft_pass(const FftArgs& a, int s, int m, const typename V::Twiddle* tw, const float2* from,
                                          float2* to, int64_t c0, int channels) {
     const int N = a.p.N, nb = N / R, pitch = pad(N) + 1;
     const int total = channels * nb;
     for (int b = threadIdx.x; b < total; b += kThreads) {
-        const int c = b / nb, j = b - c * nb;
-        const int hi = j / m, k = j - hi * m;
+        int c, hi;
+        if constexpr (CHAIN) {
+            c = (int)__umulhi((uint32_t)b, a.p.by_nb[s]);
+            hi = m > 1 ? (int)__umulhi((uint32_t)(b - c * nb), a.p.by_m[s]) : b - c * nb;
+        } else {
+            c = b / nb;
+            hi = (b - c * nb) / m;
+        }
+        const int j = b - c * nb, k = j - hi * m;
         V v[R];
         if (from) {
             const float2* x = from + c * pitch;
@@ -265,7 +286,10 @@ __device__ __forceinline__ void fft_pass(const FftArgs& a, int m, const typename
         }
         if (m > 1) {
 #pragma unroll
-            for (int q = 1; q < R; ++q) v[q] = turn(v[q], __ldg(tw + (q - 1) * m + k));
+            for (int q = 1; q < R; ++q) {
+                const typename V::Twiddle* w = tw + (q - 1) * m + k;
+                v[q] = turn(v[q], CHAIN ? *w : __ldg(w));
+            }
         }
         dft_small<R>(v);
         const int o = hi * m * R + k;
@@ -281,27 +305,33 @@ __device__ __forceinline__ void fft_pass(const FftArgs& a, int m, const typename
     }
 }
 
-template <class V>
+template <class V, bool CHAIN>
 __global__ void __launch_bounds__(kThreads) fft_kernel(const __grid_constant__ FftArgs a) {
-    extern __shared__ float2 fft_smem[];
+    extern __shared__ __align__(16) float2 fft_smem[];
     const int64_t c0 = (int64_t)blockIdx.x * a.G;
     const int channels = a.C - c0 < a.G ? (int)(a.C - c0) : a.G;
     float2* buf0 = fft_smem;
     float2* buf1 = fft_smem + (size_t)a.G * (pad(a.p.N) + 1);
     int m = 1;
     const typename V::Twiddle* tw = static_cast<const typename V::Twiddle*>(a.p.tw);
+    if constexpr (CHAIN) {
+        // (behind the buffers; in place at the first pass's barrier)
+        auto* staged = reinterpret_cast<typename V::Twiddle*>(reinterpret_cast<uint8_t*>(fft_smem) + a.tw_at);
+        for (int i = threadIdx.x; i < a.p.N - a.p.radix[0]; i += kThreads) staged[i] = __ldg(tw + i);
+        tw = staged;
+    }
     for (int s = 0; s < a.p.passes; ++s) {
         const int r = a.p.radix[s];
         const float2* from = s == 0 ? nullptr : s & 1 ? buf0 : buf1;
         float2* to = s == a.p.passes - 1 ? nullptr : s & 1 ? buf1 : buf0;
         switch (r) {
-            case 2: fft_pass<2, V>(a, m, tw, from, to, c0, channels); break;
-            case 3: fft_pass<3, V>(a, m, tw, from, to, c0, channels); break;
-            case 4: fft_pass<4, V>(a, m, tw, from, to, c0, channels); break;
-            case 5: fft_pass<5, V>(a, m, tw, from, to, c0, channels); break;
-            case 7: fft_pass<7, V>(a, m, tw, from, to, c0, channels); break;
-            case 8: fft_pass<8, V>(a, m, tw, from, to, c0, channels); break;
-            default: fft_pass<16, V>(a, m, tw, from, to, c0, channels); break;
+            case 2: fft_pass<2, V, CHAIN>(a, s, m, tw, from, to, c0, channels); break;
+            case 3: fft_pass<3, V, CHAIN>(a, s, m, tw, from, to, c0, channels); break;
+            case 4: fft_pass<4, V, CHAIN>(a, s, m, tw, from, to, c0, channels); break;
+            case 5: fft_pass<5, V, CHAIN>(a, s, m, tw, from, to, c0, channels); break;
+            case 7: fft_pass<7, V, CHAIN>(a, s, m, tw, from, to, c0, channels); break;
+            case 8: fft_pass<8, V, CHAIN>(a, s, m, tw, from, to, c0, channels); break;
+            default: fft_pass<16, V, CHAIN>(a, s, m, tw, from, to, c0, channels); break;
         }
         if (m > 1) tw += (r - 1) * m;
         m *= r;
@@ -361,6 +391,10 @@ inline bool fft_factors(int N, FftPlan* p) {
 inline cudaError_t fft_create(int N, bool wide, FftPlan* p) {
     if (!fft_factors(N, p)) return cudaErrorInvalidValue;
     p->wide = wide;
+    for (int s = 0, product = 1; s < p->passes; product *= p->radix[s++]) {
+        p->by_nb[s] = over(N / p->radix[s]);
+        p->by_m[s] = over(product);
+    }
     std::vector<float> tw;
     auto put = [&](double x) {
         tw.push_back((float)x);
@@ -397,10 +431,14 @@ inline cudaError_t launch_fft(const FftPlan& p, const float2* P, int64_t C, floa
     a.C = C;
     a.G = tile_channels(p, C);
     const unsigned grid = (unsigned)((C + a.G - 1) / a.G);
-    if (p.wide)
-        fft_kernel<Double><<<grid, kThreads, tile_bytes(p, a.G), s>>>(a);
-    else
-        fft_kernel<Single><<<grid, kThreads, tile_bytes(p, a.G), s>>>(a);
+    const bool chain = !p.wide && p.N >= kChainMinN && p.N <= kChainMaxN;  // (more than one pass)
+    size_t smem = tile_bytes(p, a.G);
+    if (chain) {
+        a.tw_at = (uint32_t)((smem + 15) / 16 * 16);
+        smem = a.tw_at + (size_t)(p.N - p.radix[0]) * sizeof(float2);
+    }
+    auto* k = p.wide ? fft_kernel<Double, false> : chain ? fft_kernel<Single, true> : fft_kernel<Single, false>;
+    k<<<grid, kThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
