@@ -160,8 +160,7 @@ int accumulate_run(pcal_plan* p, const uint8_t* d, int64_t n, cudaStream_t s) {
         if (e == cudaSuccess && f32 && head + tail > 0)
             e = launch_ragged_f32(p, d, head, k0, behind, tail, (k0 + done) % L, s);
         else if (e == cudaSuccess && tail > 0 && !inside)
-            e = bytes_of(p, tail) < kShortMinBytes ? launch_ragged(p, behind, tail, (k0 + done) % L, s)
-                                                   : launch_short(p, behind, tail, (k0 + done) % L, s);
+            e = launch_ragged(p, behind, tail, (k0 + done) % L, s);  // (no whole row: few_samples)
     }
     if (e != cudaSuccess) return cuda_status(e);
     p->n_abs += n;

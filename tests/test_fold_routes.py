@@ -98,14 +98,14 @@ def test_fold_of_a_call(pcal, route):
             assert np.all(np.abs(bins - oracle.sums_f32(x, 0, p.L)) <= 2.0**-31 * mag)
 
 
-# fmt, fs, f_offset (L 390625, 140625 and 703125: rows of 6.25, 2.25 and 11.25 MB), samples, fold
+# fmt, fs, f_offset (L 390625, 140625 and 703125: rows of 6.25, 2.25 and 11.25 MB), samples, fold, its ragged edges
 LARGE = [
-    ("i8", 25 * MHZ, 64, 300_000_007, "short_folds"),      # 256 MB and more of few wide rows
-    ("i8", 1125 * MHZ, 8_000, 270_000_000, "short_folds"),
-    ("i8", 25 * MHZ, 64, 130 * 6_250_000, "bulk"),
-    ("i8", 45 * MHZ, 64, 130 * 11_250_000, "bulk"),        # 10,987 column groups
-    ("f32", 45 * MHZ, 64, 257 * 703_125, "bulk"),
-    ("f32", 45 * MHZ, 64, 256 * 703_125, "short_folds"),
+    ("i8", 25 * MHZ, 64, 300_000_007, "short_folds", 0),   # 256 MB and more of few wide rows
+    ("i8", 1125 * MHZ, 8_000, 270_000_000, "short_folds", 0),
+    ("i8", 25 * MHZ, 64, 130 * 6_250_000, "bulk", 2),      # (13 bytes before, most of a row behind)
+    ("i8", 45 * MHZ, 64, 130 * 11_250_000, "bulk", 2),     # 10,987 column groups
+    ("f32", 45 * MHZ, 64, 257 * 703_125, "bulk", 1),
+    ("f32", 45 * MHZ, 64, 256 * 703_125, "short_folds", 0),
 ]
 
 
@@ -113,7 +113,7 @@ LARGE = [
 def test_large_calls_of_wide_rows(pcal, case):
     import torch
 
-    fmt, fs, fo, n, fold = case
+    fmt, fs, fo, n, fold, ragged = case
     gen = torch.Generator(device="cuda").manual_seed(n)
     if fmt == "i8":
         x = torch.randint(-128, 128, (n + 3,), dtype=torch.int8, generator=gen, device="cuda")[3:]
@@ -122,8 +122,8 @@ def test_large_calls_of_wide_rows(pcal, case):
     with pcal.Plan(fs, MHZ, fo, fmt) as p:
         p.accumulate(x.data_ptr(), n)
         f = p.fold_counts()
-        assert f[fold] == 1 and f["bulk"] + f["short_folds"] - f[fold] <= (fold == "bulk"), f  # (its tail: a short fold)
-        assert f["ragged"] <= 2
+        assert f[fold] == 1 and f["bulk"] + f["short_folds"] == 1, f
+        assert f["ragged"] == ragged, f
         bins, L = torch.from_numpy(p.bins()).cuda(), p.L
 
     def fold_of(v, dtype):
