@@ -847,17 +847,14 @@ def run_c1(args, emit=True, n_buffers=8):
 DFT_WORKLOAD = "batched tone DFT, 4096 channels x N 1024 (complex64 P -> T), seeded complex Gaussian P plus a pulse"
 
 
-def run_tensor_dft(args, emit=True, C=4096, N=1024, reps=20):
+def dft_modes(C, N, reps):
     """pcal_dft_execute in every mode on one batch of P: time per launch (CUDA events over back-to-back
     launches), bandwidth of its one read and one write against the measured copy bandwidth, and the
     error against the DFT definition in FP64."""
     import torch
 
     import paper_2501_05993_gb300 as pcal
-    from paper_2501_05993_gb300 import build as libbuild
 
-    libbuild.build()
-    pcal.load()
     rng = np.random.default_rng(2501059932 + 5)
     P = (rng.standard_normal((C, N)) + 1j * rng.standard_normal((C, N))).astype(np.complex64)
     P += (3 * np.sqrt(N) * np.exp(2j * np.pi * rng.integers(0, N, (C, 1)) * np.arange(N) / N)).astype(np.complex64)
@@ -881,17 +878,29 @@ def run_tensor_dft(args, emit=True, C=4096, N=1024, reps=20):
             flags = d.check()
         T = dT.cpu().numpy()
         err = np.max(np.abs(T - ref), axis=1) / np.max(np.abs(ref), axis=1)
-        # N here has small prime factors only: every mode is the FFT, one read of P and one write of T
-        moved = 2.0 * 8 * C * N
+        moved = 2.0 * 8 * C * N  # one read of P and one write of T
         gbs = moved / (ms / 1e3) / 1e9
         roof = {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "traffic": None,
                 "algorithmic_bytes_per_launch": moved, "peak_kind": f"{peak_kind} (copy bandwidth)"}
         modes[mode] = {"ms": ms, "tflops": method_flops / (ms / 1e3) / 1e12, "max_rel_err": float(err.max()),
                        "median_rel_err": float(np.median(err)), "device_error_bits": flags, "roofline": roof}
+    return modes
+
+
+def run_tensor_dft(args, emit=True, C=4096, N=1024, N_other=1012, reps=20):
+    """Every mode on the two kinds of tone counts: N with small prime factors (the FFT) and N_other (4 x 11 x 23: the
+    contraction, or the direct sum)."""
+    import paper_2501_05993_gb300 as pcal
+    from paper_2501_05993_gb300 import build as libbuild
+
+    libbuild.build()
+    pcal.load()
+    modes = dft_modes(C, N, reps)
     out = {"metric": "batched tone DFT time per launch", "value": modes["tf32x3"]["ms"], "unit": "ms",
            "higher_is_better": False, "data": "synthetic", "config": {"workload": DFT_WORKLOAD, "C": C, "N": N},
            "modes": modes,
-           "speedup_vs_fp32": {m: modes["fp32"]["ms"] / modes[m]["ms"] for m in ("tf32x3", "bf16x6")}}
+           "speedup_vs_fp32": {m: modes["fp32"]["ms"] / modes[m]["ms"] for m in ("tf32x3", "bf16x6")},
+           "other_counts": {"N": N_other, "modes": dft_modes(C, N_other, reps)}}
     if emit:
         print(json.dumps(out))
     return out
