@@ -577,8 +577,7 @@ int pcal_rotfold_get_acc(pcal_rotfold* r, float* host_out);
  * double-float; then the DFT, the products and the post-processing of the
  * folded path.  fs and f_comb integral Hz, N = fs/f_comb <= PCAL_BATCH_MAX_N,
  * 0 <= f_offset < f_comb any value; f32, int8 or 2-bit samples; at most 2^52
- * samples per plan.  The throughput is arithmetic-bound (below the folded
- * path).
+ * samples per plan.  The throughput is below the folded path's.
  */
 typedef struct pcal_rotplan pcal_rotplan;
 
@@ -594,7 +593,8 @@ int pcal_rotplan_set_levels(pcal_rotplan* plan, const double levels[4]);
 /* samples: DEVICE, n samples continuing the absolute index (any alignment; float32 PCAL_EINVAL off
  * 4 bytes); asynchronous on stream. */
 int pcal_rotplan_accumulate(pcal_rotplan* plan, const void* samples, int64_t n, void* stream);
-/* Finalize on `stream` (results stay on the device) and start the next period. */
+/* Finalize on `stream` (asynchronous; the results go to pinned host memory, from which
+ * pcal_rotplan_read_results takes them) and start the next period. */
 int pcal_rotplan_finalize_device(pcal_rotplan* plan, void* stream);
 /* Results of the last finalize (synchronises; layout as pcal_read_results and pcal_read_post;
  * any pointer may be NULL).  PCAL_ETIMEOUT if a bounded device wait gave up. */
@@ -611,7 +611,8 @@ int pcal_rotplan_read_results(pcal_rotplan* plan, double* phasors, double* amp, 
  * FFT: PCAL_DFT_FP32 in FP32, the tensor-core modes in FP32 from 500 tones on
  * and with double-float values inside each pass below (and at every N inside a
  * batch's finalize).  Errors vs FP64 at N = 1024, rms over rms: 1.1e-7 and
- * 0.4e-7; the contractions below 2.0e-7 and 1.7e-7, the direct sum 8e-7.
+ * 0.4e-7; the contractions below 2.0e-7 and 1.7e-7, the direct sum 8e-7 (at every
+ * such N the FFT is the more accurate in each mode, rms and worst tone).
  * For the other N:
  *   PCAL_DFT_FP32       CUDA cores, FP32 sums
  *   PCAL_DFT_TC_TF32X3  tensor cores (tcgen05): [Re P | Im P] . W as one real

@@ -862,7 +862,7 @@ class RotFold:
 
 
 class RotPlan:
-    """Per-sample double-float rotation for prime or non-integral offsets."""
+    """Every sample rotated, for prime or non-integral offsets."""
 
     def __init__(self, fs, f_comb, f_offset, fmt: str = "i8", N=None):
         self.N = int(N if N is not None else round(fs / f_comb))

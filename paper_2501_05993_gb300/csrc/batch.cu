@@ -2,8 +2,8 @@
 // sample rate, comb offset, period L and length, folded by ONE launch
 // and finalized by one launch with a thread-block cluster per channel.
 //
-// Two folds.  The direct fold (below) takes every call of a batch whose
-// schedule was neither set nor tuned; the persistent fold the others.
+// Two folds.  The direct fold (below) takes the calls of a batch until a
+// schedule is set or tuned (pcal_batch_set_fold); the persistent fold the others.
 //
 // Work list of the persistent fold.  Every channel's call is split like a single-plan call: a
 // ragged head up to its first 16-byte boundary, whole rows of row_samples

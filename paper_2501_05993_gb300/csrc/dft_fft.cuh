@@ -16,8 +16,10 @@
 // to be no less accurate than the contraction.  Its rms error grows with N (split
 // BF16 0.55e-7 at N = 20, 1.08e-7 at 256, 1.72e-7 at 1024; split TF32 1.2 to
 // 2.0e-7), that of FP32 butterflies hardly (0.66e-7, 0.92e-7, 1.07e-7): from
-// kFftSingleN tones on FP32 is the more accurate in every measure (rms, worst
-// channel, worst tone; at 486 tones the worst channel was not).  Below it, and
+// kFftSingleN tones on FP32 is the more accurate in every measure (rms, mean,
+// worst channel, worst tone) at every count that comes here, of noise and of
+// pulses; closest at N = 500 against split BF16, 1.13e-7 and 1.22e-7 rms (at 486
+// tones the worst channel was not).  Below it, and
 // wherever a delay follows (a batch's finalize), they carry double-float values
 // through each pass and round to FP32 between passes (0.35 to 0.5e-7): with FP32
 // alone the delay of a strong comb of 1024 tones moved by 1.07e-3 of its sigma.
@@ -25,10 +27,11 @@
 // Why not the dense contraction of dft_tc.cu here: that does 8 N^2 operations a
 // channel, this one 5 N log2 N, and its sums are log2 N long instead of N.
 // C 4096, N 1024, 67 MB: FP32 direct sum 2930 us, split-TF32 contraction 176 us,
-// this kernel 23 us in FP32 (bound by latency and issue slots, index arithmetic
-// and shared-memory exchanges beside the butterflies; HBM alone would take
-// 10 us) and 50 us with double-float passes (the FP32 pipes: about 300
-// operations a value).  N 256, C 4096, double-float: 33 -> 12.5 us.
+// this kernel 25 us a call in FP32 (20 in a graph that finds its data in L2; bound
+// by latency and issue slots, index arithmetic and shared-memory exchanges beside
+// the butterflies; HBM alone would take 10 us) and 50 us with double-float passes
+// (the FP32 pipes: about 300 operations a value).  N 256, C 4096, double-float:
+// 33 -> 12.5 us.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -51,6 +54,7 @@ struct FftPlan {
 };
 
 constexpr int kThreads = 128;
+constexpr int kSms = 152;  // of a GB300
 constexpr int kTileValues = 2048;  // values a CTA holds, where N allows (35 KB in two buffers)
 // FP32 transforms whose calls of few channels are one chain of latencies: their
 // kernel stages the twiddles and divides by multiplication, as a load of
@@ -346,7 +350,7 @@ inline size_t tile_bytes(const FftPlan& p, int G) {
 // Channels per CTA: kTileValues values, but fewer where that leaves SMs idle.
 inline int tile_channels(const FftPlan& p, int64_t C) {
     int64_t G = kTileValues / p.N > 0 ? kTileValues / p.N : 1;
-    const int64_t even = (C + 151) / 152;
+    const int64_t even = (C + kSms - 1) / kSms;
     if (G > even) G = even;
     return (int)G;
 }

@@ -27,8 +27,9 @@
 // distributed shared memory, and CTA 0 runs the DFT from shared memory and the
 // products, so no result makes a round trip through global memory and the
 // launch runs beside the next fold on the SMs that it leaves free.  That takes
-// every integer plan of N <= 1024 and every float32 plan of N <= 1024 and
-// L <= 131072 (large_plan).  Otherwise the fold kernel gives each CTA whole
+// every integer plan of N <= 1024, and float32 plans of N <= 256 and L <= 32768
+// or of more tones at such periods or without pending partials (large_plan).
+// Otherwise the fold kernel gives each CTA whole
 // residues b (no two CTAs add into the same P[b]); the last CTA to finish (an
 // atomic ticket, no waiting) runs the DFT for small N and the products.  For
 // large N a second kernel spreads the DFT over CTAs and its last CTA runs the
@@ -157,8 +158,9 @@ __device__ __forceinline__ double read_bin(const FinArgs& a, int64_t k) {
 }
 
 // The rotator table of integer bins: each component as W = round(x * 2^54) in
-// two halves, W = hi * 2^27 + lo with 0 <= lo < 2^27 (an FP64 sincospi rounds
-// at 2^-54 near 1, so nothing is lost).
+// two halves, W = hi * 2^27 + lo with 0 <= lo < 2^27: within 2^-55 of the FP64
+// sincospi, which itself rounds at 2^-54 above one half and finer below (the
+// sums that it enters are rounded to about 48 bits at their end, and P to FP32).
 constexpr int kRotBits = 54, kRotHalf = 27;
 
 __device__ __forceinline__ int2 rotator_fixed(double x) {
@@ -1482,8 +1484,7 @@ __device__ __forceinline__ bool cluster_finalize(const FinArgs& a) {
         if (r != 0) return false;
         if (KIND == kFew)
             dft_few(sP, sTw, N, sT, dft_threads(N));
-        else
-{
+        else {
             const int g = dft_threads(N);
             dft_tones_smem<true>(sP, sTw, N, 1, N / 2 + 1, sT, g);
             dft_zero(sP, sTw[0], N, sT, g, kClusterThreads / 2);

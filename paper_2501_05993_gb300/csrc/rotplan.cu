@@ -23,10 +23,13 @@
 //   int8            W in fixed point, six balanced base-256 digits (2^-46):
 //                   each digit's sum is exact in int32 with __dp4a over four
 //                   stripes at a time
-// Bound: float32 and 2-bit the FP32 pipes (22 operations a sample), int8 the
-// half-rate integer dot product (3 IDP4A and half a PRMT a sample).  Measured
-// (fold kernel alone): 256M int8 samples 64 us, 4.0 TB/s; 16M float32 samples
-// 21.5 us, 3.0 TB/s.  A double-float rotator advanced by one complex
+// Bound: 2-bit the issue slots (85 % of them, 180 us for 256M samples).  int8 and
+// float32 no pipe: 3 IDP4A (half rate) and half a PRMT a sample are 44 of int8's 64 us
+// for 256M samples (4.0 TB/s; issue slots 59 %, the FMA pipe 37 %, throttled between),
+// 22 FP32 operations a sample 9 of float32's 22 us for 16M (3.0 TB/s; issue slots 66 %, the
+// FMA pipe 54 % while the SMs are busy, which is four fifths of the time); with 13 to 15
+// warps an SM the rest is latency, and the start and the merge of CTAs of 26 and
+// 6 stages.  A double-float rotator advanced by one complex
 // multiplication per sample (about 120 dependent FP32 operations) took 1152
 // and 90 us.  Also measured on int8: three CTAs per SM with 16 KB stages 68 us
 // (the fixed cost per CTA outweighs the warps), four stages of 16 KB 74 us.
