@@ -793,8 +793,9 @@ int bulk_tiling(const pcal_plan* p, int64_t n_rows, BulkTiling* t) {
     if (maxb > cap) maxb = cap;
     int64_t stat = avg < 16 ? avg * 7 / 8 : avg * 3 / 4;  // (short folds: see the grab size below)
     // One CTA per column group: it takes every box of the group, with nothing
-    // to share out and so no counter.  Rows above 8 MB (odd L above 2^19, four
-    // periods of up to 4 MB each) have more groups than there are counters.
+    // to share out and so no counter (a step of 512 MB of int8, 128 groups: 79.0
+    // -> 75.5 us without the grabs).  Rows above 8 MB (odd L above 2^19) have more
+    // groups than there are counters.
     if (gr == 1) stat = maxb = total;
     if (gr > 1 && gc > kSchedCounters) return -1;
     z.row_groups = gr;
