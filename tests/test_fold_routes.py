@@ -66,6 +66,7 @@ ROUTES = [
     ("f32", 256 * MHZ, 7_000, 256 * 256_000, 0, counts(short_folds=1)),  # at most 256 periods of wider rows
     ("f32", 256 * MHZ, 7_000, 257 * 256_000, 0, counts(bulk=1)),
     ("2bit", 1024 * MHZ, 7_000, 4 * 18 * 256_000, 0, counts(bulk=1)),    # wide 2-bit rows all the same
+    ("2bit", 45 * MHZ, 64, 4 * 2 * 11_250_000, 0, counts(bulk=1)),       # (10,987 column groups)
     ("i8", 256 * MHZ, 7_000, 128 * 256_000, 0, counts(short_folds=1)),   # at most 128 wide rows
     ("i8", 256 * MHZ, 7_000, 129 * 256_000, 0, counts(bulk=1)),
 ]
