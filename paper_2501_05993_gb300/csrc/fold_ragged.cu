@@ -3,10 +3,11 @@
 // The ragged kernels fold any run of samples at any alignment straight into
 // the plan's bins (Eq. 2 with the period L of Eq. 4).  They handle the head
 // before the first 16-byte boundary, the tail after the last whole bulk row,
-// and inputs of a few KB; the short folds below take what else is too short
-// for the bulk kernel.  2-bit and int8 bins are exact
-// integers, so atomic order does not matter; float32 bins are summed by one
-// thread per bin in sample order, so they are deterministic.
+// and runs with next to nothing to add up before their atomics or stores
+// (api.cu: few_samples); the short folds below take what else is too short for
+// the bulk kernel.  2-bit and int8 bins are exact integers, so atomic order does
+// not matter; float32 bins are summed by one thread per bin in sample order, so
+// they are deterministic.
 //
 // Every kernel that touches the bins here is launched as a programmatic
 // dependent of the kernel before it: it lets its own successor start
